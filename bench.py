@@ -58,10 +58,8 @@ FP32_LANES_PER_SM = 128
 # capture (dram__bytes_read.sum + dram__bytes_write.sum) of a 4-frame launch of
 # the current kernels, scaled to a launch by its frame count.  None for a
 # kernel changed since that capture.
-DRAM_BYTES_PER_FRAME = {"k_fine_carve": 7.28576e6 / 4, "k_bisect": 17.22496e6 / 4,
-                        "k_coarse_carve": (4.332032e6 + 5120) / 4,
-                        "k_zbuffer<1>": None, "k_zbuffer<2>": None,
-                        "k_zbuffer<4>": (179.26144e6 + 9.915392e6) / 4}
+DRAM_BYTES_PER_FRAME = {"k_fine_carve": 7.28576e6 / 4, "k_bisect": None,
+                        "k_coarse_carve": (4.332032e6 + 5120) / 4, "k_zbuffer": None}
 
 
 def parse_args():
@@ -548,9 +546,8 @@ def run_ours(args):
                    FLOPS_PER_TEST, "camera tests (+ midpoints as test equivalents)"),
         "depth": (tsum["n_tris"] * rig.n_cams, FLOPS_PER_PAIR, "(triangle, camera) pairs"),
     }
-    zc = r.get_tuning()["zbuffer_cams"]
     kernel_of = {"coarse": "k_coarse_carve", "fine": "k_fine_carve", "bisect": "k_bisect",
-                 "depth": f"k_zbuffer<{zc}>"}
+                 "depth": "k_zbuffer"}
 
     sms = torch.cuda.get_device_properties(local).multi_processor_count
     alu = measure_alu(fvv, torch, sms)

@@ -440,15 +440,16 @@ enum { FVV_TILE_4x4x8 = 0, FVV_TILE_4x4x4 = 1, FVV_TILE_4x8x8 = 2, FVV_N_TILES =
 
 /* Ints of a tuning configuration: threads per block of each FVV_TUNE_*
  * kernel, then its resident blocks per SM, then the fine-hull tile shape
- * (FVV_TILE_*), then the cameras one z-buffer block serves (1, 2 or 4; each
- * triangle record is read once per that many cameras). */
+ * (FVV_TILE_*), then the groups of four cameras a z-buffer warp takes a batch
+ * of triangles through (1, 2 or 4; the triangles' vertex indices are read
+ * once per that many groups). */
 #define FVV_TUNE_INTS (2 * FVV_N_TUNE + 2)
 
 /* Autotuning (no counterpart in the paper).
  * Time candidate launch shapes (threads per block 64/128/256 x resident
  * blocks per SM 2/4/8/16/32/64) of each tunable kernel, for the fine hull
- * each tile shape too and for the z-buffer each number of cameras per block
- * (1, 2, 4), on the given slots, which must hold reconstructed
+ * each tile shape too and for the z-buffer each number of camera groups per
+ * warp (1, 2, 4), on the given slots, which must hold reconstructed
  * frames; keep the fastest, then reconstruct the slots once more with it so
  * that their results and counts are those of one reconstruction.  Results
  * never depend on the choice.  Synchronises `stream`.  config (may be NULL)
@@ -458,7 +459,7 @@ fvv_status fvv_autotune(fvv_rig *rig, const int *slots, int n_slots, void *strea
 /* Read or set the configuration (no counterpart in the paper):
  * FVV_TUNE_INTS ints as for fvv_autotune; threads must be 32..256 in steps
  * of 32, blocks per SM 1..64, the tile shape one of FVV_TILE_*, the z-buffer
- * cameras per block 1, 2 or 4 (else FVV_ERR_INVALID_ARG). */
+ * camera groups per warp 1, 2 or 4 (else FVV_ERR_INVALID_ARG). */
 fvv_status fvv_get_tuning(fvv_rig *rig, int *config);
 fvv_status fvv_set_tuning(fvv_rig *rig, const int *config);
 

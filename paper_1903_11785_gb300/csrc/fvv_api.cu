@@ -112,6 +112,38 @@ void segment_margins(CamSet& cs, const Grid& g) {
     }
 }
 
+// The cameras whose pixel cells (write_cells) decide: every point of the
+// volume's box (as in segment_margins) is in front of the camera, and two
+// points of one fine cell lie less than 64 pixels apart in its image, so that
+// cells kept modulo 128 differ wherever the cells do.  A mesh triangle lies
+// in one fine cell, up to rounding (its vertices are points of the cell's
+// edges); with image positions u, v of two such points, u inside the image,
+// |u - v| <= (sum |p_0j| d + (W + 1) sum |p_2j| d) / w_min for |X_j - X'_j| <= d.
+void cell_cameras(CamSet& cs, const Grid& g) {
+    cs.cells = 0;
+    const int dims[3] = {g.nx, g.ny, g.nz};
+    for (int n = 0; n < cs.n; ++n) {
+        const Cam& c = cs.c[n];
+        double wmin = 1e300, row[3];
+        for (int k = 0; k < 8; ++k) {
+            double w = (double)c.P[11];
+            for (int a = 0; a < 3; ++a) {
+                const double pad = (double)g.sc + 2.0 * (double)g.sf;
+                const double X = (k >> a & 1) ? (double)g.o[a] + (double)dims[a] * (double)g.sc + pad
+                                              : (double)g.o[a] - pad;
+                w += (double)c.P[8 + a] * X;
+            }
+            wmin = std::min(wmin, w);
+        }
+        for (int r = 0; r < 3; ++r)
+            row[r] = std::fabs((double)c.P[4 * r]) + std::fabs((double)c.P[4 * r + 1]) + std::fabs((double)c.P[4 * r + 2]);
+        const double d = 1.01 * (double)g.sf;
+        const double du = (row[0] + (c.W + 1.0) * row[2]) * d, dv = (row[1] + (c.H + 1.0) * row[2]) * d;
+        if (c.seg_du >= 0.0f && c.seg_du < 1.0f && c.seg_dv < 1.0f && wmin > 0.0 && std::max(du, dv) < 64.0 * wmin)
+            cs.cells |= 1ull << n;
+    }
+}
+
 struct Plan {
     CamSet cams;
     Grid grid;
@@ -182,6 +214,7 @@ fvv_status make_plan(const fvv_rig_desc* d, const fvv_recon_params* p, Plan& pl,
     g.sf = p->fine_m;
     if (p->bisect_steps < 0 || p->bisect_steps > 30) { err = "bisect_steps must be 0..30"; return FVV_ERR_INVALID_ARG; }
     segment_margins(cs, g);
+    cell_cameras(cs, g);
     g.steps = p->bisect_steps;
     if (p->surface_rule != FVV_SURFACE_BISECT && p->surface_rule != FVV_SURFACE_LAMBDA) {
         err = "bad surface_rule";
@@ -235,6 +268,7 @@ fvv_status make_plan(const fvv_rig_desc* d, const fvv_recon_params* p, Plan& pl,
     take(L.chunk_len, (size_t)g.max_chunks * 4);
     take(L.vrec, (size_t)mv * 8);
     take(L.verts, (size_t)mv * 12);
+    take(L.vcell, (size_t)mv * ((d->n_cams + 3) / 4) * 8);
     take(L.tris, (size_t)mt * 12);
     take(L.tsoup, (size_t)mt * 48);
     take(L.trec, (size_t)mt * 8);
@@ -598,7 +632,7 @@ fvv_status fvv_set_tuning(fvv_rig* rig, const int* config) {
     const int tile = config[2 * FVV_N_TUNE];
     if (tile < 0 || tile >= FVV_N_TILES) return fail(rig, FVV_ERR_INVALID_ARG, "tile shape must be one of FVV_TILE_*");
     const int zc = config[2 * FVV_N_TUNE + 1];
-    if (zc != 1 && zc != 2 && zc != 4) return fail(rig, FVV_ERR_INVALID_ARG, "z-buffer cameras per block must be 1, 2 or 4");
+    if (zc != 1 && zc != 2 && zc != 4) return fail(rig, FVV_ERR_INVALID_ARG, "z-buffer camera groups per warp must be 1, 2 or 4");
     for (int k = 0; k < FVV_N_TUNE; ++k) {
         rig->tune.threads[k] = config[k];
         rig->tune.waves[k] = config[FVV_N_TUNE + k];
@@ -641,7 +675,7 @@ fvv_status fvv_autotune(fvv_rig* rig, const int* slots, int n_slots, void* strea
         float best = 1e30f;
         Tuning keep = rig->tune;
         // the fine hull also tries each tile shape, the z-buffer each number
-        // of cameras per block (1, 2, 4)
+        // of camera groups per warp (1, 2, 4)
         const int n_tiles = knob == FVV_TUNE_FINE ? FVV_N_TILES : knob == FVV_TUNE_ZBUFFER ? 3 : 1;
         for (int tile = 0; tile < n_tiles && e == cudaSuccess; ++tile)
         for (int th : threads)

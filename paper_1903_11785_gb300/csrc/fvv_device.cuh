@@ -199,6 +199,84 @@ __device__ __forceinline__ void load_smem_cams(const CamSet& cams, int n, SmemCa
     }
 }
 
+// ---- pixel cells: which pixel centres a vertex lies between, per camera
+//
+// A triangle covers no pixel centre of a camera if no column of centres, or
+// no row, lies between its vertices' image positions; for meshes of one-pixel
+// triangles that turns away two pairs (triangle, camera) out of three.  The
+// cell of an image position u is floor(u - 1/2): the centres (integers plus
+// 1/2) at or left of it.  Per vertex and camera the low 7 bits of its column
+// and of its row cell are kept, one byte each, four cameras to a uint2 (x:
+// columns, y: rows), with bit 7 set where the cell is not certain: u - 1/2 is
+// within a slack of an integer, or the camera's cells do not decide
+// (CamSet::cells; it then may have points that are not in front of it).
+// Positions outside the image count as the cell before the first centre or
+// at the last one.  Three
+// equal bytes without bit 7 then mean that no column (row) of centres lies
+// between the vertices: their cells are equal modulo 128 and, where
+// CamSet::cells says so, less than 128 apart.
+constexpr float kMagic = 12582912.0f;        // 1.5 * 2^23: floats within 2^22 of it are integers
+
+// What a camera's cells take beside its matrix.
+struct __align__(16) CellCam {
+    float iW, iH;            // 1 / W, 1 / H
+    float certain;           // 1/2 - slack: a position nearer than that to its cell's middle is certain; -1: never
+    float pad_;
+};
+
+// The slack bounds, twice over, the error of an image position formed as in
+// cell_at: seven roundings of at most 2^-23 relative to a position of at most W.
+__device__ __forceinline__ void load_cell_cams(const CamSet& cams, int n, CellCam* cc) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const float W = cams.c[i].Wf, H = cams.c[i].Hf;
+        const float slack = __fmaf_rn(fadd(fmaxf(W, H), 2.0f), 0x1p-19f, 0x1p-12f);
+        cc[i].iW = __frcp_rn(W);
+        cc[i].iH = __frcp_rn(H);
+        cc[i].certain = (cams.cells >> i) & 1u ? fsub(0.5f, slack) : -1.0f;
+        cc[i].pad_ = 0.0f;
+    }
+}
+
+// The cell of u = n s, s = x iw clamped to [0, 1] (all on the FMA pipe: the
+// integer ALU is the busier one in the kernels that call this): floor(u - 1/2)
+// is u - 1 rounded to the nearest integer, in the low bits of the result,
+// unless u - 1/2 is near an integer, which the distance to it shows.
+__device__ __forceinline__ uint32_t cell_at(float x, float iw, float n, float certain, bool& sure) {
+    float s;
+    asm("mul.rn.sat.f32 %0, %1, %2;" : "=f"(s) : "f"(x), "f"(iw));
+    const float a = __fmaf_rn(s, n, kMagic - 1.0f);
+    const float e = __fmaf_rn(s, n, fsub(kMagic - 1.0f, a));   // u - 1 - cell
+    sure = fabsf(e) < certain;
+    return __float_as_uint(a);
+}
+
+// The pixel cells of vertex (X, Y, Z) in the ncam cameras of sc and cc (all
+// lanes use the same camera at a time), out[g] for cameras 4g .. 4g + 3.
+__device__ __forceinline__ void write_cells(const SmemCam* sc, const CellCam* cc, int ncam, float X, float Y, float Z,
+                                            uint2* out) {
+#pragma unroll 1
+    for (int g = 0; 4 * g < ncam; ++g) {
+        uint32_t cx[4] = {0u, 0u, 0u, 0u}, cy[4] = {0u, 0u, 0u, 0u};
+        uint32_t fx = 0, fy = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int n = 4 * g + k;
+            if (n >= ncam) break;
+            float xp, yp, wp;
+            project(sc[n].P, X, Y, Z, xp, yp, wp);
+            const float r = rcp_approx(wp);
+            bool sx, sy;
+            cx[k] = cell_at(xp, fmul(r, cc[n].iW), sc[n].Wf, cc[n].certain, sx);
+            cy[k] = cell_at(yp, fmul(r, cc[n].iH), sc[n].Hf, cc[n].certain, sy);
+            if (!sx) fx |= 0x80u << (8 * k);
+            if (!sy) fy |= 0x80u << (8 * k);
+        }
+        const uint32_t bx = __byte_perm(__byte_perm(cx[0], cx[1], 0x0040), __byte_perm(cx[2], cx[3], 0x0040), 0x5410);
+        const uint32_t by = __byte_perm(__byte_perm(cy[0], cy[1], 0x0040), __byte_perm(cy[2], cy[3], 0x0040), 0x5410);
+        out[g] = make_uint2((bx & 0x7F7F7F7Fu) | fx, (by & 0x7F7F7F7Fu) | fy);
+    }
+}
+
 // The ROI holding fine word w: the last ROI whose first word is <= w.
 __device__ __forceinline__ int roi_of_word(const DRoi* rois, int n, uint32_t w) {
     int lo = 0, hi = n - 1;

@@ -43,6 +43,7 @@ struct Cam {
 struct CamSet {
     int n;
     int oob;             // FVV_OOB_*
+    uint64_t cells;      // bit n: camera n's pixel cells (Layout::vcell) decide (see cell_cameras in fvv_api.cu)
     Cam c[FVV_MAX_CAMS];
 };
 
@@ -115,6 +116,7 @@ struct Layout {
     size_t chunk_len;           // uint32 per chunk: words of its staged slab (a multiple of 4), 0: not staged
     size_t vrec;                // uint64 vertex records, max_verts
     size_t verts;               // float x3, max_verts
+    size_t vcell;               // uint2 per vertex and four cameras: its pixel cells (write_cells), max_verts
     size_t tris;                // uint32 x3, max_tris
     size_t tsoup;               // float4 x3 per triangle: its vertices and centroid
                                 // (v0 xyz, v1 xyz, v2 xyz, centroid xyz), max_tris
@@ -157,7 +159,7 @@ struct Tuning {
     int threads[FVV_N_TUNE];
     int waves[FVV_N_TUNE];
     int fine_tile;       // index into kFineTiles
-    int zb_cams;         // cameras per z-buffer block: 1, 2 or 4
+    int zb_cams;         // groups of four cameras per z-buffer block: 1, 2 or 4
 };
 
 // The grid with the tuned fine-carve tile shape.

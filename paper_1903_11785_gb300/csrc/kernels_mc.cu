@@ -593,6 +593,14 @@ __device__ __forceinline__ void bisect_steps(const SmemCam* sc, int ncam, const 
     }
 }
 
+// Vertex i of a slot: its position and its pixel cells for the z-buffer.
+__device__ __forceinline__ void store_vertex(float* verts, uint2* vcell, uint32_t i, const float* v,
+                                             const SmemCam* sc, const CellCam* cc, int ncam) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) verts[3 * (size_t)i + d] = v[d];
+    write_cells(sc, cc, ncam, v[0], v[1], v[2], vcell + (size_t)i * (unsigned)((ncam + 3) >> 2));
+}
+
 // Vertices a warp sorts at once, per lane, and the bucket of the sort that
 // holds every list of kSortCap - 1 or more cameras (one more bucket, the
 // last, holds the window's empty places).
@@ -629,10 +637,12 @@ __global__ void __launch_bounds__(256) k_bisect(const __grid_constant__ CamSet c
     pdl_begin();
     __shared__ unsigned long long sh_t[32];
     __shared__ SmemCam sc[FVV_MAX_CAMS];
+    __shared__ CellCam cc[FVV_MAX_CAMS];
     extern __shared__ __align__(16) unsigned char bisect_smem[];   // BisectWarpSmem per warp
     BisectWarpSmem* wsm = reinterpret_cast<BisectWarpSmem*>(bisect_smem);
     const int ncam = NC > 0 ? NC : cams.n;
     load_smem_cams(cams, ncam, sc);
+    load_cell_cams(cams, ncam, cc);
     __syncthreads();
     const bool abstain = cams.oob == FVV_OOB_ABSTAIN;
     const int slot = sl.s[blockIdx.y];
@@ -642,6 +652,7 @@ __global__ void __launch_bounds__(256) k_bisect(const __grid_constant__ CamSet c
     const uint32_t* __restrict__ sil = slot_ptr<uint32_t>(L, slot, L.sil);
     const uint64_t* vrec = slot_ptr<uint64_t>(L, slot, L.vrec);
     float* verts = slot_ptr<float>(L, slot, L.verts);
+    uint2* vcell = slot_ptr<uint2>(L, slot, L.vcell);
     unsigned long long tests = 0, reads = 0;
     const uint32_t nthreads = gridDim.x * blockDim.x;
     int kv = 1;                                    // the same in every block of the slot
@@ -655,7 +666,8 @@ __global__ void __launch_bounds__(256) k_bisect(const __grid_constant__ CamSet c
             const uint64_t undecided = g.steps > 0 ? bisect_undecided(sc, ncam, sil, a, b, seen_fg, reads) : 0ull;
             bisect_steps(sc, ncam, sil, g.steps, abstain, undecided, seen_fg, a, b, tests, reads);
 #pragma unroll
-            for (int d = 0; d < 3; ++d) verts[3 * (size_t)i + d] = fmul(fadd(a[d], b[d]), 0.5f);
+            for (int d = 0; d < 3; ++d) a[d] = fmul(fadd(a[d], b[d]), 0.5f);
+            store_vertex(verts, vcell, i, a, sc, cc, ncam);
         }
     } else {
         const int lane = threadIdx.x & 31;
@@ -730,7 +742,8 @@ __global__ void __launch_bounds__(256) k_bisect(const __grid_constant__ CamSet c
                     bisect_ends(vrec[i], rois, g, a, b);
                     bisect_steps(sc, ncam, sil, g.steps, abstain, w.und[p], (id >> 31) != 0u, a, b, tests, reads);
 #pragma unroll
-                    for (int d = 0; d < 3; ++d) verts[3 * (size_t)i + d] = fmul(fadd(a[d], b[d]), 0.5f);
+                    for (int d = 0; d < 3; ++d) a[d] = fmul(fadd(a[d], b[d]), 0.5f);
+                    store_vertex(verts, vcell, i, a, sc, cc, ncam);
                 }
             }
             __syncwarp();   // the window's shared memory is read before the next one writes it
@@ -801,6 +814,12 @@ __global__ void __launch_bounds__(256) k_lambda(const __grid_constant__ CamSet c
                                                 const __grid_constant__ Layout L, const __grid_constant__ SlotList sl) {
     pdl_begin();
     __shared__ unsigned long long sh_t[32];
+    __shared__ SmemCam sc[FVV_MAX_CAMS];
+    __shared__ CellCam cc[FVV_MAX_CAMS];
+    const int ncam = NC > 0 ? NC : cams.n;
+    load_smem_cams(cams, ncam, sc);
+    load_cell_cams(cams, ncam, cc);
+    __syncthreads();
     const int slot = sl.s[blockIdx.y];
     const SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
     const uint32_t nv = info->n_words ? info->n_verts : 0u;
@@ -808,6 +827,7 @@ __global__ void __launch_bounds__(256) k_lambda(const __grid_constant__ CamSet c
     const uint32_t* __restrict__ sil = slot_ptr<uint32_t>(L, slot, L.sil);
     const uint64_t* vrec = slot_ptr<uint64_t>(L, slot, L.vrec);
     float* verts = slot_ptr<float>(L, slot, L.verts);
+    uint2* vcell = slot_ptr<uint2>(L, slot, L.vcell);
     uint32_t tests = 0;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += gridDim.x * blockDim.x) {
         const uint64_t rec = vrec[i];
@@ -836,7 +856,8 @@ __global__ void __launch_bounds__(256) k_lambda(const __grid_constant__ CamSet c
             }
         }
 #pragma unroll
-        for (int d = 0; d < 3; ++d) verts[3 * (size_t)i + d] = fadd(a[d], fmul(lam, fsub(b[d], a[d])));
+        for (int d = 0; d < 3; ++d) a[d] = fadd(a[d], fmul(lam, fsub(b[d], a[d])));
+        store_vertex(verts, vcell, i, a, sc, cc, ncam);
     }
     // every pixel visited is one silhouette word read
     const unsigned long long t = block_sum<unsigned long long>(tests, sh_t);

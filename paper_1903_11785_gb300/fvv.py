@@ -38,14 +38,14 @@ STAGES = ("pack", "coarse", "ccl", "fine", "mc", "bisect", "depth", "colour")
 TUNE_KNOBS = ("coarse", "fine", "bisect", "zbuffer", "triangles")
 N_TUNE = len(TUNE_KNOBS)
 FINE_TILES = ((4, 4, 8), (4, 4, 4), (4, 8, 8))   # FVV_TILE_*: fine-hull tile (x, y, z) samples
-ZBUFFER_CAMS = (1, 2, 4)                          # cameras one z-buffer block serves
+ZBUFFER_CAMS = (1, 2, 4)                          # groups of four cameras a z-buffer warp takes a batch through
 TUNE_INTS = 2 * N_TUNE + 2
 
 
 def tuning_dict(cfg):
     """{kernel: (threads per block, blocks per SM)}, the fine-hull tile
-    shape ("fine_tile": (x, y, z)) and the cameras per z-buffer block
-    ("zbuffer_cams") from the flat C layout."""
+    shape ("fine_tile": (x, y, z)) and the groups of four cameras per z-buffer
+    warp ("zbuffer_cams") from the flat C layout."""
     d = {k: (cfg[i], cfg[N_TUNE + i]) for i, k in enumerate(TUNE_KNOBS)}
     d["fine_tile"] = FINE_TILES[cfg[2 * N_TUNE]]
     d["zbuffer_cams"] = cfg[2 * N_TUNE + 1]
