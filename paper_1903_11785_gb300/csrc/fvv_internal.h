@@ -177,6 +177,7 @@ inline Tuning default_tuning() {
         t.waves[k] = 8;
     }
     t.waves[FVV_TUNE_ZBUFFER] = 16;
+    t.waves[FVV_TUNE_FINE] = 16;
     t.fine_tile = FVV_TILE_4x4x8;
     t.zb_cams = 4;
     return t;

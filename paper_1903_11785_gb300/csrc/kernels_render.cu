@@ -265,7 +265,7 @@ __device__ __forceinline__ uint32_t nonzero_bytes(uint32_t v) {
 // it (`resident`) two such units is cut into units of one group each.
 // Court-shaped frames (800,000 triangles, 16 cameras): 72 -> 40 us a frame in
 // a batch of 64; 4K court (180,000 triangles of 9 pixels): 82 -> 40 us.
-__global__ void __launch_bounds__(256, 4) k_zbuffer(const __grid_constant__ CamSet cams,
+__global__ void __launch_bounds__(256) k_zbuffer(const __grid_constant__ CamSet cams,
                                                     const __grid_constant__ Layout L,
                                                     const __grid_constant__ SlotList sl, int quads,
                                                     uint32_t resident) {
