@@ -59,7 +59,7 @@ FP32_LANES_PER_SM = 128
 # the current kernels, scaled to a launch by its frame count.  None for a
 # kernel changed since that capture.
 DRAM_BYTES_PER_FRAME = {"k_fine_carve": None, "k_bisect": None,
-                        "k_coarse_carve": (4.332032e6 + 5120) / 4, "k_zbuffer": None}
+                        "k_coarse_first + k_coarse_rest": None, "k_zbuffer": None}
 
 
 def parse_args():
@@ -546,7 +546,7 @@ def run_ours(args):
                    FLOPS_PER_TEST, "camera tests (+ midpoints as test equivalents)"),
         "depth": (tsum["n_tris"] * rig.n_cams, FLOPS_PER_PAIR, "(triangle, camera) pairs"),
     }
-    kernel_of = {"coarse": "k_coarse_carve", "fine": "k_fine_carve", "bisect": "k_bisect",
+    kernel_of = {"coarse": "k_coarse_first + k_coarse_rest", "fine": "k_fine_carve", "bisect": "k_bisect",
                  "depth": "k_zbuffer"}
 
     sms = torch.cuda.get_device_properties(local).multi_processor_count

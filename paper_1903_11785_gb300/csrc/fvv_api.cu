@@ -24,6 +24,7 @@ struct fvv_rig {
     bool own_arena = false;
     uint8_t* mc_ntri = nullptr;    // device
     uint8_t* mc_edges = nullptr;   // device
+    CoarseTable table{};           // device, in the arena
     size_t sil_words = 0, npix = 0;
     std::vector<int> state;        // per slot: 0 empty, 1 uploaded, 2 reconstructed
     std::string err;
@@ -144,11 +145,25 @@ void cell_cameras(CamSet& cs, const Grid& g) {
     }
 }
 
+// Cameras of the coarse table: the first eight, which settle nearly every
+// voxel, or as many as fit 1 GiB, but at least one (a court frame's grid of 7
+// million voxels takes 28 MB each; 64 frames: 1220 us with four, 1110 with 16),
+// of those whose images are not too large for a 32-bit bit index.  At the others voxels are tested by projecting them.
+int coarse_table_cams(const CamSet& cs, const Grid& g) {
+    const double per = (double)g.nx * g.ny * g.nz * 4.0;
+    const int most = std::min(cs.n, (int)std::min(8.0, std::max(1.0, (double)(1ull << 30) / per)));
+    for (int n = 0; n < most; ++n)
+        if ((unsigned long long)((cs.c[n].H + 31) / 32) * cs.c[n].Wq * 1024ull >= kNoPixel) return n;
+    return most;
+}
+
 struct Plan {
     CamSet cams;
     Grid grid;
     Layout L;        // offsets only (base unset)
     size_t common = 0;   // bytes before the slots region
+    size_t table = 0;    // offset of the coarse table
+    int table_cams = 0;
     size_t total = 0;
     size_t sil_words = 0, npix = 0;
 };
@@ -164,7 +179,7 @@ fvv_status make_plan(const fvv_rig_desc* d, const fvv_recon_params* p, Plan& pl,
     cs.n = d->n_cams;
     if (p->oob_policy != FVV_OOB_STRICT && p->oob_policy != FVV_OOB_ABSTAIN) { err = "bad oob_policy"; return FVV_ERR_INVALID_ARG; }
     cs.oob = p->oob_policy;
-    size_t words = 0, pix = 0;
+    size_t words = 0, blocked = 0, pix = 0;
     for (int n = 0; n < cs.n; ++n) {
         Cam& c = cs.c[n];
         for (int k = 0; k < 12; ++k) {
@@ -182,10 +197,12 @@ fvv_status make_plan(const fvv_rig_desc* d, const fvv_recon_params* p, Plan& pl,
         c.Wf = (float)c.W;
         c.Hf = (float)c.H;
         c.bit_off = (uint32_t)words;
+        c.blk_off = (uint32_t)blocked;
         c.pix_off = pix;
+        blocked += (size_t)((c.H + 31) / 32) * c.Wq * 32;
         words += (size_t)c.H * c.Wq;
         pix += (size_t)c.H * c.W;
-        if (words >= (1ull << 32)) { err = "silhouettes too large"; return FVV_ERR_INVALID_ARG; }
+        if (std::max(words, blocked) >= (1ull << 32)) { err = "silhouettes too large"; return FVV_ERR_INVALID_ARG; }
     }
     pl.sil_words = words;
     pl.npix = pix;
@@ -248,6 +265,7 @@ fvv_status make_plan(const fvv_rig_desc* d, const fvv_recon_params* p, Plan& pl,
     g.tile_y = kFineTiles[FVV_TILE_4x4x8][0];
     g.tile_z = kFineTiles[FVV_TILE_4x4x8][1];
 
+    pl.table_cams = coarse_table_cams(cs, g);
     Layout& L = pl.L;
     std::memset(&L, 0, sizeof(L));
     size_t o = 0;
@@ -255,7 +273,9 @@ fvv_status make_plan(const fvv_rig_desc* d, const fvv_recon_params* p, Plan& pl,
     const size_t nvox = (size_t)g.nx * g.ny * g.nz;
     take(L.info, sizeof(SlotInfo));
     take(L.sil, words * 4);
+    take(L.silb, blocked * 4);
     take(L.coarse, (size_t)g.nz * g.ny * g.nxw * 4);
+    take(L.front, (size_t)g.nz * g.ny * g.nxw * 16);
     take(L.parent, nvox * 4);
     take(L.roots, (size_t)g.max_comp * 4);
     take(L.cstat, (size_t)g.max_comp * 7 * 4);
@@ -281,6 +301,8 @@ fvv_status make_plan(const fvv_rig_desc* d, const fvv_recon_params* p, Plan& pl,
     if (d->host_staging == 1) take(L.rgb_stage, pix * 3);
     L.stride = o;
     pl.common = align_up(256) + align_up(256 * kMaxTriPerCell * 3) + align_up(FVV_MAX_BATCH * 3 * sizeof(float));
+    pl.table = pl.common;
+    pl.common += align_up(nvox * pl.table_cams * 4);
     pl.total = pl.common + (size_t)d->max_slots * L.stride;
     return FVV_OK;
 }
@@ -398,6 +420,11 @@ fvv_status fvv_create_rig(const fvv_rig_desc* desc, const fvv_recon_params* para
     build_mc_table(ntri.data(), edges.data());
     e = cudaMemcpy(rig->mc_ntri, ntri.data(), ntri.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(rig->mc_edges, edges.data(), edges.size(), cudaMemcpyHostToDevice);
+    if (pl.table_cams) {
+        uint32_t* tab = reinterpret_cast<uint32_t*>(rig->arena + pl.table);
+        rig->table = CoarseTable{tab, pl.table_cams};
+        if (e == cudaSuccess) e = launch_coarse_table(rig->cams, rig->grid, tab, pl.table_cams, nullptr);
+    }
     // every depth image starts empty; each depth stage then clears only the
     // box its slot's previous z-buffer wrote
     if (e == cudaSuccess) e = launch_init_depth(rig->cams, rig->L, rig->max_slots, rig->sms, nullptr);
@@ -540,7 +567,7 @@ static cudaError_t enqueue_reconstruct(fvv_rig* rig, const SlotList& sl, cudaStr
         e = (call);                             \
         stage_end(rig, t, st);                  \
     }
-    FVV_STAGE(FVV_STAGE_COARSE, launch_coarse_carve(rig->cams, g, rig->L, sl, rig->sms, tu, st));
+    FVV_STAGE(FVV_STAGE_COARSE, launch_coarse_carve(rig->cams, g, rig->L, sl, rig->table, rig->sms, tu, st));
     FVV_STAGE(FVV_STAGE_CCL, launch_ccl(g, rig->L, sl, rig->sms, st));
     FVV_STAGE(FVV_STAGE_FINE, launch_fine_carve(rig->cams, g, rig->L, sl, rig->sms, tu, st));
     FVV_STAGE(FVV_STAGE_MC, launch_mc_prefix(g, rig->L, sl, mc, rig->sms, st));
@@ -661,7 +688,9 @@ fvv_status fvv_autotune(fvv_rig* rig, const int* slots, int n_slots, void* strea
     auto run = [&](int knob, const Tuning& tu) -> cudaError_t {
         const Grid g = tuned_grid_params(rig->grid, tu);
         switch (knob) {
-            case FVV_TUNE_COARSE: return launch_coarse_carve(rig->cams, g, rig->L, sl, rig->sms, tu, st);
+            case FVV_TUNE_COARSE:
+                if (const cudaError_t r = launch_reset_coarse(rig->L, sl, st); r != cudaSuccess) return r;
+                return launch_coarse_carve(rig->cams, g, rig->L, sl, rig->table, rig->sms, tu, st);
             case FVV_TUNE_FINE: return launch_fine_carve(rig->cams, g, rig->L, sl, rig->sms, tu, st);
             case FVV_TUNE_BISECT: return launch_bisect(rig->cams, g, rig->L, sl, rig->sms, tu, st);
             case FVV_TUNE_ZBUFFER:

@@ -32,6 +32,7 @@ struct Cam {
     int W, H, Wq;        // Wq = 32-bit words per silhouette row
     float Wf, Hf;        // W and H as floats
     uint32_t bit_off;    // first silhouette word of this camera in a slot
+    uint32_t blk_off;    // first word of its blocked silhouette
     uint64_t pix_off;    // first pixel of this camera in per-slot pixel arrays
     // Bound (pixels) on how far the computed image position of any point the
     // bisection of a grid edge can test lies from the box of the edge ends'
@@ -81,6 +82,7 @@ struct SlotInfo {
     uint32_t next_chunk;        // the compaction's next unclaimed 256-word chunk
     uint32_t n_verts, n_tris;
     uint32_t n_on;
+    uint32_t n_front;           // coarse words that camera 0 does not empty
     unsigned long long tests_coarse, tests_fine, tests_bisect;
     unsigned long long look_fine, look_bisect;   // silhouette words read
 };
@@ -103,7 +105,12 @@ struct Layout {
     size_t stride;              // bytes per slot
     size_t info;                // SlotInfo
     size_t sil;                 // uint32 silhouette bits
+    size_t silb;                // uint32 silhouette bits again, blocked: per camera, tiles of 32 x 32 pixels (row-major,
+                                // Wq a row), in a tile 8 x 4 words of 8 x 4 pixels (row-major, bit 8 (y % 4) + x % 8),
+                                // so that a 128-byte line holds a square of pixels
     size_t coarse;              // uint32 coarse bits (nz*ny*nxw)
+    size_t front;               // uint4 per word that camera 0 leaves voxels of: the word, voxels left, their
+                                // foreground votes, first voxel
     size_t parent;              // int32 union-find parents, nx*ny*nz
     size_t roots;               // int32 root linear indices, max_comp
     size_t cstat;               // int32 per component: count, min xyz, max xyz (7 each)
@@ -133,6 +140,17 @@ template <typename T>
 __host__ __device__ inline T* slot_ptr(const Layout& L, int slot, size_t off) {
     return reinterpret_cast<T*>(L.base + (size_t)slot * L.stride + off);
 }
+
+// Where the coarse voxels fall in the first n cameras' silhouettes: the cameras
+// are static and so is the grid, so this is laid out once, when the rig is
+// created.  e[c * voxels + L]: the bit of voxel L's pixel in camera c's blocked
+// silhouette (word * 32 + bit, see Layout::silb), or kNoPixel where the voxel is
+// not in front of the camera or not inside its image.
+constexpr uint32_t kNoPixel = 0xFFFFFFFFu;
+struct CoarseTable {
+    const uint32_t* e;
+    int n;                      // see coarse_table_cams in fvv_api.cu
+};
 
 struct SlotList {
     int n;
@@ -177,6 +195,7 @@ inline Tuning default_tuning() {
         t.waves[k] = 8;
     }
     t.waves[FVV_TUNE_ZBUFFER] = 16;
+    t.waves[FVV_TUNE_COARSE] = 16;
     t.waves[FVV_TUNE_FINE] = 16;
     t.fine_tile = FVV_TILE_4x4x8;
     t.zb_cams = 4;
@@ -205,8 +224,11 @@ void build_mc_table(uint8_t ntri[256], uint8_t edges[256 * kMaxTriPerCell * 3]);
 // host_src: the sources are mapped page-locked host memory.
 cudaError_t launch_pack(const CamSet& cams, const Layout& L, int n_frames, const int* slots,
                         const uint8_t* const* src, bool host_src, int sms, cudaStream_t st);
+cudaError_t launch_coarse_table(const CamSet& cams, const Grid& g, uint32_t* e, int n, cudaStream_t st);
+// The coarse hull; the slots' n_front must be zero (k_zero_info, or launch_reset_coarse to run it again).
+cudaError_t launch_reset_coarse(const Layout& L, const SlotList& sl, cudaStream_t st);
 cudaError_t launch_coarse_carve(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl,
-                                int sms, const Tuning& tu, cudaStream_t st);
+                                const CoarseTable& tab, int sms, const Tuning& tu, cudaStream_t st);
 cudaError_t launch_ccl(const Grid& g, const Layout& L, const SlotList& sl, int sms, cudaStream_t st);
 // The filter and ROI table alone (k_filter), e.g. again for another fine-carve tile shape.
 cudaError_t launch_filter(const Grid& g, const Layout& L, const SlotList& sl, cudaStream_t st);

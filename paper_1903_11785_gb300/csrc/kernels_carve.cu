@@ -2,12 +2,9 @@
 // visual hulls (Sec. II-B-1 and II-B-3).
 //
 // Silhouettes are kept as 1 bit per pixel (a 1080p camera is 260 KB, a
-// 16-camera frame 4 MB, so a frame's silhouettes stay in L2).  A coarse
-// carve warp takes a row of the occupancy bitset one 32-voxel word at a time:
-// lane i tests voxel 32w+i, the warp walks the cameras in index order and
-// stops as soon as a ballot shows no lane is still occupied, so the warp's
-// loads stay coherent (the 32 voxels of a word project close together) and
-// empty space costs one camera.
+// 16-camera frame 4 MB, so a frame's silhouettes stay in L2), row by row for
+// the fine hull and the surface, which scan short rows of them, and once more in
+// square blocks for the coarse hull, whose gathers run across them.
 #include "fvv_device.cuh"
 
 namespace fvv {
@@ -28,81 +25,295 @@ __device__ __forceinline__ uint32_t nonzero_bytes4(uint32_t w) {
 }
 
 // Step a0: uint8 mask (nonzero = foreground) -> 1 bit per pixel, 32 pixels per
-// word, bit x%32 of word x/32 of its row.  One thread per output word; grid
-// (blocks, cameras, frames).
+// word, bit x%32 of word x/32 of its row; and the same bits blocked
+// (Layout::silb), whose words are the transposed bytes of four rows' words.
+// One thread per 32 x 4 pixels; grid (blocks, cameras, frames).  Bound by
+// HBM: eight 16-byte loads are in flight per thread.
 __global__ void __launch_bounds__(256) k_pack(const __grid_constant__ CamSet cams, const __grid_constant__ PackSrc a,
                                               const __grid_constant__ Layout L) {
     pdl_begin();
     const Cam& c = cams.c[blockIdx.y];
     const uint8_t* src = a.src[blockIdx.z * (unsigned)cams.n + blockIdx.y];
-    uint32_t* __restrict__ sil = slot_ptr<uint32_t>(L, a.slot[blockIdx.z], L.sil);
-    const size_t words = (size_t)c.H * (unsigned)c.Wq;
+    uint32_t* __restrict__ sil = slot_ptr<uint32_t>(L, a.slot[blockIdx.z], L.sil) + c.bit_off;
+    uint32_t* __restrict__ silb = slot_ptr<uint32_t>(L, a.slot[blockIdx.z], L.silb) + c.blk_off;
+    const unsigned Wq = (unsigned)c.Wq;
+    const size_t units = (size_t)((c.H + 3) >> 2) * Wq;
     const bool vec = (c.W % 32 == 0) && ((reinterpret_cast<uintptr_t>(src) & 15u) == 0);
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t row = i / (unsigned)c.Wq;
-        const int wq = (int)(i - row * (unsigned)c.Wq);
-        const uint8_t* p = src + row * (unsigned)c.W + (size_t)wq * 32;
-        uint32_t bits = 0;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < units; i += (size_t)gridDim.x * blockDim.x) {
+        const size_t r4 = i / Wq;
+        const unsigned wq = (unsigned)(i - r4 * Wq);
+        const int rows = min(4, c.H - (int)(4 * r4));
+        const uint8_t* p = src + 4 * r4 * (unsigned)c.W + (size_t)wq * 32;
+        uint32_t bits[4] = {0u, 0u, 0u, 0u};
         if (vec) {
-            const uint4 a0 = __ldcs(reinterpret_cast<const uint4*>(p));
-            const uint4 a1 = __ldcs(reinterpret_cast<const uint4*>(p) + 1);
-            bits = nonzero_bytes4(a0.x) | nonzero_bytes4(a0.y) << 4 | nonzero_bytes4(a0.z) << 8 |
-                   nonzero_bytes4(a0.w) << 12 | nonzero_bytes4(a1.x) << 16 | nonzero_bytes4(a1.y) << 20 |
-                   nonzero_bytes4(a1.z) << 24 | nonzero_bytes4(a1.w) << 28;
+            uint4 v[8];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const uint4* q = reinterpret_cast<const uint4*>(p + (size_t)min(r, rows - 1) * (unsigned)c.W);
+                v[2 * r] = __ldcs(q);
+                v[2 * r + 1] = __ldcs(q + 1);
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const uint4 a0 = v[2 * r], a1 = v[2 * r + 1];
+                bits[r] = nonzero_bytes4(a0.x) | nonzero_bytes4(a0.y) << 4 | nonzero_bytes4(a0.z) << 8 |
+                          nonzero_bytes4(a0.w) << 12 | nonzero_bytes4(a1.x) << 16 | nonzero_bytes4(a1.y) << 20 |
+                          nonzero_bytes4(a1.z) << 24 | nonzero_bytes4(a1.w) << 28;
+            }
         } else {
-            const int nb = min(32, c.W - wq * 32);
-            for (int b = 0; b < nb; ++b) bits |= (uint32_t)(p[b] != 0) << b;
+            const int nb = min(32, c.W - (int)wq * 32);
+#pragma unroll 1
+            for (int b = 0; b < nb; ++b)
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+                    if (r < rows) bits[r] |= (uint32_t)(p[(size_t)r * (unsigned)c.W + b] != 0) << b;
         }
-        sil[c.bit_off + i] = bits;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            if (r < rows) sil[(4 * r4 + r) * Wq + wq] = bits[r];
+            else bits[r] = 0u;
+        }
+        // byte k of the four rows' words: the blocked word of columns 8k .. 8k + 7
+        const uint32_t lo01 = __byte_perm(bits[0], bits[1], 0x5140), hi01 = __byte_perm(bits[0], bits[1], 0x7362);
+        const uint32_t lo23 = __byte_perm(bits[2], bits[3], 0x5140), hi23 = __byte_perm(bits[2], bits[3], 0x7362);
+        const size_t at = ((r4 >> 3) * Wq + wq) * 32 + (r4 & 7) * 4;
+        *reinterpret_cast<uint4*>(silb + at) =
+            make_uint4(__byte_perm(lo01, lo23, 0x5410), __byte_perm(lo01, lo23, 0x7632),
+                       __byte_perm(hi01, hi23, 0x5410), __byte_perm(hi01, hi23, 0x7632));
     }
 }
 
-// Sec. II-B-1: the coarse hull over the whole volume.  Occupied voxels also
-// start the union-find forest of Sec. II-B-2: each run of consecutive
-// occupied voxels within a 32-voxel word is one tree, rooted at the run's
-// first voxel (in this word), which is its smallest linear index.
-template <int NC>
-__global__ void __launch_bounds__(256) k_coarse_carve(const __grid_constant__ CamSet cams,
-                                                      const __grid_constant__ Grid g,
+// The coarse table (see CoarseTable), one thread per voxel.
+__global__ void __launch_bounds__(256) k_coarse_table(const __grid_constant__ CamSet cams, const __grid_constant__ Grid g,
+                                                      uint32_t* __restrict__ table, int ncams) {
+    const size_t nvox = (size_t)g.nx * g.ny * g.nz;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvox; i += (size_t)gridDim.x * blockDim.x) {
+        const uint32_t row = (uint32_t)(i / (uint32_t)g.nx);
+        const int x = (int)(i - (size_t)row * (uint32_t)g.nx);
+        const float X = fadd(g.o[0], fmul(fadd((float)x, 0.5f), g.sc));
+        const float Y = fadd(g.o[1], fmul(fadd((float)(int)(row % (uint32_t)g.ny), 0.5f), g.sc));
+        const float Z = fadd(g.o[2], fmul(fadd((float)(int)(row / (uint32_t)g.ny), 0.5f), g.sc));
+        for (int n = 0; n < ncams; ++n) {
+            int px, py;
+            cam_pixel(cams.c[n], X, Y, Z, px, py);
+            const uint32_t tile = (uint32_t)(py >> 5) * (uint32_t)cams.c[n].Wq + (uint32_t)(px >> 5);
+            const uint32_t word = tile * 32u + ((uint32_t)py & 28u) + ((uint32_t)px >> 3 & 3u);
+            table[n * nvox + i] = px < 0 ? kNoPixel : word * 32u + ((uint32_t)py & 3u) * 8u + ((uint32_t)px & 7u);
+        }
+    }
+}
+
+// Sec. II-B-1: the coarse hull over the whole volume, a 32-voxel word of the
+// occupancy bitset at a time, a voxel per lane, in two passes.  Occupied voxels
+// also start the union-find forest of Sec. II-B-2: each run of consecutive
+// occupied voxels within a word is one tree, rooted at the run's first voxel
+// (in this word), which is its smallest linear index.
+//
+// The pixels are read from the coarse table.  A camera's test of a 32-voxel word is then a coalesced load of
+// the table, a gather from the blocked silhouette and a ballot, about 14
+// instructions instead of 55.  The gather bounds the row-major layout:
+// 32 voxels project to a line of some 100 pixels, and unless the line is level
+// each lane reads another row, so another 128-byte line (7 million voxels x
+// 1.4 tests at the 312 G gathers/s measured for the L2 are 31 us a court
+// frame); blocked, the line crosses 4 to 8 lines.
+//
+// The first pass takes every word through the first `levels` cameras, kWords
+// words of a warp in flight together, writes the empty ones and lists the
+// others; the second takes the listed words through the other cameras, one at a
+// time per warp.  In one pass, the warps whose words cross a player's outline
+// held the launch up: 48 to 60 us a court frame however the words were grouped.
+// Court frames (229,000 words, 16 cameras): 52 -> 37 us for one, 1960 -> 1070 us
+// for 64; four 4K court frames (10 abstaining cameras, 23 million voxels each)
+// 453 -> 235 us, against every voxel projected.
+constexpr int kWords = 8;
+template <bool ABSTAIN, bool MORE>            // MORE: levels > 1
+__global__ void __launch_bounds__(256) k_coarse_first(const __grid_constant__ CamSet cams, const __grid_constant__ Grid g,
                                                       const __grid_constant__ Layout L,
-                                                      const __grid_constant__ SlotList sl) {
+                                                      const __grid_constant__ SlotList sl,
+                                                      const __grid_constant__ CoarseTable tab, int levels) {
     pdl_begin();
-    __shared__ unsigned long long sh_t[32];
-    __shared__ unsigned long long sh_n[32];
+    __shared__ unsigned long long sh[32];
+    __shared__ uint32_t s_at[2][8];           // per turn and warp: words it lists, then where they go
     const int slot = sl.s[blockIdx.y];
+    const uint32_t* __restrict__ silb = slot_ptr<uint32_t>(L, slot, L.silb);
+    uint32_t* bits = slot_ptr<uint32_t>(L, slot, L.coarse);
+    uint4* front = slot_ptr<uint4>(L, slot, L.front);
+    SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
+    const int lane = threadIdx.x & 31;
+    const int wid = threadIdx.x >> 5, bw = blockDim.x >> 5;
+    const uint32_t nwords = (uint32_t)g.nz * (uint32_t)g.ny * (uint32_t)g.nxw;
+    const size_t nvox = (size_t)g.nz * g.ny * g.nx;
+    const uint32_t turn = (uint32_t)bw * (uint32_t)kWords;   // words of the block in a turn
+    uint32_t tests = 0;                       // of this lane's words
+    int buf = 0;
+    for (uint32_t b0 = blockIdx.x * turn; b0 < nwords; b0 += gridDim.x * turn, buf ^= 1) {
+        const uint32_t w0 = b0 + (uint32_t)wid * (uint32_t)kWords;
+        // lane q < kWords answers for word w0 + q
+        const uint32_t w = min(w0 + (uint32_t)(lane % kWords), nwords - 1u);
+        const uint32_t row = w / (uint32_t)g.nxw;
+        const int x0 = (int)(w - row * (uint32_t)g.nxw) * 32;
+        const uint32_t first = row * (uint32_t)g.nx + (uint32_t)x0;
+        const int nv = w0 + (uint32_t)(lane % kWords) < nwords ? min(32, g.nx - x0) : 0;
+        uint32_t m[kWords];                   // voxels left of each word (the same in every lane)
+        uint32_t voted = 0u;                  // foreground votes of this lane's word
+        uint32_t any = 0u;
+        {   // camera 0
+            uint32_t e[kWords], word[kWords];
+#pragma unroll
+            for (int q = 0; q < kWords; ++q) {
+                const uint32_t f = __shfl_sync(kFull, first, q);
+                e[q] = lane < __shfl_sync(kFull, nv, q) ? __ldg(tab.e + f + lane) : kNoPixel;
+            }
+#pragma unroll
+            for (int q = 0; q < kWords; ++q) word[q] = e[q] != kNoPixel ? __ldg(silb + cams.c[0].blk_off + (e[q] >> 5)) : 0u;
+#pragma unroll
+            for (int q = 0; q < kWords; ++q) {
+                const bool bit = (word[q] >> (e[q] & 31u)) & 1u;
+                m[q] = __ballot_sync(kFull, bit);
+                if (ABSTAIN) {
+                    if (lane == q) voted = m[q];
+                    const int n = __shfl_sync(kFull, nv, q);
+                    m[q] |= __ballot_sync(kFull, e[q] == kNoPixel) & (n > 0 ? kFull >> (32 - n) : 0u);
+                }
+                any |= m[q];
+            }
+            if (lane < kWords) tests += (uint32_t)nv;
+        }
+        const uint32_t* te = tab.e + nvox + lane;
+#pragma unroll 1
+        for (int c = 1; MORE && c < levels && any; ++c, te += nvox) {
+            const uint32_t* __restrict__ sb = silb + cams.c[c].blk_off;
+            uint32_t e[kWords], word[kWords];
+#pragma unroll
+            for (int q = 0; q < kWords; ++q) {
+                const uint32_t f = __shfl_sync(kFull, first, q);
+                e[q] = (m[q] >> lane) & 1u ? __ldg(te + f) : kNoPixel;
+            }
+#pragma unroll
+            for (int q = 0; q < kWords; ++q) word[q] = e[q] != kNoPixel ? __ldg(sb + (e[q] >> 5)) : 0u;
+            any = 0u;
+#pragma unroll
+            for (int q = 0; q < kWords; ++q) {
+                tests += lane == q ? (uint32_t)__popc(m[q]) : 0u;
+                const bool bit = (word[q] >> (e[q] & 31u)) & 1u;
+                const uint32_t v = __ballot_sync(kFull, bit);
+                if (ABSTAIN) {
+                    if (lane == q) voted |= v;
+                    m[q] &= v | __ballot_sync(kFull, e[q] == kNoPixel);
+                } else {
+                    m[q] = v;
+                }
+                any |= m[q];
+            }
+        }
+        uint32_t left = 0u;
+#pragma unroll
+        for (int q = 0; q < kWords; ++q) left = lane == q ? m[q] : left;
+        const bool own = lane < kWords && nv > 0;
+        if (own && !left) bits[w] = 0u;
+        // places in the list, one atomic a block and turn (one a warp took 20 us
+        // of a single frame: a counter serves about one atomic a nanosecond)
+        const uint32_t who = __ballot_sync(kFull, own && left != 0u);
+        if (lane == 0) s_at[buf][wid] = (uint32_t)__popc(who);
+        __syncthreads();
+        if (wid == 0) {
+            const uint32_t n = lane < bw ? s_at[buf][lane] : 0u;
+            uint32_t incl = n;
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const uint32_t all = __shfl_sync(kFull, incl, 7);
+            uint32_t at = 0;
+            if (lane == 0 && all) at = atomicAdd(&info->n_front, all);
+            at = __shfl_sync(kFull, at, 0);
+            if (lane < bw) s_at[buf][lane] = at + incl - n;
+        }
+        __syncthreads();
+        // (a word is listed once, so the places stay below nwords from a counter that started at zero)
+        const uint32_t at = s_at[buf][wid] + (uint32_t)__popc(who & ((1u << lane) - 1u));
+        if (((who >> lane) & 1u) && at < nwords) front[at] = make_uint4(w, left, voted, first);
+    }
+    const unsigned long long t = block_sum<unsigned long long>(tests, sh);
+    if (threadIdx.x == 0 && t) atomicAdd(&info->tests_coarse, t);
+}
+
+template <bool ABSTAIN>
+__global__ void __launch_bounds__(256) k_coarse_rest(const __grid_constant__ CamSet cams, const __grid_constant__ Grid g,
+                                                     const __grid_constant__ Layout L,
+                                                     const __grid_constant__ SlotList sl,
+                                                     const __grid_constant__ CoarseTable tab, int levels) {
+    pdl_begin();
+    __shared__ uint32_t s_blk[FVV_MAX_CAMS];
+    __shared__ unsigned long long sh[32];
+    const int slot = sl.s[blockIdx.y];
+    SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
+    const uint32_t nfront = min(info->n_front, (uint32_t)g.nz * (uint32_t)g.ny * (uint32_t)g.nxw);
+    if (((blockIdx.x * blockDim.x) >> 5) >= nfront) return;   // the whole block
+    for (int n = threadIdx.x; n < cams.n; n += blockDim.x) s_blk[n] = cams.c[n].blk_off;
+    __syncthreads();
+    const uint32_t* __restrict__ silb = slot_ptr<uint32_t>(L, slot, L.silb);
     const uint32_t* __restrict__ sil = slot_ptr<uint32_t>(L, slot, L.sil);
     uint32_t* bits = slot_ptr<uint32_t>(L, slot, L.coarse);
     int* parent = slot_ptr<int>(L, slot, L.parent);
-    const uint32_t nrows = (uint32_t)g.nz * (uint32_t)g.ny;
+    const uint4* front = slot_ptr<uint4>(L, slot, L.front);
     const int lane = threadIdx.x & 31;
+    const size_t nvox = (size_t)g.nz * g.ny * g.nx;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    uint32_t tests = 0, on_count = 0;
-    // a warp takes a whole row (y, z) and walks its words, so the row is
-    // decoded once and Y, Z are formed once
-    for (uint32_t row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < nrows; row += nwarps) {
-        const int y = (int)(row % (uint32_t)g.ny), z = (int)(row / (uint32_t)g.ny);
-        const float Y = fadd(g.o[1], fmul(fadd((float)y, 0.5f), g.sc));
-        const float Z = fadd(g.o[2], fmul(fadd((float)z, 0.5f), g.sc));
-        for (int wx = 0; wx < g.nxw; ++wx) {
-            const int x = wx * 32 + lane;
+    uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    unsigned long long tests = 0;             // (the same in every lane)
+    uint32_t on_count = 0;
+    uint4 f = i < nfront ? __ldcg(front + i) : make_uint4(0u, 0u, 0u, 0u);
+    for (; i < nfront; i += nwarps) {
+        const uint4 cur = f;
+        if (i + nwarps < nfront) f = __ldcg(front + i + nwarps);
+        uint32_t m = cur.y;                   // voxels left (the same in every lane)
+        bool voted = (cur.z >> lane) & 1u;
+        const uint32_t* te = tab.e + levels * nvox + cur.w + (uint32_t)lane;
+        int n = levels;
+        uint32_t e = n < tab.n && ((m >> lane) & 1u) ? __ldg(te) : kNoPixel;
+        for (; n < tab.n && m; ++n) {
+            const bool live = (m >> lane) & 1u;
+            const uint32_t word = live && e != kNoPixel ? __ldg(silb + s_blk[n] + (e >> 5)) : 0u;
+            // the next camera's entries are on their way while this one's gather is
+            te += nvox;
+            const uint32_t next = live && n + 1 < tab.n ? __ldg(te) : kNoPixel;
+            tests += (unsigned)__popc(m);
+            const bool bit = (word >> (e & 31u)) & 1u;
+            if (ABSTAIN) voted |= bit;
+            m = __ballot_sync(kFull, live && (bit || (ABSTAIN && e == kNoPixel)));
+            e = next;
+        }
+        if (m && n < cams.n) {                // cameras past the table
+            const uint32_t row = cur.w / (uint32_t)g.nx;
+            const int x = (int)(cur.w - row * (uint32_t)g.nx) + lane;
             const float X = fadd(g.o[0], fmul(fadd((float)x, 0.5f), g.sc));
-            const bool on = warp_test<NC>(cams, sil, X, Y, Z, x < g.nx, tests);
-            const uint32_t word = __ballot_sync(kFull, on);
-            if (on) {
-                const uint32_t starts = word & ~(word << 1);   // first voxel of each run
-                const int run0 = 31 - __clz(starts & (0xFFFFFFFFu >> (31 - lane)));
-                parent[(int)(row * (uint32_t)g.nx) + x] = (int)(row * (uint32_t)g.nx) + wx * 32 + run0;
-            }
-            if (lane == 0) {
-                bits[row * (uint32_t)g.nxw + (uint32_t)wx] = word;
-                on_count += __popc(word);
+            const float Y = fadd(g.o[1], fmul(fadd((float)(int)(row % (uint32_t)g.ny), 0.5f), g.sc));
+            const float Z = fadd(g.o[2], fmul(fadd((float)(int)(row / (uint32_t)g.ny), 0.5f), g.sc));
+#pragma unroll 1
+            for (; n < cams.n && m; ++n) {
+                bool live = (m >> lane) & 1u;
+                tests += (unsigned)__popc(m);
+                if (live) test_cam<ABSTAIN>(cams.c[n], sil, X, Y, Z, live, voted);
+                m = __ballot_sync(kFull, live);
             }
         }
+        if (ABSTAIN) m = __ballot_sync(kFull, ((m >> lane) & 1u) && voted);
+        // occupied voxels start the union-find forest: each run one tree
+        if ((m >> lane) & 1u) {
+            const uint32_t starts = m & ~(m << 1);   // first voxel of each run
+            const int run0 = 31 - __clz(starts & (0xFFFFFFFFu >> (31 - lane)));
+            parent[cur.w + (uint32_t)lane] = (int)cur.w + run0;
+        }
+        if (lane == 0) {
+            bits[cur.x] = m;
+            on_count += __popc(m);
+        }
     }
-    const unsigned long long t = block_sum<unsigned long long>(tests, sh_t);
-    const unsigned long long c = block_sum<unsigned long long>(on_count, sh_n);
+    const unsigned long long t = block_sum<unsigned long long>(lane == 0 ? tests : 0ull, sh);
+    const unsigned long long c = block_sum<unsigned long long>((unsigned long long)on_count, sh);
     if (threadIdx.x == 0) {
-        SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
         if (t) atomicAdd(&info->tests_coarse, t);
         if (c) atomicAdd(&info->n_on, (uint32_t)c);
     }
@@ -268,7 +479,6 @@ __device__ __forceinline__ void fine_tiles(const Grid& g, const SmemCam* sc, int
                                            const DRoi* rois, const uint32_t* __restrict__ sil, uint32_t* fine,
                                            uint32_t* next_tile, uint32_t claim, unsigned long long& tests,
                                            uint32_t& reads) {
-    constexpr int T = 32 / CG;
     constexpr int kSubsY = TY / kSubY, kSubs = kSubsY * (TZ / kSubZ);
     constexpr uint64_t kGroup = (1ull << CG) - 1ull;
     const int lane = threadIdx.x & 31, own = lane % CG;
@@ -513,7 +723,8 @@ cudaError_t launch_debug_pixels(const CamSet& cams, int cam, long long n, const 
 cudaError_t launch_pack(const CamSet& cams, const Layout& L, int n_frames, const int* slots,
                         const uint8_t* const* src, bool host_src, int sms, cudaStream_t st) {
     size_t max_words = 0;
-    for (int n = 0; n < cams.n; ++n) max_words = std::max(max_words, (size_t)cams.c[n].H * (unsigned)cams.c[n].Wq);
+    for (int n = 0; n < cams.n; ++n)
+        max_words = std::max(max_words, (size_t)((cams.c[n].H + 3) / 4) * (unsigned)cams.c[n].Wq);   // a thread per 4 rows
     const int per_launch = std::min(kPackPtrs / 4, kPackPtrs / std::max(1, cams.n));
     // Device sources: enough blocks to stream HBM at full rate.  Masks read in
     // place from host memory are bound by the host link, which about two
@@ -536,13 +747,43 @@ cudaError_t launch_pack(const CamSet& cams, const Layout& L, int n_frames, const
     return cudaGetLastError();
 }
 
-cudaError_t launch_coarse_carve(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl, int sms,
-                                const Tuning& tu, cudaStream_t st) {
-    const long long rows = (long long)g.nz * g.ny;    // a warp per row
+cudaError_t launch_coarse_table(const CamSet& cams, const Grid& g, uint32_t* e, int n, cudaStream_t st) {
+    const size_t nvox = (size_t)g.nx * g.ny * g.nz;
+    k_coarse_table<<<(unsigned)std::min<size_t>((nvox + 255) / 256, 16384), 256, 0, st>>>(cams, g, e, n);
+    return cudaGetLastError();
+}
+
+namespace {
+__global__ void k_reset_coarse(const __grid_constant__ Layout L, const __grid_constant__ SlotList sl) {
+    pdl_begin();
+    if (threadIdx.x == 0) slot_ptr<SlotInfo>(L, sl.s[blockIdx.x], L.info)->n_front = 0u;
+}
+}  // namespace
+
+cudaError_t launch_reset_coarse(const Layout& L, const SlotList& sl, cudaStream_t st) {
+    return launch_pdl(k_reset_coarse, dim3(sl.n), dim3(32), 0, st, L, sl);
+}
+
+cudaError_t launch_coarse_carve(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl,
+                                const CoarseTable& tab, int sms, const Tuning& tu, cudaStream_t st) {
     const int th = tu.threads[FVV_TUNE_COARSE];
-    const int gx = tuned_grid(tu, FVV_TUNE_COARSE, sms, sl.n, rows * 32);
-#define FVV_LAUNCH(NC) launch_pdl(k_coarse_carve<NC>, dim3(gx, sl.n), dim3(th), 0, st, cams, g, L, sl)
-    FVV_DISPATCH_NC(cams.n, FVV_LAUNCH)
+    const long long words = (long long)g.nz * g.ny * g.nxw;
+    const int g1 = tuned_grid(tu, FVV_TUNE_COARSE, sms, sl.n, (words + kWords - 1) / kWords * 32);
+    const int g2 = tuned_grid(tu, FVV_TUNE_COARSE, sms, sl.n, words * 32);
+    // Cameras of the first pass: three where the launch is too small to hide the
+    // second pass's chains of loads (a court frame, 229,000 words: 49 us with one
+    // camera, 37 with three), else one (64 frames: 988 us against 1085).
+    const int levels = std::min(tab.n, words * sl.n < 600000 ? 3 : 1);
+#define FVV_LAUNCH(A, M) launch_pdl(k_coarse_first<A, M>, dim3(g1, sl.n), dim3(th), 0, st, cams, g, L, sl, tab, levels)
+    if (cams.oob == FVV_OOB_ABSTAIN) {
+        if (levels > 1) FVV_LAUNCH(true, true);
+        else FVV_LAUNCH(true, false);
+        launch_pdl(k_coarse_rest<true>, dim3(g2, sl.n), dim3(th), 0, st, cams, g, L, sl, tab, levels);
+    } else {
+        if (levels > 1) FVV_LAUNCH(false, true);
+        else FVV_LAUNCH(false, false);
+        launch_pdl(k_coarse_rest<false>, dim3(g2, sl.n), dim3(th), 0, st, cams, g, L, sl, tab, levels);
+    }
 #undef FVV_LAUNCH
     return cudaGetLastError();
 }

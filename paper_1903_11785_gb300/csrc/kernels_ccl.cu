@@ -455,7 +455,7 @@ __global__ void k_debug_labels(const __grid_constant__ Grid g, const __grid_cons
 
 // A given coarse grid (parity tests of the labelling): copies the words into
 // the slot with the bits past nx cleared, and starts the union-find forest
-// exactly as k_coarse_carve does (each run of a word one tree rooted at its
+// exactly as k_coarse_rest does (each run of a word one tree rooted at its
 // first voxel), counting the occupied voxels.  One thread per word.
 namespace {
 __global__ void k_debug_seed(const __grid_constant__ Grid g, const __grid_constant__ Layout L, int slot,
