@@ -199,6 +199,22 @@ __device__ __forceinline__ void load_smem_cams(const CamSet& cams, int n, SmemCa
     }
 }
 
+// Silhouette bit of a point that is known to be in front of camera c and
+// inside its image (where `on`; 0 elsewhere): cam_bit without the clamps and
+// the tests.
+__device__ __forceinline__ uint32_t cam_bit_inside(const SmemCam& c, const uint32_t* __restrict__ sil, float X, float Y,
+                                                   float Z, bool on) {
+    float xp, yp, wp;
+    project(c.P, X, Y, Z, xp, yp, wp);
+    const float r = rcp_approx(wp);
+    const float tx = __fadd_rz(fmul(xp, r), 8388608.0f), ty = __fadd_rz(fmul(yp, r), 8388608.0f);
+    const float rx = __fmaf_rn(-fsub(tx, 8388608.0f), wp, xp), ry = __fmaf_rn(-fsub(ty, 8388608.0f), wp, yp);
+    const unsigned px = (__float_as_uint(tx) & 0x7FFFFFu) + (rx >= wp ? 1u : 0u) - (rx < 0.0f ? 1u : 0u);
+    const unsigned py = (__float_as_uint(ty) & 0x7FFFFFu) + (ry >= wp ? 1u : 0u) - (ry < 0.0f ? 1u : 0u);
+    const uint32_t word = on ? __ldg(sil + c.bit_off + py * (unsigned)c.Wq + (px >> 5)) : 0u;
+    return (word >> (px & 31u)) & 1u;
+}
+
 // ---- pixel cells: which pixel centres a vertex lies between, per camera
 //
 // A triangle covers no pixel centre of a camera if no column of centres, or

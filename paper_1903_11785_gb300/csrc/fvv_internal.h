@@ -196,6 +196,7 @@ inline Tuning default_tuning() {
     }
     t.waves[FVV_TUNE_ZBUFFER] = 16;
     t.waves[FVV_TUNE_COARSE] = 16;
+    t.waves[FVV_TUNE_BISECT] = 16;
     t.waves[FVV_TUNE_FINE] = 16;
     t.fine_tile = FVV_TILE_4x4x8;
     t.zb_cams = 4;

@@ -471,40 +471,52 @@ __global__ void __launch_bounds__(kChunk) k_mc_compact(const __grid_constant__ G
     }
 }
 
-// Does camera c see every point the bisection of the edge (a, b) can test in
-// its silhouette?  True when the pixels of the box spanned by the ends'
-// approximate image positions, widened by the camera's margins (see
-// segment_margins on the host), are all inside the image and set.  Boxes
-// wider than 32 or taller than 8 pixels are not scanned (false).
-template <class CamT>
-__device__ __forceinline__ bool segment_all_fg(const CamT& c, const uint32_t* __restrict__ sil, const float* a,
-                                               const float* b, unsigned long long& reads) {
-    if (!(c.du >= 0.0f)) return false;
-    float xa, ya, wa, xb, yb, wb;
-    project(c.P, a[0], a[1], a[2], xa, ya, wa);
-    project(c.P, b[0], b[1], b[2], xb, yb, wb);
-    if (!(wa > 0.0f && wb > 0.0f)) return false;
-    const float ra = rcp_approx(wa), rb = rcp_approx(wb);
-    const float ua = fmul(xa, ra), va = fmul(ya, ra), ub = fmul(xb, rb), vb = fmul(yb, rb);
-    const float u0 = fsub(fminf(ua, ub), c.du), u1 = fadd(fmaxf(ua, ub), c.du);
-    const float v0 = fsub(fminf(va, vb), c.dv), v1 = fadd(fmaxf(va, vb), c.dv);
-    if (!(u0 >= 0.0f && v0 >= 0.0f && u1 < c.Wf && v1 < c.Hf)) return false;
-    const int x0 = (int)u0, x1 = (int)u1, y0 = (int)v0, y1 = (int)v1;   // truncation = floor here
-    if (x1 - x0 > 31 || y1 - y0 > 7) return false;
-    const int w0 = x0 >> 5, w1 = x1 >> 5;
-    const uint32_t m0 = ~0u << (x0 & 31), m1 = ~0u >> (31 - (x1 & 31));
-    const uint32_t* row = sil + c.bit_off + (unsigned)y0 * (unsigned)c.Wq;
-    bool all = true;
-    for (int y = y0; y <= y1; ++y, row += c.Wq) {
-        if (w0 == w1) {
-            all &= (__ldg(row + w0) & (m0 & m1)) == (m0 & m1);
-        } else {
-            all &= (__ldg(row + w0) & m0) == m0;
-            all &= (__ldg(row + w1) & m1) == m1;
+// What camera c sees of the grid edge m - h .. m + h, that is of every point
+// its bisection can test.  With u = x'/w' at m and (dx, dy, dw) the rows of P
+// applied to h, the ends lie at u +- (dx - u dw) / (w' +- dw), so within
+// |dx - u dw| / (w' - |dw|) of u, and 1 / (w' - |dw|) <= (1 + 2 |dw| / w') / w'
+// where |dw| <= w' / 2.  The box of that, widened by 0.2% and 2^-10 pixels for
+// the bound's own roundings and by the camera's margins (segment_margins on the
+// host; its allowance of 32 half ulps for a point's deviation holds 30
+// midpoints and m), holds every tested point's pixel.  all_fg: the box's pixels
+// are all inside the image and set.  inside: they are all inside the image.
+// Boxes wider than 32 or taller than 8 pixels are not scanned.
+__device__ __forceinline__ void check_edge(const SmemCam& c, const uint32_t* __restrict__ sil, const float* m,
+                                           const float* h, bool& all_fg, bool& inside, uint32_t& reads) {
+    all_fg = inside = false;
+    float xh, yh, wh;
+    project(c.P, m[0], m[1], m[2], xh, yh, wh);
+    const float dx = __fmaf_rn(c.P[0], h[0], __fmaf_rn(c.P[1], h[1], fmul(c.P[2], h[2])));
+    const float dy = __fmaf_rn(c.P[4], h[0], __fmaf_rn(c.P[5], h[1], fmul(c.P[6], h[2])));
+    const float dw = __fmaf_rn(c.P[8], h[0], __fmaf_rn(c.P[9], h[1], fmul(c.P[10], h[2])));
+    const float r = rcp_approx(wh), u = fmul(xh, r), v = fmul(yh, r);
+    const float rw = fmul(r, __fmaf_rn(fmul(fabsf(dw), r), 2.0f, 1.002f));
+    const float eu = __fmaf_rn(fabsf(__fmaf_rn(-u, dw, dx)), rw, fadd(c.du, 0x1p-10f));
+    const float ev = __fmaf_rn(fabsf(__fmaf_rn(-v, dw, dy)), rw, fadd(c.dv, 0x1p-10f));
+    const float u0 = fsub(u, eu), u1 = fadd(u, eu), v0 = fsub(v, ev), v1 = fadd(v, ev);
+    inside = wh > fmul(2.0f, fabsf(dw)) && c.du >= 0.0f && u0 >= 0.0f && v0 >= 0.0f && u1 < c.Wf && v1 < c.Hf;
+    if (!inside) return;
+    // floors on the FMA pipe: kMagic + floor, and differences of the bits
+    const int x0 = __float_as_int(__fadd_rd(u0, kMagic)) - 0x4B400000, y0 = __float_as_int(__fadd_rd(v0, kMagic)) - 0x4B400000;
+    const int nx = __float_as_int(__fadd_rd(u1, kMagic)) - 0x4B400000 - x0, ny = __float_as_int(__fadd_rd(v1, kMagic)) - 0x4B400000 - y0;
+    if (nx > 31 || ny > 7) return;
+    const uint32_t want = (2u << nx) - 1u;           // nx + 1 pixels from x0 on
+    const int sh = x0 & 31, two = sh + nx > 31 ? 1 : 0;
+    const uint32_t* row = sil + c.bit_off + (unsigned)y0 * (unsigned)c.Wq + ((unsigned)x0 >> 5);
+    uint32_t miss = 0u;
+    for (int y = 0; y <= ny; y += 2) {               // two rows a turn, the last one twice if they are odd in number
+        const uint32_t* next = row + (y < ny ? c.Wq : 0);
+        const uint32_t a0 = __ldg(row), b0 = __ldg(next);
+        uint32_t a1 = 0u, b1 = 0u;
+        if (two) {
+            a1 = __ldg(row + 1);
+            b1 = __ldg(next + 1);
         }
+        miss |= ~(__funnelshift_r(a0, a1, sh) & __funnelshift_r(b0, b1, sh)) & want;
+        row = next + c.Wq;
     }
-    reads += (unsigned)((y1 - y0 + 1) * (w1 - w0 + 1));
-    return all;
+    reads += (unsigned)((ny + 1) << two);
+    all_fg = miss == 0u;
 }
 
 // Sec. II-C, exact intersection: between the ON end a and the OFF end b of a
@@ -512,7 +524,7 @@ __device__ __forceinline__ bool segment_all_fg(const CamT& c, const uint32_t* __
 // the vertex is the final midpoint.
 //
 // Every point tested lies on the edge (up to rounding), so a camera that sees
-// the whole edge inside its silhouette (segment_all_fg) votes foreground for
+// the whole edge inside its silhouette (check_edge) votes foreground for
 // all of them: it is decided once per edge, and only the other cameras are
 // tested at each midpoint, from the vertex's list.  A midpoint's first
 // background camera in index order is then the first listed camera that votes
@@ -520,76 +532,97 @@ __device__ __forceinline__ bool segment_all_fg(const CamT& c, const uint32_t* __
 // or N when the midpoint is occupied) are those of the plain early-exit loop
 // over all cameras.
 
-// The ends of vertex record `rec`'s grid edge: a the ON sample, b the OFF one.
-__device__ __forceinline__ void bisect_ends(uint64_t rec, const DRoi* rois, const Grid& g, float* a, float* b) {
-    const int k = (int)(rec & 0x3FFFu), axis = (int)(rec >> 14 & 3u), s0 = (int)(rec >> 16 & 1u);
+// A grid edge: its point X with coordinate `axis` running from a, the ON
+// sample's, to b, the OFF one's.
+struct Edge {
+    float X[3], a, b;
+    int axis;
+};
+
+__device__ __forceinline__ Edge edge_of_record(uint64_t rec, const DRoi* rois, const Grid& g) {
+    const int k = (int)(rec & 0x3FFFu), s0 = (int)(rec >> 16 & 1u);
     const int q[3] = {(int)(rec >> 17 & 0x7FFFu), (int)(rec >> 32 & 0x7FFFu), (int)(rec >> 47 & 0x7FFFu)};
     const DRoi& r = rois[k];
+    Edge e;
+    e.axis = (int)(rec >> 14 & 3u);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const float c0 = fadd(r.fo[d], fmul(fadd((float)(q[d] - 1), 0.5f), g.sf));
-        const float c1 = fadd(r.fo[d], fmul(fadd((float)(q[d] - 1 + (d == axis)), 0.5f), g.sf));
-        a[d] = s0 ? c0 : c1;
-        b[d] = s0 ? c1 : c0;
-    }
+    for (int d = 0; d < 3; ++d) e.X[d] = fadd(r.fo[d], fmul(fadd((float)(q[d] - 1), 0.5f), g.sf));
+    const int qa = e.axis == 0 ? q[0] : e.axis == 1 ? q[1] : q[2];
+    const float c0 = e.axis == 0 ? e.X[0] : e.axis == 1 ? e.X[1] : e.X[2];
+    const float c1 = fadd(r.fo[e.axis], fmul(fadd((float)qa, 0.5f), g.sf));
+    e.a = s0 ? c0 : c1;
+    e.b = s0 ? c1 : c0;
+    return e;
 }
 
-// The cameras that must be tested at each midpoint of the edge (a, b) (bit n:
-// camera n); seen_fg: some camera votes foreground on the whole edge.
-__device__ __forceinline__ uint64_t bisect_undecided(const SmemCam* sc, int ncam, const uint32_t* __restrict__ sil,
-                                                     const float* a, const float* b, bool& seen_fg,
-                                                     unsigned long long& reads) {
-    uint64_t undecided = 0;
+// The point of edge e whose running coordinate is t.
+__device__ __forceinline__ void edge_point(const Edge& e, float t, float* p) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) p[d] = e.axis == d ? t : e.X[d];
+}
+
+// The cameras that must be tested at each midpoint of edge e (bit n: camera
+// n); seen_fg: some camera votes foreground on the whole edge; inside: the edge
+// is inside the image of every camera to be tested.
+template <class Mask>
+__device__ __forceinline__ Mask edge_undecided(const SmemCam* sc, int ncam, const uint32_t* __restrict__ sil,
+                                               const Edge& e, bool& seen_fg, bool& inside, uint32_t& reads) {
+    Mask undecided = 0;
     seen_fg = false;
-    // one compact loop over the cameras' fields in shared memory (the camera
-    // is the same in every lane): 16 inlined copies of this check cost more
-    // in instruction-cache misses than the loads
-#pragma unroll 1
+    inside = true;
+    float m[3], h[3];
+    edge_point(e, fmul(fadd(e.a, e.b), 0.5f), m);
+    const float half = fmul(fsub(e.b, e.a), 0.5f);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) h[d] = e.axis == d ? half : 0.0f;
+    // the cameras' fields come from shared memory (the camera is the same in
+    // every lane); four checks at a time overlap their loads (one at a time: 3772
+    // instead of 3636 us for 64 court frames), 16 inlined copies with constant
+    // operands cost more in instruction-cache misses than the loads
+#pragma unroll 4
     for (int n = 0; n < ncam; ++n) {
-        const bool fg = segment_all_fg(sc[n], sil, a, b, reads);
-        undecided |= fg ? 0ull : 1ull << n;
+        bool fg, in;
+        check_edge(sc[n], sil, m, h, fg, in, reads);
+        undecided |= fg ? (Mask)0 : (Mask)1 << n;
         seen_fg |= fg;
+        inside &= in;                        // (a camera that is not inside is never decided)
     }
     return undecided;
 }
 
-// The `steps` bisection steps of the edge (a, b) with the cameras of
-// `undecided` tested at each midpoint; a and b end as the last bracket.
-__device__ __forceinline__ void bisect_steps(const SmemCam* sc, int ncam, const uint32_t* __restrict__ sil, int steps,
-                                             bool abstain, uint64_t undecided, bool seen_fg, float* a, float* b,
-                                             unsigned long long& tests, unsigned long long& reads) {
+__device__ __forceinline__ int first_bit(uint32_t m) { return __ffs((int)m) - 1; }
+__device__ __forceinline__ int first_bit(uint64_t m) { return __ffsll((long long)m) - 1; }
+
+// The `steps` bisection steps of edge e with the cameras of `undecided` tested at
+// each midpoint; e.a and e.b end as the last bracket.  INSIDE: the edge is
+// inside every such camera's image (no clamps, no tests of the pixel).
+template <bool INSIDE, class Mask>
+__device__ __forceinline__ void edge_bisect(const SmemCam* sc, int ncam, const uint32_t* __restrict__ sil, int steps,
+                                            bool abstain, Mask undecided, bool seen_fg, Edge& e, uint32_t& tests,
+                                            uint32_t& reads) {
     for (int it = 0; it < steps; ++it) {
+        const float t = fmul(fadd(e.a, e.b), 0.5f);
         float m[3];
-#pragma unroll
-        for (int d = 0; d < 3; ++d) m[d] = fmul(fadd(a[d], b[d]), 0.5f);
+        edge_point(e, t, m);
         int stop = -1;
         bool voted = !abstain || seen_fg;
-        for (uint64_t u = undecided; u; u &= u - 1) {
-            const int n = __ffsll((long long)u) - 1;
-            const SmemCam& c = sc[n];
-            float xp, yp, wp;
-            project(c.P, m[0], m[1], m[2], xp, yp, wp);
-            const float rw = rcp_approx(wp);
-            const int px = pixel_floor(xp, wp, rw, c.Wf);
-            const int py = pixel_floor(yp, wp, rw, c.Hf);
-            const bool in = wp > 0.0f && (unsigned)px < (unsigned)c.W && (unsigned)py < (unsigned)c.H;
-            const uint32_t word =
-                in ? __ldg(sil + c.bit_off + (unsigned)py * (unsigned)c.Wq + ((unsigned)px >> 5)) : 0u;
+        for (Mask u = undecided; u; u &= u - 1) {
+            const int n = first_bit(u);
+            bool in = true;
+            uint32_t bit;
+            if constexpr (INSIDE) bit = cam_bit_inside(sc[n], sil, m[0], m[1], m[2], true);
+            else bit = cam_bit(sc[n], sil, m[0], m[1], m[2], in);
             reads += in ? 1u : 0u;
-            const bool bit = (word >> (px & 31)) & 1u;
             if (abstain ? (in && !bit) : !bit) {
                 stop = n;
                 break;
             }
-            voted |= bit;
+            voted |= bit != 0u;
         }
         tests += stop < 0 ? (unsigned)ncam : (unsigned)(stop + 1);
         const bool on = stop < 0 && voted;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            a[d] = on ? m[d] : a[d];
-            b[d] = on ? b[d] : m[d];
-        }
+        e.a = on ? t : e.a;
+        e.b = on ? e.b : t;
     }
 }
 
@@ -612,9 +645,10 @@ static_assert(kSortBuckets * kBisectWin % 32 == 0 && kBisectWin <= 8, "sort coun
 
 // Per-warp shared memory of the sorted path (dynamic shared memory, one per
 // warp of the block).
+template <class Mask>
 struct BisectWarpSmem {
-    unsigned long long und[32 * kBisectWin];   // undecided cameras, in window order
-    uint32_t id[32 * kBisectWin];              // vertex | seen_fg << 31, or ~0u for an empty place
+    Mask und[32 * kBisectWin];                 // undecided cameras, in window order
+    uint32_t id[32 * kBisectWin];              // vertex | inside << 30 | seen_fg << 31, or ~0u for an empty place
     uint8_t perm[32 * kBisectWin];             // window places in sorted order
     int cnt[kSortBuckets * kBisectWin];        // bucket-major counts, then their exclusive prefix
 };
@@ -630,7 +664,12 @@ struct BisectWarpSmem {
 // block barrier) and then bisects them 32 at a time in that order, so that a
 // warp's lanes walk lists of about the same length.  Each vertex's
 // arithmetic is the same in both orders; only the lane that does it changes.
-template <int NC>
+//
+// Bound by instruction issue.  Mask is uint32_t for up to 32 cameras.  64 court
+// frames 4655 -> 3636 us, one 109 -> 83 us, four 4K court frames 126 -> 77 us
+// against projecting both ends of an edge in every camera and all three
+// coordinates of every midpoint with the tests a point anywhere needs.
+template <class Mask>
 __global__ void __launch_bounds__(256) k_bisect(const __grid_constant__ CamSet cams, const __grid_constant__ Grid g,
                                                 const __grid_constant__ Layout L, const __grid_constant__ SlotList sl,
                                                 uint32_t resident_warps) {
@@ -639,8 +678,8 @@ __global__ void __launch_bounds__(256) k_bisect(const __grid_constant__ CamSet c
     __shared__ SmemCam sc[FVV_MAX_CAMS];
     __shared__ CellCam cc[FVV_MAX_CAMS];
     extern __shared__ __align__(16) unsigned char bisect_smem[];   // BisectWarpSmem per warp
-    BisectWarpSmem* wsm = reinterpret_cast<BisectWarpSmem*>(bisect_smem);
-    const int ncam = NC > 0 ? NC : cams.n;
+    BisectWarpSmem<Mask>* wsm = reinterpret_cast<BisectWarpSmem<Mask>*>(bisect_smem);
+    const int ncam = cams.n;
     load_smem_cams(cams, ncam, sc);
     load_cell_cams(cams, ncam, cc);
     __syncthreads();
@@ -658,20 +697,39 @@ __global__ void __launch_bounds__(256) k_bisect(const __grid_constant__ CamSet c
     int kv = 1;                                    // the same in every block of the slot
     for (int k = kBisectWin; k >= 2; k >>= 1)
         if (kv == 1 && (unsigned long long)nv >= 64ull * resident_warps * (unsigned)k) kv = k;
+    // the steps of vertex i (edge e, undecided cameras `und`; where `have`), and
+    // its results; all lanes of a warp call it together and take the same form
+    auto finish = [&](bool have, uint32_t i, Edge& e, Mask und, bool seen_fg, bool inside) {
+        const bool all_inside = __all_sync(kFull, inside || !have);
+        if (!have) return;
+        uint32_t t = 0, rd = 0;
+        if (all_inside) edge_bisect<true>(sc, ncam, sil, g.steps, abstain, und, seen_fg, e, t, rd);
+        else edge_bisect<false>(sc, ncam, sil, g.steps, abstain, und, seen_fg, e, t, rd);
+        tests += t;
+        reads += rd;
+        float v[3];
+        edge_point(e, fmul(fadd(e.a, e.b), 0.5f), v);
+        store_vertex(verts, vcell, i, v, sc, cc, ncam);
+    };
     if (kv == 1 || g.steps == 0) {
-        for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += nthreads) {
-            float a[3], b[3];
-            bisect_ends(vrec[i], rois, g, a, b);
-            bool seen_fg = false;
-            const uint64_t undecided = g.steps > 0 ? bisect_undecided(sc, ncam, sil, a, b, seen_fg, reads) : 0ull;
-            bisect_steps(sc, ncam, sil, g.steps, abstain, undecided, seen_fg, a, b, tests, reads);
-#pragma unroll
-            for (int d = 0; d < 3; ++d) a[d] = fmul(fadd(a[d], b[d]), 0.5f);
-            store_vertex(verts, vcell, i, a, sc, cc, ncam);
+        const uint32_t lane = threadIdx.x & 31;
+        for (uint32_t base = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < nv; base += nthreads) {
+            const uint32_t i = base + lane;
+            const bool have = i < nv;
+            Edge e{};
+            Mask und = 0;
+            bool seen_fg = false, inside = true;
+            if (have) {
+                e = edge_of_record(vrec[i], rois, g);
+                uint32_t rd = 0;
+                if (g.steps > 0) und = edge_undecided<Mask>(sc, ncam, sil, e, seen_fg, inside, rd);
+                reads += rd;
+            }
+            finish(have, i, e, und, seen_fg, inside);
         }
     } else {
         const int lane = threadIdx.x & 31;
-        BisectWarpSmem& w = wsm[threadIdx.x >> 5];
+        BisectWarpSmem<Mask>& w = wsm[threadIdx.x >> 5];
         const uint32_t win = 32u * (uint32_t)kv;
         const uint32_t nwarps = nthreads >> 5;
         // windows of the slot's vertices, taken by the warps in turn (the loop
@@ -681,14 +739,15 @@ __global__ void __launch_bounds__(256) k_bisect(const __grid_constant__ CamSet c
             // (1) each lane's kv vertices: their undecided cameras
             for (int j = 0; j < kv; ++j) {
                 const uint32_t i = base + (uint32_t)(j * 32 + lane);
-                uint64_t und = 0;
+                Mask und = 0;
                 uint32_t id = ~0u;
                 if (i < nv) {
-                    float a[3], b[3];
-                    bisect_ends(vrec[i], rois, g, a, b);
-                    bool seen_fg;
-                    und = bisect_undecided(sc, ncam, sil, a, b, seen_fg, reads);
-                    id = i | (seen_fg ? 0x80000000u : 0u);
+                    const Edge e = edge_of_record(vrec[i], rois, g);
+                    bool seen_fg, inside;
+                    uint32_t rd = 0;
+                    und = edge_undecided<Mask>(sc, ncam, sil, e, seen_fg, inside, rd);
+                    reads += rd;
+                    id = i | (inside ? 0x40000000u : 0u) | (seen_fg ? 0x80000000u : 0u);
                 }
                 w.und[j * 32 + lane] = und;
                 w.id[j * 32 + lane] = id;
@@ -701,7 +760,7 @@ __global__ void __launch_bounds__(256) k_bisect(const __grid_constant__ CamSet c
             // that key (worked out twice, so that nothing stays in registers)
             auto place = [&](int j, int& key, int& rank) {
                 const int p = j * 32 + lane;
-                key = w.id[p] == ~0u ? kSortCap : min(__popcll(w.und[p]), kSortCap - 1);
+                key = w.id[p] == ~0u ? kSortCap : min(__popcll((unsigned long long)w.und[p]), kSortCap - 1);
                 const unsigned same = __match_any_sync(kFull, key);
                 rank = __popc(same & ((1u << lane) - 1u));
                 return __popc(same);
@@ -736,15 +795,11 @@ __global__ void __launch_bounds__(256) k_bisect(const __grid_constant__ CamSet c
                 const int p = w.perm[j * 32 + lane];
                 const uint32_t id = w.id[p];
                 if (__all_sync(kFull, id == ~0u)) break;
-                if (id != ~0u) {
-                    const uint32_t i = id & 0x7FFFFFFFu;
-                    float a[3], b[3];
-                    bisect_ends(vrec[i], rois, g, a, b);
-                    bisect_steps(sc, ncam, sil, g.steps, abstain, w.und[p], (id >> 31) != 0u, a, b, tests, reads);
-#pragma unroll
-                    for (int d = 0; d < 3; ++d) a[d] = fmul(fadd(a[d], b[d]), 0.5f);
-                    store_vertex(verts, vcell, i, a, sc, cc, ncam);
-                }
+                const bool have = id != ~0u;
+                const uint32_t i = id & 0x3FFFFFFFu;
+                Edge e{};
+                if (have) e = edge_of_record(vrec[i], rois, g);
+                finish(have, i, e, w.und[p], (id >> 31) != 0u, (id >> 30 & 1u) != 0u);
             }
             __syncwarp();   // the window's shared memory is read before the next one writes it
         }
@@ -942,16 +997,16 @@ cudaError_t launch_mc_prefix(const Grid& g, const Layout& L, const SlotList& sl,
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// Resident blocks per SM of a k_bisect instantiation (index nc: its camera
-// count, 0 for the generic one) with `threads` threads and `smem` bytes of
+// Resident blocks per SM of a k_bisect instantiation (index: 0 for up to 32
+// cameras, else 1) with `threads` threads and `smem` bytes of
 // dynamic shared memory, asked of the runtime once per shape and kept.  The
 // figure is that of the GPU current at the first call; on a host that mixes
 // GPU models it may not fit the others, which changes only how the
 // vertices are grouped into windows, never a result.
 template <class K>
-int bisect_blocks_per_sm(K kernel, int nc, int threads, size_t smem) {
-    static std::atomic<int> known[FVV_MAX_CAMS + 1][9];   // [nc][threads / 32]; 0: not asked yet
-    std::atomic<int>& slot = known[nc][threads / 32];
+int bisect_blocks_per_sm(K kernel, int which, int threads, size_t smem) {
+    static std::atomic<int> known[2][9];   // [which][threads / 32]; 0: not asked yet
+    std::atomic<int>& slot = known[which][threads / 32];
     int n = slot.load(std::memory_order_relaxed);
     if (n == 0) {
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) != cudaSuccess || n < 1) {
@@ -963,6 +1018,19 @@ int bisect_blocks_per_sm(K kernel, int nc, int threads, size_t smem) {
     return n;
 }
 
+template <class Mask>
+cudaError_t launch_bisect_mask(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl, int sms, int th,
+                               int gv, cudaStream_t st) {
+    // the warps that can be resident for each slot: those launched, or the
+    // slot's share of what the GPU holds if that is fewer
+    const size_t smem = (size_t)(th / 32) * sizeof(BisectWarpSmem<Mask>);
+    const int per_sm = bisect_blocks_per_sm(k_bisect<Mask>, sizeof(Mask) == 8, th, smem);
+    const long long launched = (long long)gv * (th / 32);
+    const long long fit = (long long)std::max(per_sm, 1) * sms * (th / 32) / std::max(sl.n, 1);
+    const uint32_t resident = (uint32_t)std::max(1LL, std::min(launched, fit));
+    return launch_pdl(k_bisect<Mask>, dim3(gv, sl.n), dim3(th), smem, st, cams, g, L, sl, resident);
+}
+
 cudaError_t launch_bisect(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl, int sms,
                           const Tuning& tu, cudaStream_t st) {
     const int th = tu.threads[FVV_TUNE_BISECT];
@@ -971,22 +1039,11 @@ cudaError_t launch_bisect(const CamSet& cams, const Grid& g, const Layout& L, co
 #define FVV_LAUNCH(NC) launch_pdl(k_lambda<NC>, dim3(gv, sl.n), dim3(th), 0, st, cams, g, L, sl)
         FVV_DISPATCH_NC(cams.n, FVV_LAUNCH)
 #undef FVV_LAUNCH
-    } else {
-        // the warps that can be resident for each slot: those launched, or the
-        // slot's share of what the GPU holds if that is fewer
-        const size_t smem = (size_t)(th / 32) * sizeof(BisectWarpSmem);
-        int per_sm = 0;
-#define FVV_OCC(NC) per_sm = bisect_blocks_per_sm(k_bisect<NC>, NC, th, smem)
-        FVV_DISPATCH_NC(cams.n, FVV_OCC)
-#undef FVV_OCC
-        const long long launched = (long long)gv * (th / 32);
-        const long long fit = (long long)std::max(per_sm, 1) * sms * (th / 32) / std::max(sl.n, 1);
-        const uint32_t resident = (uint32_t)std::max(1LL, std::min(launched, fit));
-#define FVV_LAUNCH(NC) launch_pdl(k_bisect<NC>, dim3(gv, sl.n), dim3(th), smem, st, cams, g, L, sl, resident)
-        FVV_DISPATCH_NC(cams.n, FVV_LAUNCH)
-#undef FVV_LAUNCH
+        return cudaGetLastError();
     }
-    return cudaGetLastError();
+    const cudaError_t e = cams.n <= 32 ? launch_bisect_mask<uint32_t>(cams, g, L, sl, sms, th, gv, st)
+                                       : launch_bisect_mask<uint64_t>(cams, g, L, sl, sms, th, gv, st);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_mc_triangles(const Grid& g, const Layout& L, const SlotList& sl, const McTable& mc, int sms,
