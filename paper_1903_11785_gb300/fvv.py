@@ -144,19 +144,6 @@ def _stream(stream=None):
     return _vp(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 
 
-def _used_on(stream, *tensors):
-    """Tensors allocated on the current stream that work on `stream` writes:
-    their memory is not handed out again before that work is done."""
-    if stream is None:
-        return
-    handle = int(getattr(stream, "cuda_stream", stream))
-    if handle != torch.cuda.current_stream().cuda_stream:
-        s = stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(handle)
-        for t in tensors:
-            if t is not None:
-                t.record_stream(s)
-
-
 def _ptr_array(ptrs):
     return (_vp * len(ptrs))(*[_vp(int(p)) for p in ptrs])
 
@@ -313,7 +300,6 @@ def fvv_render_view(rig_ptr, slot, rgb, P, centre, width, height, stream=None, w
                                 Pm.ctypes.data_as(C.POINTER(C.c_float)), Cm.ctypes.data_as(C.POINTER(C.c_float)),
                                 width, height, _vp(key.data_ptr()), _vp(out.data_ptr()),
                                 _vp(cam.data_ptr()) if cam is not None else None, _stream(stream)), rig_ptr)
-    _used_on(stream, key, out, cam)
     return key, out, cam
 
 
