@@ -283,7 +283,9 @@ def fvv_render_view(rig_ptr, slot, rgb, P, centre, width, height, stream=None, w
     rgb: per-camera (H,W,3) uint8 tensors (or an (N,H,W,3) tensor), all on
     the device or all in host memory.  Returns device tensors (key (H,W)
     int64 = squared-distance bits << 32 | triangle, -1 where empty; rgb
-    (H,W,3) uint8; capture camera (H,W) int32 or None)."""
+    (H,W,3) uint8; capture camera (H,W) int32 or None).  They are allocated on
+    the current stream: with another `stream`, keep them until it has run, or
+    record it on them (Tensor.record_stream) before they are dropped."""
     imgs = list(rgb) if not torch.is_tensor(rgb) else list(rgb.unbind(0))
     on_dev = None
     for t in imgs:
