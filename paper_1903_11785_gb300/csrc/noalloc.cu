@@ -2,8 +2,9 @@
 // coarse occupancy bitset with the size filter, for callers that cannot
 // allocate device memory.
 //
-// Its scratch (union-find parents, the component list and per-component
-// statistics) lives in one file-scope static __device__ array, so the call
+// Its scratch (union-find parents and the component list; the components' voxel
+// counts are kept in the labels' array until the labels are written) lives in
+// one file-scope static __device__ array, so the call
 // allocates nothing: no cudaMalloc, no cudaFree, no allocating library call.
 // The array is part of the library image, so every GPU that loads the
 // library holds it (kScratchInts ints, about 32.4 MB) until the process exits.
@@ -18,19 +19,16 @@
 // clears what must start at zero; the rest is written before it is read.
 #include <mutex>
 
-#include "fvv_device.cuh"
+#include "ccl_device.cuh"
 
 namespace fvv {
 namespace {
 
 constexpr int kNaMaxVoxels = 8 * 1024 * 1024;       // 8,388,608 coarse voxels
 constexpr int kNaMaxComponents = kMaxComponents;    // 8192 raw components
-// layout, in ints: [0] root count, [1] flags, [64 ..) roots, then per-component
-// statistics (7 each), then labels per component, then parents per voxel
+// layout, in ints: [0] root count, [1] flags, [64 ..) roots, then parents per voxel
 constexpr int kNaRoots = 64;
-constexpr int kNaStats = kNaRoots + kNaMaxComponents;
-constexpr int kNaLabel = kNaStats + 7 * kNaMaxComponents;
-constexpr int kNaParent = (kNaLabel + kNaMaxComponents + 63) / 64 * 64;
+constexpr int kNaParent = (kNaRoots + kNaMaxComponents + 63) / 64 * 64;
 constexpr int kScratchInts = kNaParent + kNaMaxVoxels;
 
 static __device__ __align__(256) int g_na_scratch[kScratchInts];
@@ -41,242 +39,213 @@ struct NaGrid {
     int t_np, t_nb;
 };
 
-constexpr int kNaBudget = 1 << 22;
-
-// Root of x while unions run, shortening the path on the way; its plain
-// stores are safe only in k_na_union (see na_find_readonly).
-__device__ __forceinline__ int na_find(int* parent, int x, int& budget) {
-    int cur = __ldcg(parent + x);
-    if (cur == x || cur < 0) return x;
-    int prev = x;
-    while (budget > 0) {
-        --budget;
-        const int next = __ldcg(parent + cur);
-        if (next == cur || next < 0) return cur;
-        __stcg(parent + prev, next);
-        prev = cur;
-        cur = next;
-    }
-    return cur;
+// Word w of the grid with the bits past nx cleared.
+__device__ __forceinline__ uint32_t na_word(const NaGrid& g, uint32_t w) {
+    const uint32_t word = __ldg(g.bits + w);
+    const bool last = (g.nx & 31) && w % (uint32_t)g.nxw == (uint32_t)g.nxw - 1u;
+    return last ? word & ((1u << (g.nx & 31)) - 1u) : word;
 }
 
-// Root of x after the unions, writing nothing.  In k_na_compress each thread
-// stores only its own voxel's root, so every entry changes at most once, from
-// an ancestor to the root; no other store can overwrite that root afterwards
-// (a shortening store here could, which would leave the voxel pointing at an
-// intermediate node and out of its component's count and box).
-__device__ __forceinline__ int na_find_readonly(const int* parent, int x, int& budget) {
-    int cur = x;
-    while (budget > 0) {
-        --budget;
-        const int next = __ldcg(parent + cur);
-        if (next == cur || next < 0) return cur;
-        cur = next;
-    }
-    return cur;
+// The word at (wx, y, z), 0 outside the grid.
+__device__ __forceinline__ uint32_t na_word_at(const NaGrid& g, int y, int z, int wx) {
+    if (y < 0 || z < 0 || y >= g.ny || z >= g.nz || wx < 0 || wx >= g.nxw) return 0u;
+    const uint32_t word = __ldg(g.bits + ((uint32_t)z * (uint32_t)g.ny + (uint32_t)y) * (uint32_t)g.nxw + (uint32_t)wx);
+    return (g.nx & 31) && wx == g.nxw - 1 ? word & ((1u << (g.nx & 31)) - 1u) : word;
 }
 
-__device__ __forceinline__ void na_unite(int* parent, int a, int b, int& budget) {
-    while (budget > 0) {
-        a = na_find(parent, a, budget);
-        b = na_find(parent, b, budget);
-        if (a == b) return;
-        if (a < b) {
-            const int t = a;
-            a = b;
-            b = t;
+// Calls f(word, row, wx) for the words of the grid that are not empty, one at a
+// time and the same in every lane, so that a lane can take a voxel: a warp
+// reads 32 words, a lane each, interleaved over the warps (lane l of warp k
+// reads word base + l * nwarps + k), so that neighbouring words, which often
+// belong to one object, are worked on by different warps.
+template <class F>
+__device__ __forceinline__ void na_for_words(const NaGrid& g, F&& f) {
+    const uint32_t nwords = (uint32_t)g.nz * (uint32_t)g.ny * (uint32_t)g.nxw;
+    const int lane = threadIdx.x & 31;
+    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5, gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    for (uint32_t base = 0; base < nwords; base += nwarps * 32u) {
+        const uint32_t mw = base + (uint32_t)lane * nwarps + gw;
+        const uint32_t mine = mw < nwords ? na_word(g, mw) : 0u;
+        for (uint32_t pending = __ballot_sync(kFull, mine != 0u); pending; pending &= pending - 1u) {
+            const int src = __ffs(pending) - 1;
+            const uint32_t w = base + (uint32_t)src * nwarps + gw;
+            const uint32_t row = w / (uint32_t)g.nxw;
+            f(__shfl_sync(kFull, mine, src), row, (int)(w - row * (uint32_t)g.nxw));
         }
-        const int old = atomicMin(parent + a, b);
-        if (old == a) return;
-        a = old;
     }
 }
 
-__device__ __forceinline__ bool na_on(const NaGrid& g, int x, int y, int z) {
-    if (x < 0 || y < 0 || z < 0 || x >= g.nx || y >= g.ny || z >= g.nz) return false;
-    return (__ldg(g.bits + ((size_t)z * g.ny + y) * g.nxw + (x >> 5)) >> (x & 31)) & 1u;
+// First voxel (bit) of the run of `word` that voxel `lane` belongs to.
+__device__ __forceinline__ int run_start(uint32_t word, int lane) {
+    const uint32_t starts = word & ~(word << 1);
+    return 31 - __clz(starts & (0xFFFFFFFFu >> (31 - lane)));
 }
 
-// Zero the counters, start a tree at every occupied voxel.
-__global__ void k_na_init(NaGrid g, int* sc) {
+// Zero the counters, start a tree at each run of consecutive occupied voxels of
+// a word, and a count at its first voxel.  `count` (the labels' array, written in
+// full at the end) holds a component's voxels at its root.
+__global__ void __launch_bounds__(256) k_na_seed(NaGrid g, int* sc, int32_t* __restrict__ count) {
+    pdl_begin();
     if (blockIdx.x == 0 && threadIdx.x < 64) sc[threadIdx.x] = 0;
     int* parent = sc + kNaParent;
-    const uint32_t nwords = (uint32_t)g.nz * g.ny * g.nxw;
-    for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < nwords; w += gridDim.x * blockDim.x) {
-        uint32_t word = __ldg(g.bits + w);
-        const uint32_t row = w / (uint32_t)g.nxw;
-        const int wx = (int)(w - row * g.nxw);
-        if (wx == g.nxw - 1 && (g.nx & 31)) word &= (1u << (g.nx & 31)) - 1u;   // ignore bits past nx
-        while (word) {
-            const int b = __ffs(word) - 1;
-            word &= word - 1;
-            const int L = (int)row * g.nx + wx * 32 + b;
-            parent[L] = L;
-        }
-    }
+    const int lane = threadIdx.x & 31;
+    na_for_words(g, [&](uint32_t word, uint32_t row, int wx) {
+        if (!((word >> lane) & 1u)) return;
+        const int first = (int)row * g.nx + wx * 32, run = run_start(word, lane);
+        parent[first + lane] = first + run;
+        if (run == lane) count[first + lane] = 0;
+    });
 }
 
-__global__ void k_na_union(NaGrid g, int* sc) {
+// The unions of k_union (kernels_ccl.cu, where the rule is): runs across a word
+// boundary, and with the four rows before that touch the row; a lane per voxel.
+// A thread that walked 32 voxels through 13 neighbours each, one union after
+// the other, took 318 us on a court-sized grid (400 x 220 x 80, 12 players and
+// 2,000 stray voxels), this takes 24; the call 496 -> 63 us, and 10.1 ms -> 0.7
+// on that grid with a quarter of its voxels occupied at random.
+__global__ void __launch_bounds__(256) k_na_union(NaGrid g, int* sc) {
+    pdl_begin();
     int* parent = sc + kNaParent;
-    const uint32_t nwords = (uint32_t)g.nz * g.ny * g.nxw;
-    int budget = kNaBudget;
-    for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < nwords && budget > 0; w += gridDim.x * blockDim.x) {
-        uint32_t word = __ldg(g.bits + w);
-        const uint32_t row = w / (uint32_t)g.nxw;
-        const int wx = (int)(w - row * g.nxw);
-        if (wx == g.nxw - 1 && (g.nx & 31)) word &= (1u << (g.nx & 31)) - 1u;
+    const int lane = threadIdx.x & 31;
+    int budget = kStepBudget;
+    na_for_words(g, [&](uint32_t word, uint32_t row, int wx) {
+        if (!((word >> lane) & 1u) || budget <= 0) return;
         const int y = (int)(row % (uint32_t)g.ny), z = (int)(row / (uint32_t)g.ny);
-        while (word) {
-            const int b = __ffs(word) - 1;
-            word &= word - 1;
-            const int x = wx * 32 + b;
-            const int L = (int)row * g.nx + x;
-            for (int dz = -1; dz <= 0; ++dz)
-                for (int dy = -1; dy <= 1; ++dy)
-                    for (int dx = -1; dx <= 1; ++dx) {
-                        if (dz == 0 && (dy > 0 || (dy == 0 && dx >= 0))) continue;
-                        if (!na_on(g, x + dx, y + dy, z + dz)) continue;
-                        na_unite(parent, L, ((z + dz) * g.ny + (y + dy)) * g.nx + (x + dx), budget);
-                    }
+        const int run = run_start(word, lane), run0 = (int)row * g.nx + wx * 32 + run;
+        if (lane == 0 && (na_word_at(g, y, z, wx - 1) >> 31)) unite(parent, run0, run0 - 1, budget);
+        for (int k = 0; k < 4; ++k) {
+            const int dy = k == 0 ? -1 : k - 2, dz = k == 0 ? 0 : -1;
+            const uint32_t n = na_word_at(g, y + dy, z + dz, wx);
+            const bool left = lane > 0 ? (n >> (lane - 1)) & 1u : na_word_at(g, y + dy, z + dz, wx - 1) >> 31;
+            const bool mid = (n >> lane) & 1u;
+            const bool right = lane < 31 ? (n >> (lane + 1)) & 1u : na_word_at(g, y + dy, z + dz, wx + 1) & 1u;
+            const int nrow = ((z + dz) * g.ny + (y + dy)) * g.nx + wx * 32;
+            if (run == lane && (left || mid)) unite(parent, run0, nrow + (left ? lane - 1 : lane), budget);
+            if (!mid && right) unite(parent, run0, nrow + lane + 1, budget);
         }
-    }
+    });
     if (budget <= 0) atomicOr(sc + 1, (int)FVV_FLAG_LOOP);
 }
 
-__global__ void k_na_compress(NaGrid g, int* sc) {
+// Point every voxel at its root, list the roots and count each component's
+// voxels.  A warp keeps the count of the component it met last, so that a
+// large one costs it one atomic and not one a word.
+__global__ void __launch_bounds__(256) k_na_compress(NaGrid g, int* sc, int32_t* __restrict__ count) {
+    pdl_begin();
     int* parent = sc + kNaParent;
-    const uint32_t nwords = (uint32_t)g.nz * g.ny * g.nxw;
-    int budget = kNaBudget;
-    for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < nwords && budget > 0; w += gridDim.x * blockDim.x) {
-        uint32_t word = __ldg(g.bits + w);
-        const uint32_t row = w / (uint32_t)g.nxw;
-        const int wx = (int)(w - row * g.nxw);
-        if (wx == g.nxw - 1 && (g.nx & 31)) word &= (1u << (g.nx & 31)) - 1u;
-        while (word) {
-            const int b = __ffs(word) - 1;
-            word &= word - 1;
-            const int L = (int)row * g.nx + wx * 32 + b;
-            const int r = na_find_readonly(parent, L, budget);
-            if (r == L) {
-                const int k = atomicAdd(sc, 1);
-                if (k < kNaMaxComponents) sc[kNaRoots + k] = L;
-            } else {
-                parent[L] = r;
-            }
+    const int lane = threadIdx.x & 31;
+    int budget = kStepBudget, cur = -1, held = 0;   // cur, held: the same in every lane
+    na_for_words(g, [&](uint32_t word, uint32_t row, int wx) {
+        const int L = (int)row * g.nx + wx * 32 + lane;
+        int r = -1;
+        if (((word >> lane) & 1u) && budget > 0) {
+            r = find_root_readonly(parent, L, budget);
+            if (r != L) parent[L] = r;
         }
-    }
+        const uint32_t roots = __ballot_sync(kFull, r == L);
+        if (roots) {
+            int at = 0;
+            if (lane == 0) at = atomicAdd(sc, __popc(roots));
+            at = __shfl_sync(kFull, at, 0) + __popc(roots & ((1u << lane) - 1u));
+            if (r == L && at < kNaMaxComponents) sc[kNaRoots + at] = L;
+        }
+        const uint32_t any = __ballot_sync(kFull, r >= 0);
+        if (!any) return;
+        const int lead = __shfl_sync(kFull, r, __ffs(any) - 1);
+        const int n = __popc(__ballot_sync(kFull, r == lead));
+        if (lead != cur) {
+            if (lane == 0 && cur >= 0) atomicAdd(count + cur, held);
+            cur = lead;
+            held = 0;
+        }
+        held += n;
+        const uint32_t same = __match_any_sync(kFull, r);
+        if (r >= 0 && r != lead && lane == __ffs(same) - 1) atomicAdd(count + r, __popc(same));
+    });
+    if (lane == 0 && cur >= 0) atomicAdd(count + cur, held);
     if (budget <= 0) atomicOr(sc + 1, (int)FVV_FLAG_LOOP);
 }
 
-// One block: sort the roots, tag each root's parent entry with -(i+1), reset
-// the statistics.
-__global__ void __launch_bounds__(1024) k_na_sort(int* sc) {
-    __shared__ int key[kNaMaxComponents];
-    const int n = sc[0];
-    if (n > kNaMaxComponents) return;
-    int* parent = sc + kNaParent;
-    int m = 1;
-    while (m < n) m <<= 1;
-    for (int i = threadIdx.x; i < m; i += blockDim.x) key[i] = i < n ? sc[kNaRoots + i] : 0x7FFFFFFF;
-    __syncthreads();
-    for (int k = 2; k <= m; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < m; i += blockDim.x) {
-                const int p = i ^ j;
-                if (p > i) {
-                    const bool up = (i & k) == 0;
-                    const int a = key[i], b = key[p];
-                    if ((a > b) == up) {
-                        key[i] = b;
-                        key[p] = a;
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        parent[key[i]] = -(i + 1);
-        int* s = sc + kNaStats + 7 * i;
-        s[0] = 0;
-        s[1] = s[2] = s[3] = 0x7FFFFFFF;
-        s[4] = s[5] = s[6] = -1;
-    }
-}
-
-// Component index of occupied voxel L after tagging, or -1.
-__device__ __forceinline__ int na_comp(const int* parent, int L) {
-    const int r = parent[L];
-    const int t = r < 0 ? r : parent[r];
-    return t < 0 ? -t - 1 : -1;
-}
-
-__global__ void k_na_stats(NaGrid g, int* sc) {
-    if (sc[0] > kNaMaxComponents) return;
-    const int* parent = sc + kNaParent;
-    const uint32_t nwords = (uint32_t)g.nz * g.ny * g.nxw;
-    for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < nwords; w += gridDim.x * blockDim.x) {
-        uint32_t word = __ldg(g.bits + w);
-        const uint32_t row = w / (uint32_t)g.nxw;
-        const int wx = (int)(w - row * g.nxw);
-        if (wx == g.nxw - 1 && (g.nx & 31)) word &= (1u << (g.nx & 31)) - 1u;
-        const int y = (int)(row % (uint32_t)g.ny), z = (int)(row / (uint32_t)g.ny);
-        while (word) {
-            const int b = __ffs(word) - 1;
-            word &= word - 1;
-            const int x = wx * 32 + b;
-            const int c = na_comp(parent, (int)row * g.nx + x);
-            if (c < 0) continue;
-            int* s = sc + kNaStats + 7 * c;
-            atomicAdd(s, 1);
-            atomicMin(s + 1, x); atomicMin(s + 2, y); atomicMin(s + 3, z);
-            atomicMax(s + 4, x); atomicMax(s + 5, y); atomicMax(s + 6, z);
-        }
-    }
-}
-
-// One block: keep iff t_np <= count <= t_nb, labels 1..K in component order.
-__global__ void __launch_bounds__(1024) k_na_filter(NaGrid g, int* sc, int32_t* counts) {
-    __shared__ uint32_t sh[33];
+// Canonical labels: a kept component (t_np <= voxels <= t_nb) has label 1 + the
+// number of kept ones with a smaller root, which is left in its root's parent
+// entry as -(label + 1), a removed one's as -1.  Four lanes count for a root, a
+// quarter of all kept roots each (8192 at most), 64 roots a block; a block that
+// has none leaves.  (A bitonic sort in one block took 40 us for 2,200 roots.)
+constexpr int kNaRankRoots = 64;
+__global__ void __launch_bounds__(256) k_na_rank(NaGrid g, int* sc, const int32_t* __restrict__ count,
+                                                 int32_t* __restrict__ counts) {
+    pdl_begin();
+    __shared__ __align__(16) int key[2048];
+    __shared__ int sh[32];
     const int n = sc[0];
     const bool over = n > kNaMaxComponents;
-    uint32_t base = 0;
-    for (int t0 = 0; t0 < (over ? 0 : n); t0 += blockDim.x) {
-        const int i = t0 + threadIdx.x;
-        uint32_t keep = 0;
-        if (i < n) {
-            const int c = sc[kNaStats + 7 * i];
-            keep = (c >= g.t_np && c <= g.t_nb) ? 1u : 0u;
-        }
-        uint32_t tot;
-        const uint32_t ex = block_exclusive_scan(keep, sh, tot);
-        if (i < n) sc[kNaLabel + i] = keep ? (int)(base + ex + 1) : 0;
-        base += tot;
+    if (blockIdx.x > 0 && (over || (int)blockIdx.x * kNaRankRoots >= n)) return;   // the whole block
+    int* parent = sc + kNaParent;
+    const int i = blockIdx.x * kNaRankRoots + threadIdx.x / 4;
+    const int root = !over && i < n ? sc[kNaRoots + i] : -1;
+    int before = 0, kept = 0;
+    bool keep = false;
+    if (root >= 0) {
+        const int c = __ldcg(count + root);
+        keep = c >= g.t_np && c <= g.t_nb;
     }
-    if (threadIdx.x == 0) {
+    for (int t0 = 0; t0 < (over ? 0 : n); t0 += 2048) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int k = (int)threadIdx.x + 256 * q;
+            int v = 0x7FFFFFFF;                     // past the end, or removed: before nobody
+            if (t0 + k < n) {
+                const int r = sc[kNaRoots + t0 + k], c = __ldcg(count + r);
+                if (c >= g.t_np && c <= g.t_nb) v = r;
+            }
+            key[k] = v;
+            kept += v != 0x7FFFFFFF;
+        }
+        __syncthreads();
+        const int m = min(2048, (n - t0 + 15) & ~15);
+        for (int k = 4 * (threadIdx.x & 3); k < m; k += 16) {
+            const int4 v = *reinterpret_cast<const int4*>(key + k);
+            before += (v.x < root) + (v.y < root) + (v.z < root) + (v.w < root);
+        }
+        __syncthreads();
+    }
+    before += __shfl_xor_sync(kFull, before, 1);
+    before += __shfl_xor_sync(kFull, before, 2);
+    if (root >= 0 && (threadIdx.x & 3) == 0) parent[root] = keep ? -(before + 2) : -1;
+    const int total = block_sum<int>(kept, sh);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
         counts[0] = n;
-        counts[1] = over ? 0 : (int)base;
+        counts[1] = total;
         counts[2] = sc[1] | (over ? (int)FVV_FLAG_ROOTS : 0);
     }
 }
 
-// Every voxel of the output: its canonical label, 0 for empty or removed.
-__global__ void k_na_labels(NaGrid g, const int* sc, int32_t* labels) {
-    const bool ok = sc[0] <= kNaMaxComponents;
+// Every voxel of the output: its canonical label, 0 for empty or removed.  A
+// warp takes 32 words, a lane per voxel of each, so that a word's labels go out
+// in one piece.
+__global__ void __launch_bounds__(256) k_na_labels(NaGrid g, const int* sc, int32_t* __restrict__ labels) {
+    pdl_begin();
     const int* parent = sc + kNaParent;
-    const uint32_t nwords = (uint32_t)g.nz * g.ny * g.nxw;
-    for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < nwords; w += gridDim.x * blockDim.x) {
-        const uint32_t word = __ldg(g.bits + w);
-        const uint32_t row = w / (uint32_t)g.nxw;
-        const int wx = (int)(w - row * g.nxw);
-        const int nb = min(32, g.nx - wx * 32);
-        for (int b = 0; b < nb; ++b) {
-            const int L = (int)row * g.nx + wx * 32 + b;
+    const uint32_t nwords = (uint32_t)g.nz * (uint32_t)g.ny * (uint32_t)g.nxw;
+    const int lane = threadIdx.x & 31;
+    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+    for (uint32_t base = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32u; base < nwords; base += nwarps * 32u) {
+        const uint32_t mw = base + (uint32_t)lane;
+        const uint32_t mine = mw < nwords ? na_word(g, mw) : 0u;
+        const uint32_t row = min(mw, nwords - 1u) / (uint32_t)g.nxw;
+        const int x0 = (int)(min(mw, nwords - 1u) - row * (uint32_t)g.nxw) * 32;
+        const int first = (int)row * g.nx + x0, nv = min(32, g.nx - x0);
+        const int m = (int)min(32u, nwords - base);
+#pragma unroll 4
+        for (int k = 0; k < m; ++k) {
+            const uint32_t word = __shfl_sync(kFull, mine, k);
+            const int L = __shfl_sync(kFull, first, k) + lane;
             int lab = 0;
-            if (ok && ((word >> b) & 1u)) {
-                const int c = na_comp(parent, L);
-                lab = c >= 0 ? sc[kNaLabel + c] : 0;
+            if ((word >> lane) & 1u) {
+                const int r = __ldg(parent + L), t = r < 0 ? r : __ldg(parent + r);
+                lab = t < 0 ? -t - 1 : 0;           // else: roots were not tagged (too many components)
             }
-            labels[L] = lab;
+            if (lane < __shfl_sync(kFull, nv, k)) __stcs(labels + L, lab);
         }
     }
 }
@@ -309,13 +278,23 @@ extern "C" fvv_status fvv_label_components_noalloc(const uint32_t* coarse_bits, 
     const cudaStream_t st = static_cast<cudaStream_t>(stream);
     NaGrid g{coarse_bits, nx, ny, nz, (nx + 31) / 32, t_np, t_nb};
     const long long words = (long long)nz * ny * g.nxw;
-    const unsigned blocks = (unsigned)std::max(1LL, std::min((words + 255) / 256, 4096LL));
-    k_na_init<<<blocks, 256, 0, st>>>(g, sc);
-    k_na_union<<<blocks, 256, 0, st>>>(g, sc);
-    k_na_compress<<<blocks, 256, 0, st>>>(g, sc);
-    k_na_sort<<<1, 1024, 0, st>>>(sc);
-    k_na_stats<<<blocks, 256, 0, st>>>(g, sc);
-    k_na_filter<<<1, 1024, 0, st>>>(g, sc, counts);
-    k_na_labels<<<blocks, 256, 0, st>>>(g, sc, labels);
+    // four words a warp, so that a small grid's objects are spread over many, up to 2048 blocks
+    const unsigned blocks = (unsigned)std::max(1LL, std::min((words + 31) / 32, 2048LL));
+    // Dependent launch hides the gaps between a small grid's kernels (60 x 60 x 30
+    // voxels: 67 -> 57 us); a large one's run slower with it (400 x 220 x 80: 63
+    // -> 71 us, the next kernel's waiting blocks take room on the SMs).
+    if (blocks < 2048) {
+        launch_pdl(k_na_seed, dim3(blocks), dim3(256), 0, st, g, sc, labels);
+        launch_pdl(k_na_union, dim3(blocks), dim3(256), 0, st, g, sc);
+        launch_pdl(k_na_compress, dim3(blocks), dim3(256), 0, st, g, sc, labels);
+        launch_pdl(k_na_rank, dim3(kNaMaxComponents / kNaRankRoots), dim3(256), 0, st, g, sc, labels, counts);
+        launch_pdl(k_na_labels, dim3(blocks), dim3(256), 0, st, g, sc, labels);
+    } else {
+        k_na_seed<<<blocks, 256, 0, st>>>(g, sc, labels);
+        k_na_union<<<blocks, 256, 0, st>>>(g, sc);
+        k_na_compress<<<blocks, 256, 0, st>>>(g, sc, labels);
+        k_na_rank<<<kNaMaxComponents / kNaRankRoots, 256, 0, st>>>(g, sc, labels, counts);
+        k_na_labels<<<blocks, 256, 0, st>>>(g, sc, labels);
+    }
     return cudaGetLastError() == cudaSuccess ? FVV_OK : FVV_ERR_CUDA;
 }
