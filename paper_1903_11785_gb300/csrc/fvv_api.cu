@@ -41,6 +41,7 @@ struct fvv_rig {
     std::vector<Graph> graph_cache;
     unsigned long long graph_clock = 0;
     SlotInfo* host_info = nullptr;   // page-locked, FVV_MAX_BATCH entries: counts read by fvv_get_results_batch
+    SlotInfo* host_info_dev = nullptr;   // its device address
 };
 
 namespace {
@@ -430,7 +431,8 @@ fvv_status fvv_create_rig(const fvv_rig_desc* desc, const fvv_recon_params* para
     if (e == cudaSuccess) e = launch_init_depth(rig->cams, rig->L, rig->max_slots, rig->sms, nullptr);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e == cudaSuccess) e = cudaHostAlloc(reinterpret_cast<void**>(&rig->host_info), FVV_MAX_BATCH * sizeof(SlotInfo),
-                                            cudaHostAllocDefault);
+                                            cudaHostAllocMapped);
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&rig->host_info_dev), rig->host_info, 0);
     if (e != cudaSuccess) {
         if (rig->own_arena) cudaFree(rig->arena);
         if (rig->host_info) cudaFreeHost(rig->host_info);
@@ -909,8 +911,17 @@ static bool fill_counts(const SlotInfo& info, fvv_counts* out) {
     out->tests_bisect = (long long)info.tests_bisect;
     out->lookups_fine = (long long)info.look_fine;
     out->lookups_bisect = (long long)info.look_bisect;
-    const unsigned cap = FVV_FLAG_ROOTS | FVV_FLAG_ROIS | FVV_FLAG_FINE | FVV_FLAG_VERTS | FVV_FLAG_TRIS | FVV_FLAG_LOOP;
-    return (info.flags & cap) != 0u;
+    return (info.flags & kOverCapacity) != 0u;
+}
+
+// Whether p is memory of `device` (its kernels can write it without more ado).
+static bool on_device(const void* p, int device) {
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == device;
 }
 
 // Enqueue the copies of a slot's vertices, triangles, colours and cameras
@@ -958,13 +969,38 @@ fvv_status fvv_get_results_batch(fvv_rig* rig, const int* slots, int n_slots, fv
     }
     const cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaSuccess;
+    // buffers on the rig's own device: one launch copies the results and the
+    // counts; then the one wait of the call
+    bool gather = dst_on_device != 0;
+    for (int i = 0; i < n_slots && gather; ++i)
+        for (const void* p : {(const void*)dst[i].verts, (const void*)dst[i].tris, (const void*)dst[i].rgb,
+                              (const void*)dst[i].cam})
+            gather = gather && (!p || on_device(p, rig->device));
+    if (gather) {
+        thread_local GatherSlots gs;   // 9 KB: kept off the stack
+        gs.n = n_slots;
+        for (int i = 0; i < n_slots; ++i) {
+            gs.slot[i] = slots[i];
+            gs.dst[i][0] = reinterpret_cast<char*>(dst[i].verts);
+            gs.dst[i][1] = reinterpret_cast<char*>(dst[i].tris);
+            gs.dst[i][2] = reinterpret_cast<char*>(dst[i].rgb);
+            gs.dst[i][3] = reinterpret_cast<char*>(dst[i].cam);
+        }
+        e = launch_gather_results(rig->L, gs, rig->host_info_dev, rig->sms, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return cuda_fail(rig, e, "fvv_get_results_batch");
+        bool over = false;
+        for (int i = 0; i < n_slots; ++i) over |= fill_counts(rig->host_info[i], &dst[i].counts);
+        if (over) return fail(rig, FVV_ERR_CAPACITY, "a capacity was exceeded in some slot (see its flags)");
+        return FVV_OK;
+    }
+    const cudaMemcpyKind kind = dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     for (int i = 0; i < n_slots && e == cudaSuccess; ++i)
         e = cudaMemcpyAsync(rig->host_info + i, slot_ptr<SlotInfo>(rig->L, slots[i], rig->L.info), sizeof(SlotInfo),
                             cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // the one wait of the call
     if (e != cudaSuccess) return cuda_fail(rig, e, "fvv_get_results_batch");
     bool over = false;
-    const cudaMemcpyKind kind = dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     for (int i = 0; i < n_slots && e == cudaSuccess; ++i) {
         fvv_results_dst& d = dst[i];
         if (fill_counts(rig->host_info[i], &d.counts)) {

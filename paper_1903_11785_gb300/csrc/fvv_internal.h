@@ -136,6 +136,10 @@ struct Layout {
     size_t rgb_stage;           // uint8 x3 per pixel (host uploads), or 0
 };
 
+// FVV_FLAG_* bits that say that a slot has no results.
+constexpr unsigned kOverCapacity =
+    FVV_FLAG_ROOTS | FVV_FLAG_ROIS | FVV_FLAG_FINE | FVV_FLAG_VERTS | FVV_FLAG_TRIS | FVV_FLAG_LOOP;
+
 template <typename T>
 __host__ __device__ inline T* slot_ptr(const Layout& L, int slot, size_t off) {
     return reinterpret_cast<T*>(L.base + (size_t)slot * L.stride + off);
@@ -258,6 +262,17 @@ struct ColourBatch {
 
 cudaError_t launch_colour(const CamSet& cams, const Grid& g, const Layout& L, const ColourBatch& cb, int sms,
                           int total_slots, cudaStream_t st);
+
+// Where the results of a call's slots go (device memory; any may be NULL).
+struct GatherSlots {
+    int n;
+    int slot[FVV_MAX_BATCH];
+    char* dst[FVV_MAX_BATCH][4];        // vertices, triangles, colours, cameras
+};
+
+// Copies every slot's results to their destinations and its SlotInfo to infos[i]
+// (page-locked host memory, device address); slots over a capacity only the latter.
+cudaError_t launch_gather_results(const Layout& L, const GatherSlots& gs, SlotInfo* infos, int sms, cudaStream_t st);
 
 // A novel view (step E) of one reconstructed slot: the virtual camera as a
 // Cam (P, C, W, H, Wf, Hf; the other fields unused) and the capture RGB.

@@ -411,6 +411,63 @@ __global__ void __launch_bounds__(256) k_colour(const __grid_constant__ CamSet c
     }
 }
 
+// ---- results
+
+// Copies n bytes, 16, 4 or 1 at a time as the destination's alignment allows
+// (the sources are 256-byte aligned), by all threads of the `blocks` blocks.
+__device__ __forceinline__ void copy_bytes(char* __restrict__ dst, const char* __restrict__ src, size_t n,
+                                           unsigned block, unsigned blocks) {
+    const size_t i0 = (size_t)block * blockDim.x + threadIdx.x, step = (size_t)blocks * blockDim.x;
+    const uintptr_t a = reinterpret_cast<uintptr_t>(dst);
+    size_t done = 0;
+    if ((a & 15u) == 0) {
+        const size_t m = n >> 4;
+        const uint4* s = reinterpret_cast<const uint4*>(src);
+        uint4* d = reinterpret_cast<uint4*>(dst);
+        size_t i = i0;
+        for (; i + 3 * step < m; i += 4 * step) {     // four loads in flight
+            const uint4 v0 = __ldcs(s + i), v1 = __ldcs(s + i + step), v2 = __ldcs(s + i + 2 * step),
+                        v3 = __ldcs(s + i + 3 * step);
+            __stcs(d + i, v0);
+            __stcs(d + i + step, v1);
+            __stcs(d + i + 2 * step, v2);
+            __stcs(d + i + 3 * step, v3);
+        }
+        for (; i < m; i += step) __stcs(d + i, __ldcs(s + i));
+        done = m << 4;
+    } else if ((a & 3u) == 0) {
+        const size_t m = n >> 2;
+        for (size_t i = i0; i < m; i += step)
+            __stcs(reinterpret_cast<uint32_t*>(dst) + i, __ldcs(reinterpret_cast<const uint32_t*>(src) + i));
+        done = m << 2;
+    }
+    for (size_t i = done + i0; i < n; i += step) dst[i] = src[i];
+}
+
+// The results of several slots in one launch, as long as the device's own
+// counts say, so that nobody waits for them first; the counts go to the host with
+// them.  Grid (blocks, slots).  Bound by HBM: 64 court frames (1.1 GB read and
+// written) FIGURES, with 64 + 256 copies and a wait between them before.
+__global__ void __launch_bounds__(256) k_gather_results(const __grid_constant__ Layout L,
+                                                        const __grid_constant__ GatherSlots gs, SlotInfo* infos) {
+    pdl_begin();
+    const int slot = gs.slot[blockIdx.y];
+    const SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
+    if (blockIdx.x == 0 && threadIdx.x < sizeof(SlotInfo) / 4)
+        reinterpret_cast<uint32_t*>(infos + blockIdx.y)[threadIdx.x] = reinterpret_cast<const uint32_t*>(info)[threadIdx.x];
+    if (info->n_words == 0u || (info->flags & kOverCapacity)) return;
+    const size_t nv = info->n_verts, nt = info->n_tris;
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+        char* dst = gs.dst[blockIdx.y][k];
+        const size_t off = k == 0 ? L.verts : k == 1 ? L.tris : k == 2 ? L.vrgb : L.vcam;
+        const size_t n = k == 0 ? 12 * nv : k == 1 ? 12 * nt : k == 2 ? 3 * nv : 4 * nv;
+        if (dst) copy_bytes(dst, slot_ptr<char>(L, slot, off), n, blockIdx.x, gridDim.x);
+    }
+}
+static_assert(sizeof(SlotInfo) % 4 == 0 && sizeof(SlotInfo) / 4 <= 256, "SlotInfo copy");
+static_assert(sizeof(GatherSlots) + sizeof(Layout) <= 32000, "k_gather_results parameters");
+
 // ---- Sec. II-E, step E: a novel view of the coloured mesh
 
 __global__ void __launch_bounds__(256) k_view_clear(unsigned long long* __restrict__ key, size_t npix) {
@@ -517,6 +574,12 @@ cudaError_t launch_colour(const CamSet& cams, const Grid& g, const Layout& L, co
     const int gv = grid_x(sms, total_slots, g.max_verts, 256);
     launch_pdl(k_colour, dim3(gv, cb.n), dim3(256), 0, st, cams, g, L, cb);
     return cudaGetLastError();
+}
+
+cudaError_t launch_gather_results(const Layout& L, const GatherSlots& gs, SlotInfo* infos, int sms, cudaStream_t st) {
+    const int gx = std::max(1, sms * 8 / std::max(1, gs.n));
+    const cudaError_t e = launch_pdl(k_gather_results, dim3(gx, gs.n), dim3(256), 0, st, L, gs, infos);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_render_view(const CamSet& cams, const Grid& g, const Layout& L, const ViewArgs& va,
