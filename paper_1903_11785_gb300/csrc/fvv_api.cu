@@ -769,13 +769,17 @@ fvv_status fvv_colour(fvv_rig* rig, const int* slots, int n_slots, const uint8_t
     const int N = rig->cams.n;
     for (size_t i = 0; i < (size_t)n_slots * N; ++i)
         if (!rgb[i]) return fail(rig, FVV_ERR_INVALID_ARG, "an rgb pointer is NULL");
-    if (rgb_on_device == FVV_MAPPED_HOST)
+    std::vector<const uint8_t*> mapped;   // device addresses of images read in place
+    if (rgb_on_device == FVV_MAPPED_HOST) {
+        mapped.reserve((size_t)n_slots * N);
         for (int i = 0; i < n_slots; ++i)
             for (int n = 0; n < N; ++n) {
                 const Cam& c = rig->cams.c[n];
-                if (!mapped_host(rgb[(size_t)i * N + n], (size_t)3 * c.W * c.H))
-                    return fail(rig, FVV_ERR_INVALID_ARG, "an rgb image is not in mapped page-locked host memory");
+                const uint8_t* d = mapped_host(rgb[(size_t)i * N + n], (size_t)3 * c.W * c.H);
+                if (!d) return fail(rig, FVV_ERR_INVALID_ARG, "an rgb image is not in mapped page-locked host memory");
+                mapped.push_back(d);
             }
+    }
     cudaError_t e = cudaSuccess;
     const int t = stage_begin(rig, FVV_STAGE_COLOUR, st);
     // slots go to the kernel in groups of kColourBatch, with their RGB sources
@@ -792,8 +796,7 @@ fvv_status fvv_colour(fvv_rig* rig, const int* slots, int n_slots, const uint8_t
                 if (rgb_on_device == 1) {
                     cb.rgb[j][n] = src;
                 } else if (rgb_on_device == FVV_MAPPED_HOST) {
-                    const Cam& c = rig->cams.c[n];
-                    cb.rgb[j][n] = mapped_host(src, (size_t)3 * c.W * c.H);   // checked above
+                    cb.rgb[j][n] = mapped[(size_t)i * N + n];
                 } else {
                     const Cam& c = rig->cams.c[n];
                     uint8_t* dst = slot_ptr<uint8_t>(rig->L, sl.s[i], rig->L.rgb_stage) + 3 * c.pix_off;

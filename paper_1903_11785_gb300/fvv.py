@@ -13,6 +13,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 
 import numpy as np
 import torch
@@ -80,7 +81,17 @@ class Counts(C.Structure):
                 ("tests_bisect", C.c_longlong), ("lookups_fine", C.c_longlong), ("lookups_bisect", C.c_longlong)]
 
     def as_dict(self):
-        return {k: getattr(self, k) for k, _ in self._fields_ if k != "pad_"}
+        return dict(zip(_COUNT_NAMES, _COUNT_STRUCT.unpack_from(self)))
+
+
+# the fields of Counts but its padding, read in one go (field by field a
+# group of 64 slots took 160 us)
+_COUNT_STRUCT = struct.Struct("@Iii4x9q")
+_COUNT_NAMES = tuple(k for k, _ in Counts._fields_ if k != "pad_")
+assert _COUNT_STRUCT.size == C.sizeof(Counts)
+
+
+_RESULTS = ("verts", "tris", "rgb", "cam")
 
 
 class ResultsDst(C.Structure):
@@ -145,7 +156,56 @@ def _stream(stream=None):
 
 
 def _ptr_array(ptrs):
-    return (_vp * len(ptrs))(*[_vp(int(p)) for p in ptrs])
+    return (_vp * len(ptrs))(*ptrs)
+
+
+def _int_array(ints):
+    return (C.c_int * len(ints))(*ints)
+
+
+def _images(groups):
+    """The images of several slots (per slot a list of tensors or a stacked
+    one): their addresses, whether they are on the GPU, and the tensors.  One
+    pass with few Python operations an image: a call on a frame of 16 cameras
+    is otherwise mostly spent here."""
+    ptrs, tensors = [], []
+    for g in groups:
+        if isinstance(g, torch.Tensor):
+            n = g.shape[0]
+            assert g.dtype is torch.uint8
+            if n and g.is_contiguous():              # one check for the whole stack
+                p, step = g.data_ptr(), g.stride(0) if n > 1 else 0
+                ptrs.extend([p + k * step for k in range(n)])
+                tensors.append(g)
+                continue
+            g = g.unbind(0)
+        elif not isinstance(g, (list, tuple)):
+            g = list(g)
+        for t in g:
+            assert t.dtype is torch.uint8 and t.is_contiguous()
+            ptrs.append(t.data_ptr())
+        tensors.extend(g)
+    assert tensors
+    on_dev = tensors[0].is_cuda
+    for t in tensors:
+        assert t.is_cuda is on_dev
+    return ptrs, int(on_dev), tensors
+
+
+def _floats(values, n):
+    """n floats in host memory as a C array, from anything numpy reads."""
+    a = np.ascontiguousarray(values, np.float32)
+    if a.size != n:
+        raise ValueError(f"expected {n} numbers, got {a.size}")
+    return (C.c_float * n).from_buffer_copy(a)
+
+
+def _check_images(status, rig_ptr, mode, tensors):
+    """_check after a call that took images; the library looks at every address
+    that it is to read in place, so pinning is looked into only when it refuses."""
+    if status == FVV_ERR_INVALID_ARG and mode == FVV_MAPPED_HOST:
+        assert all(t.is_pinned() for t in tensors), "reading in place needs pinned host tensors"
+    _check(status, rig_ptr)
 
 
 # ------------------------------------------------------------ C-named calls
@@ -219,30 +279,19 @@ def fvv_upload_silhouettes(rig_ptr, slot, masks, stream=None, in_place=False):
     """masks: list of per-camera uint8 tensors (H,W) (or one (N,H,W) tensor),
     all on the GPU or all in host memory; in_place: pinned host tensors are
     read in place by the packing kernel (FVV_MAPPED_HOST)."""
-    ms = list(masks) if not torch.is_tensor(masks) else list(masks.unbind(0))
-    on_dev = _rgb_mode(int(ms[0].is_cuda), ms, in_place)
-    for m in ms:
-        assert m.dtype == torch.uint8 and m.is_contiguous() and m.is_cuda == ms[0].is_cuda
-    _check(_lib.fvv_upload_silhouettes(rig_ptr, slot, _ptr_array([m.data_ptr() for m in ms]), on_dev,
-                                       _stream(stream)), rig_ptr)
+    ptrs, on_dev, ms = _images([masks])
+    mode = _rgb_mode(on_dev, in_place)
+    _check_images(_lib.fvv_upload_silhouettes(rig_ptr, slot, _ptr_array(ptrs), mode, _stream(stream)), rig_ptr, mode, ms)
 
 
 def fvv_upload_silhouettes_batch(rig_ptr, slots, masks, stream=None, in_place=False):
     """masks: per slot, a list of per-camera uint8 tensors (H,W) (or one
     (N,H,W) tensor, or an (F,N,H,W) tensor for all slots); memory kinds as
     for fvv_upload_silhouettes."""
-    ptrs, ms = [], []
-    for per_slot in masks:
-        imgs = list(per_slot) if not torch.is_tensor(per_slot) else list(per_slot.unbind(0))
-        for m in imgs:
-            assert m.dtype == torch.uint8 and m.is_contiguous()
-            ptrs.append(m.data_ptr())
-            ms.append(m)
-    assert ms and all(m.is_cuda == ms[0].is_cuda for m in ms)
-    on_dev = _rgb_mode(int(ms[0].is_cuda), ms, in_place)
-    arr = (C.c_int * len(slots))(*slots)
-    _check(_lib.fvv_upload_silhouettes_batch(rig_ptr, arr, len(slots), _ptr_array(ptrs), on_dev,
-                                             _stream(stream)), rig_ptr)
+    ptrs, on_dev, ms = _images(masks)
+    mode = _rgb_mode(on_dev, in_place)
+    _check_images(_lib.fvv_upload_silhouettes_batch(rig_ptr, _int_array(slots), len(slots), _ptr_array(ptrs), mode,
+                                                    _stream(stream)), rig_ptr, mode, ms)
 
 
 def fvv_reconstruct(rig_ptr, slots, stream=None):
@@ -250,11 +299,8 @@ def fvv_reconstruct(rig_ptr, slots, stream=None):
     _check(_lib.fvv_reconstruct(rig_ptr, arr, len(slots), _stream(stream)), rig_ptr)
 
 
-def _rgb_mode(on_dev, imgs, in_place):
-    if on_dev or not in_place:
-        return on_dev
-    assert all(t.is_pinned() for t in imgs), "reading in place needs pinned host tensors"
-    return FVV_MAPPED_HOST
+def _rgb_mode(on_dev, in_place):
+    return FVV_MAPPED_HOST if in_place and not on_dev else on_dev
 
 
 def fvv_colour(rig_ptr, slots, rgb, viewpoints, stream=None, in_place=False):
@@ -262,20 +308,11 @@ def fvv_colour(rig_ptr, slots, rgb, viewpoints, stream=None, in_place=False):
     (N,H,W,3) tensor); viewpoints: (n_slots,3).  in_place: pinned host
     tensors are read in place by the kernel (FVV_RGB_MAPPED_HOST) instead of
     being copied to the device."""
-    ptrs, on_dev, all_imgs = [], None, []
-    for per_slot in rgb:
-        imgs = list(per_slot) if not torch.is_tensor(per_slot) else list(per_slot.unbind(0))
-        for t in imgs:
-            assert t.dtype == torch.uint8 and t.is_contiguous()
-            on_dev = int(t.is_cuda) if on_dev is None else on_dev
-            assert int(t.is_cuda) == on_dev
-            ptrs.append(t.data_ptr())
-            all_imgs.append(t)
-    on_dev = _rgb_mode(on_dev, all_imgs, in_place)
-    vp = np.ascontiguousarray(np.asarray(viewpoints, np.float32).reshape(len(slots), 3))
-    arr = (C.c_int * len(slots))(*slots)
-    _check(_lib.fvv_colour(rig_ptr, arr, len(slots), _ptr_array(ptrs), on_dev,
-                           vp.ctypes.data_as(C.POINTER(C.c_float)), _stream(stream)), rig_ptr)
+    ptrs, on_dev, imgs = _images(rgb)
+    mode = _rgb_mode(on_dev, in_place)
+    n = len(slots)
+    _check_images(_lib.fvv_colour(rig_ptr, _int_array(slots), n, _ptr_array(ptrs), mode, _floats(viewpoints, 3 * n),
+                                  _stream(stream)), rig_ptr, mode, imgs)
 
 
 def fvv_render_view(rig_ptr, slot, rgb, P, centre, width, height, stream=None, with_cam=True, in_place=False):
@@ -286,22 +323,15 @@ def fvv_render_view(rig_ptr, slot, rgb, P, centre, width, height, stream=None, w
     (H,W,3) uint8; capture camera (H,W) int32 or None).  They are allocated on
     the current stream: with another `stream`, keep them until it has run, or
     record it on them (Tensor.record_stream) before they are dropped."""
-    imgs = list(rgb) if not torch.is_tensor(rgb) else list(rgb.unbind(0))
-    on_dev = None
-    for t in imgs:
-        assert t.dtype == torch.uint8 and t.is_contiguous()
-        on_dev = int(t.is_cuda) if on_dev is None else on_dev
-        assert int(t.is_cuda) == on_dev
-    on_dev = _rgb_mode(on_dev, imgs, in_place)
-    Pm = np.ascontiguousarray(np.asarray(P, np.float32).reshape(12))
-    Cm = np.ascontiguousarray(np.asarray(centre, np.float32).reshape(3))
+    ptrs, on_dev, imgs = _images([rgb])
+    mode = _rgb_mode(on_dev, in_place)
+    Pm, Cm = _floats(P, 12), _floats(centre, 3)
     key = torch.empty((height, width), dtype=torch.int64, device="cuda")
     out = torch.empty((height, width, 3), dtype=torch.uint8, device="cuda")
     cam = torch.empty((height, width), dtype=torch.int32, device="cuda") if with_cam else None
-    _check(_lib.fvv_render_view(rig_ptr, slot, _ptr_array([t.data_ptr() for t in imgs]), on_dev,
-                                Pm.ctypes.data_as(C.POINTER(C.c_float)), Cm.ctypes.data_as(C.POINTER(C.c_float)),
-                                width, height, _vp(key.data_ptr()), _vp(out.data_ptr()),
-                                _vp(cam.data_ptr()) if cam is not None else None, _stream(stream)), rig_ptr)
+    _check_images(_lib.fvv_render_view(rig_ptr, slot, _ptr_array(ptrs), mode, Pm, Cm, width, height, key.data_ptr(),
+                                       out.data_ptr(), cam.data_ptr() if cam is not None else None, _stream(stream)),
+                  rig_ptr, mode, imgs)
     return key, out, cam
 
 
@@ -344,15 +374,15 @@ def fvv_get_results_batch(rig_ptr, slots, outs, stream=None):
     dst = (ResultsDst * n)()
     on_dev = None
     for d, o in zip(dst, outs):
-        for k in ("verts", "tris", "rgb", "cam"):
+        for k in _RESULTS:
             t = o.get(k)
             if t is not None:
                 on_dev = t.is_cuda if on_dev is None else on_dev
-                assert t.is_cuda == on_dev and t.is_contiguous()
+                assert t.is_cuda is on_dev and t.is_contiguous()
                 setattr(d, k, t.data_ptr())
-    arr = (C.c_int * n)(*slots)
-    _check(_lib.fvv_get_results_batch(rig_ptr, arr, n, dst, int(bool(on_dev)), _stream(stream)), rig_ptr)
-    return [d.counts.as_dict() for d in dst]
+    _check(_lib.fvv_get_results_batch(rig_ptr, _int_array(slots), n, dst, int(bool(on_dev)), _stream(stream)), rig_ptr)
+    size, unpack = C.sizeof(ResultsDst), _COUNT_STRUCT.unpack_from
+    return [dict(zip(_COUNT_NAMES, unpack(dst, i * size))) for i in range(n)]
 
 
 def fvv_set_timing(rig_ptr, enable: bool):
