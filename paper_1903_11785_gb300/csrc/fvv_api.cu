@@ -296,7 +296,8 @@ fvv_status make_plan(const fvv_rig_desc* d, const fvv_recon_params* p, Plan& pl,
     take(L.vrgb, (size_t)mv * 3);
     take(L.vcam, (size_t)mv * 4);
     take(L.depth, align_up(pix * 4));
-    take(L.dbox, (size_t)FVV_MAX_CAMS * 4 * sizeof(int32_t));
+    take(L.dbox, (size_t)cs.n * g.max_rois * 4 * sizeof(int32_t));
+    take(L.dcount, (size_t)cs.n * sizeof(int32_t));
     if (d->host_staging < 0 || d->host_staging > 2) { err = "host_staging must be 0, 1 or 2"; return FVV_ERR_INVALID_ARG; }
     if (d->host_staging) take(L.mask_stage, pix);
     if (d->host_staging == 1) take(L.rgb_stage, pix * 3);
@@ -572,10 +573,10 @@ static cudaError_t enqueue_reconstruct(fvv_rig* rig, const SlotList& sl, cudaStr
     FVV_STAGE(FVV_STAGE_COARSE, launch_coarse_carve(rig->cams, g, rig->L, sl, rig->table, rig->sms, tu, st));
     FVV_STAGE(FVV_STAGE_CCL, launch_ccl(g, rig->L, sl, rig->sms, st));
     FVV_STAGE(FVV_STAGE_FINE, launch_fine_carve(rig->cams, g, rig->L, sl, rig->sms, tu, st));
-    FVV_STAGE(FVV_STAGE_MC, launch_mc_prefix(g, rig->L, sl, mc, rig->sms, st));
+    FVV_STAGE(FVV_STAGE_MC, launch_mc_prefix(rig->cams, g, rig->L, sl, mc, rig->sms, st));
     FVV_STAGE(FVV_STAGE_BISECT, launch_bisect(rig->cams, g, rig->L, sl, rig->sms, tu, st));
     FVV_STAGE(FVV_STAGE_MC, launch_mc_triangles(g, rig->L, sl, mc, rig->sms, tu, st));
-    FVV_STAGE(FVV_STAGE_DEPTH, launch_depth(rig->cams, g, rig->L, sl, rig->sms, align_up(rig->npix * 4), tu, st));
+    FVV_STAGE(FVV_STAGE_DEPTH, launch_depth(rig->cams, g, rig->L, sl, rig->sms, tu, st));
 #undef FVV_STAGE
     return e;
 }
@@ -696,7 +697,7 @@ fvv_status fvv_autotune(fvv_rig* rig, const int* slots, int n_slots, void* strea
             case FVV_TUNE_FINE: return launch_fine_carve(rig->cams, g, rig->L, sl, rig->sms, tu, st);
             case FVV_TUNE_BISECT: return launch_bisect(rig->cams, g, rig->L, sl, rig->sms, tu, st);
             case FVV_TUNE_ZBUFFER:
-                return launch_depth(rig->cams, g, rig->L, sl, rig->sms, align_up(rig->npix * 4), tu, st);
+                return launch_depth(rig->cams, g, rig->L, sl, rig->sms, tu, st);
             default: return launch_mc_triangles(g, rig->L, sl, mc, rig->sms, tu, st);
         }
     };

@@ -131,7 +131,8 @@ struct Layout {
     size_t vrgb;                // uint8 x3, max_verts
     size_t vcam;                // int32, max_verts
     size_t depth;               // uint32 per pixel of all cameras
-    size_t dbox;                // int32 x4 per camera: box of the depth pixels the last z-buffer wrote
+    size_t dbox;                // int32 x4 per camera and ROI: boxes that hold the depth pixels the last z-buffer wrote
+    size_t dcount;              // int32 per camera: its boxes
     size_t mask_stage;          // uint8 per pixel (host uploads), or 0
     size_t rgb_stage;           // uint8 x3 per pixel (host uploads), or 0
 };
@@ -239,17 +240,18 @@ cudaError_t launch_ccl(const Grid& g, const Layout& L, const SlotList& sl, int s
 cudaError_t launch_filter(const Grid& g, const Layout& L, const SlotList& sl, cudaStream_t st);
 cudaError_t launch_fine_carve(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl,
                               int sms, const Tuning& tu, cudaStream_t st);
-cudaError_t launch_mc_prefix(const Grid& g, const Layout& L, const SlotList& sl, const McTable& mc, int sms,
+cudaError_t launch_mc_prefix(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl, const McTable& mc, int sms,
                              cudaStream_t st);
 cudaError_t launch_bisect(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl, int sms,
                           const Tuning& tu, cudaStream_t st);
 cudaError_t launch_mc_triangles(const Grid& g, const Layout& L, const SlotList& sl, const McTable& mc, int sms,
                                 const Tuning& tu, cudaStream_t st);
 // Depth images of every slot to empty and their written boxes to none (once,
-// when a rig is created).
+// when a rig is created).  They are cleared again where the last z-buffer wrote
+// by launch_fine_carve, and launch_mc_prefix lists the next one's boxes.
 cudaError_t launch_init_depth(const CamSet& cams, const Layout& L, int n_slots, int sms, cudaStream_t st);
 cudaError_t launch_depth(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl,
-                         int sms, size_t depth_bytes, const Tuning& tu, cudaStream_t st);
+                         int sms, const Tuning& tu, cudaStream_t st);
 // Colour-call arguments of up to kColourBatch slots, passed by value as a
 // kernel parameter (so nothing is copied from host memory).
 constexpr int kColourBatch = 48;

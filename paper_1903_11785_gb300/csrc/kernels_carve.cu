@@ -319,9 +319,11 @@ __global__ void __launch_bounds__(256) k_coarse_rest(const __grid_constant__ Cam
     }
 }
 
-// Clears the fine grids and the compaction's chunk states, and resets the
-// fine carve's tile counter.
-__global__ void __launch_bounds__(256) k_clear_fine(const __grid_constant__ Layout L,
+// Clears the fine grids, the compaction's chunk states and the depth pixels
+// that the slot's last z-buffer may have written, and resets the fine carve's
+// tile counter.
+__global__ void __launch_bounds__(256) k_clear_fine(const __grid_constant__ CamSet cams, const __grid_constant__ Grid g,
+                                                    const __grid_constant__ Layout L,
                                                     const __grid_constant__ SlotList sl) {
     pdl_begin();
     const int slot = sl.s[blockIdx.y];
@@ -352,6 +354,33 @@ __global__ void __launch_bounds__(256) k_clear_fine(const __grid_constant__ Layo
         clen[i] = n4 <= kSlabWords ? n4 : 0u;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) info->next_tile = 0u;
+    // Depth boxes: a camera's rows, counted through all its boxes, are dealt out
+    // to the warps of its blocks (blocks i, i + cameras, ...; fewer blocks than
+    // cameras take several cameras each).
+    const int lane = threadIdx.x & 31, bw = blockDim.x >> 5;
+    const int blocks = (int)gridDim.x, block = (int)blockIdx.x;
+    const bool many = blocks >= cams.n;
+    const int sub = many ? block / cams.n : 0;
+    const int subs = many ? (blocks - block % cams.n + cams.n - 1) / cams.n : 1;
+    const int nw = subs * bw, me = sub * bw + (int)(threadIdx.x >> 5);
+    for (int n = block % cams.n; n < cams.n; n += many ? cams.n : blocks) {
+        const int W = cams.c[n].W, count = slot_ptr<int>(L, slot, L.dcount)[n];
+        const int4* box = slot_ptr<int4>(L, slot, L.dbox) + (size_t)n * (unsigned)g.max_rois;
+        uint32_t* D = slot_ptr<uint32_t>(L, slot, L.depth) + cams.c[n].pix_off;
+        int at = me;                       // this warp's first row of the box at hand
+        for (int k0 = 0; k0 < count; k0 += 32) {
+            const int4 mine = k0 + lane < count ? box[k0 + lane] : make_int4(0, -1, 0, -1);
+            for (int k = 0; k < min(32, count - k0); ++k) {
+                const int x0 = __shfl_sync(kFull, mine.x, k), x1 = __shfl_sync(kFull, mine.y, k);
+                const int y0 = __shfl_sync(kFull, mine.z, k), rows = __shfl_sync(kFull, mine.w, k) - y0 + 1;
+                for (; at < rows; at += nw) {
+                    uint32_t* row = D + (size_t)(y0 + at) * (unsigned)W;
+                    for (int x = x0 + lane; x <= x1; x += 32) __stcs(row + x, kEmptyDepth);
+                }
+                at -= rows;
+            }
+        }
+    }
 }
 
 // The ROI holding fine-carve tile t: the last ROI whose first tile is <= t.
@@ -775,7 +804,7 @@ cudaError_t launch_coarse_carve(const CamSet& cams, const Grid& g, const Layout&
 cudaError_t launch_fine_carve(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl, int sms,
                               const Tuning& tu, cudaStream_t st) {
     const int gc = grid_x(sms, sl.n, (long long)g.max_fine_words, 256);
-    launch_pdl(k_clear_fine, dim3(gc, sl.n), dim3(256), 0, st, L, sl);
+    launch_pdl(k_clear_fine, dim3(gc, sl.n), dim3(256), 0, st, cams, g, L, sl);
     const int th = tu.threads[FVV_TUNE_FINE];
     // Blocks per slot: no more than can be resident for one, nor than one per
     // 2048 words of capacity (frames use about a sixth of it; a slot given more

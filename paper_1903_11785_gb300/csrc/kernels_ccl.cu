@@ -94,9 +94,10 @@ __global__ void __launch_bounds__(256) k_union(const __grid_constant__ Grid g, c
     if (budget <= 0) atomicOr(&slot_ptr<SlotInfo>(L, slot, L.info)->flags, (unsigned)FVV_FLAG_LOOP);
 }
 
-// Point every voxel at its root and list the roots (unordered); words are
-// taken as in k_union, a lane per voxel.  A thread writes only its own
-// voxel's entry (see find_root_readonly).
+// Point every voxel at its root, list the roots (unordered), tag each one's
+// parent entry with -(its place + 1) and reset its component's statistics;
+// words are taken as in k_union, a lane per voxel.  A thread writes only its
+// own voxel's entry (see find_root_readonly; a walk ends at a tagged root).
 __global__ void __launch_bounds__(256) k_compress(const __grid_constant__ Grid g, const __grid_constant__ Layout L,
                                                   const __grid_constant__ SlotList sl) {
     pdl_begin();
@@ -104,6 +105,7 @@ __global__ void __launch_bounds__(256) k_compress(const __grid_constant__ Grid g
     const uint32_t* bits = slot_ptr<uint32_t>(L, slot, L.coarse);
     int* parent = slot_ptr<int>(L, slot, L.parent);
     int* roots = slot_ptr<int>(L, slot, L.roots);
+    int* cstat = slot_ptr<int>(L, slot, L.cstat);
     SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
     const uint32_t nwords = (uint32_t)g.nz * g.ny * g.nxw;
     const int lane = threadIdx.x & 31;
@@ -128,65 +130,22 @@ __global__ void __launch_bounds__(256) k_compress(const __grid_constant__ Grid g
             const int Lin = (int)row * g.nx + wx * 32 + lane;
             const int r = find_root_readonly(parent, Lin, budget);
             if (r == Lin) {
+                // a root: component k in the order found, until k_filter sorts them
                 const int k = atomicAdd(&info->n_roots, 1);
-                if (k < g.max_comp) roots[k] = Lin;
+                if (k < g.max_comp) {
+                    roots[k] = Lin;
+                    parent[Lin] = -(k + 1);
+                    int* st = cstat + 7 * k;
+                    st[0] = 0;
+                    st[1] = st[2] = st[3] = 0x7FFFFFFF;
+                    st[4] = st[5] = st[6] = -1;
+                }
             } else {
                 parent[Lin] = r;
             }
         }
     }
     if (budget <= 0) atomicOr(&info->flags, (unsigned)FVV_FLAG_LOOP);
-}
-
-// One block per slot: sort the roots (bitonic, in shared memory) so that
-// component i is the one with the i-th smallest least index; tag each root's
-// parent entry with -(i+1); reset the per-component statistics.
-__global__ void __launch_bounds__(1024) k_sort_roots(const __grid_constant__ Grid g, const __grid_constant__ Layout L,
-                                                     const __grid_constant__ SlotList sl) {
-    pdl_begin();
-    __shared__ int key[kMaxComponents];
-    const int slot = sl.s[blockIdx.x];
-    SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
-    int* roots = slot_ptr<int>(L, slot, L.roots);
-    int* parent = slot_ptr<int>(L, slot, L.parent);
-    int* cstat = slot_ptr<int>(L, slot, L.cstat);
-    int n = info->n_roots;
-    if (n > g.max_comp) {
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            info->flags |= FVV_FLAG_ROOTS;
-            info->n_roots = 0;
-        }
-        return;
-    }
-    int m = 1;
-    while (m < n) m <<= 1;
-    for (int i = threadIdx.x; i < m; i += blockDim.x) key[i] = i < n ? roots[i] : 0x7FFFFFFF;
-    __syncthreads();
-    for (int k = 2; k <= m; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < m; i += blockDim.x) {
-                const int p = i ^ j;
-                if (p > i) {
-                    const bool up = (i & k) == 0;
-                    const int a = key[i], b = key[p];
-                    if ((a > b) == up) {
-                        key[i] = b;
-                        key[p] = a;
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    }
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        roots[i] = key[i];
-        parent[key[i]] = -(i + 1);
-        int* s = cstat + 7 * i;
-        s[0] = 0;
-        s[1] = s[2] = s[3] = 0x7FFFFFFF;
-        s[4] = s[5] = s[6] = -1;
-    }
 }
 
 // Voxel count and inclusive box of every component (Sec. II-B-2 takes the
@@ -200,7 +159,7 @@ __global__ void __launch_bounds__(256) k_stats(const __grid_constant__ Grid g, c
     pdl_begin();
     const int slot = sl.s[blockIdx.y];
     const SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
-    if (info->n_roots <= 0) return;
+    if (info->n_roots <= 0 || info->n_roots > g.max_comp) return;   // (k_filter flags too many)
     const uint32_t* bits = slot_ptr<uint32_t>(L, slot, L.coarse);
     const int* parent = slot_ptr<int>(L, slot, L.parent);
     int* cstat = slot_ptr<int>(L, slot, L.cstat);
@@ -245,40 +204,75 @@ __global__ void __launch_bounds__(256) k_stats(const __grid_constant__ Grid g, c
     }
 }
 
-// One block per slot: Eq. (1) as its prose states it (keep iff
+// One block per slot: sort the roots (bitonic, in shared memory), so that
+// component i is the one with the i-th smallest least index; Eq. (1) as its
+// prose states it (keep iff
 // t_np <= count <= t_nb), canonical labels 1..K in component order, and the
 // ROI of each kept component: its box grown by one coarse voxel per side and
 // clamped (Sec. II-B-3 treats it as a volume of its own), covered by whole
 // fine voxels counted in integer micrometres, with the fine grid's origin and
 // word layout.  Capacity overflows set a flag and leave the slot with no ROIs.
+// `label` is indexed by the components' places in the order found.
 __global__ void __launch_bounds__(1024) k_filter(const __grid_constant__ Grid g, const __grid_constant__ Layout L,
                                                  const __grid_constant__ SlotList sl) {
     pdl_begin();
+    __shared__ int key[kMaxComponents];
     __shared__ uint32_t sh[33];
     __shared__ unsigned long long sh64[33];
     __shared__ int s_fail;
     const int slot = sl.s[blockIdx.x];
     SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
-    const int n = info->n_roots;
     const int* cstat = slot_ptr<int>(L, slot, L.cstat);
+    const int* parent = slot_ptr<int>(L, slot, L.parent);
+    const int* roots = slot_ptr<int>(L, slot, L.roots);
     int* label = slot_ptr<int>(L, slot, L.roi_label);
     DRoi* rois = slot_ptr<DRoi>(L, slot, L.rois);
+    int n = info->n_roots;
+    if (n > g.max_comp) {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            info->flags |= FVV_FLAG_ROOTS;
+            info->n_roots = 0;
+        }
+        n = 0;
+    }
+    int m = 1;
+    while (m < n) m <<= 1;
+    for (int i = threadIdx.x; i < m; i += blockDim.x) key[i] = i < n ? roots[i] : 0x7FFFFFFF;
+    __syncthreads();
+    for (int k = 2; k <= m; k <<= 1) {
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int i = threadIdx.x; i < m; i += blockDim.x) {
+                const int p = i ^ j;
+                if (p > i) {
+                    const bool up = (i & k) == 0;
+                    const int a = key[i], b = key[p];
+                    if ((a > b) == up) {
+                        key[i] = b;
+                        key[p] = a;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    }
     if (threadIdx.x == 0) s_fail = 0;
     // pass 1: labels; components are processed in tiles of blockDim
     uint32_t base = 0;
     for (int t0 = 0; t0 < n; t0 += blockDim.x) {
         const int i = t0 + threadIdx.x;
+        const int id = i < n ? -parent[key[i]] - 1 : 0;   // its place in the order found
         uint32_t keep = 0;
         if (i < n) {
-            const int c = cstat[7 * i];
+            const int c = cstat[7 * id];
             keep = (c >= g.t_np && c <= g.t_nb) ? 1u : 0u;
         }
         uint32_t tot;
         const uint32_t ex = block_exclusive_scan(keep, sh, tot);
-        if (i < n) label[i] = keep ? (int)(base + ex + 1) : 0;
+        if (i < n) label[id] = keep ? (int)(base + ex + 1) : 0;
         if (keep && base + ex < (uint32_t)g.max_rois) {
             DRoi r;
-            const int* s = cstat + 7 * i;
+            const int* s = cstat + 7 * id;
             const int dims[3] = {g.nx, g.ny, g.nz};
             bool ok = true;
             for (int a = 0; a < 3; ++a) {
@@ -354,7 +348,6 @@ cudaError_t launch_ccl(const Grid& g, const Layout& L, const SlotList& sl, int s
     const int gx = grid_x(sms, sl.n, words, 256);
     launch_pdl(k_union, dim3(gx, sl.n), dim3(256), 0, st, g, L, sl);
     launch_pdl(k_compress, dim3(gx, sl.n), dim3(256), 0, st, g, L, sl);
-    launch_pdl(k_sort_roots, dim3(sl.n), dim3(1024), 0, st, g, L, sl);
     launch_pdl(k_stats, dim3(gx, sl.n), dim3(256), 0, st, g, L, sl);
     launch_pdl(k_filter, dim3(sl.n), dim3(1024), 0, st, g, L, sl);
     return cudaGetLastError();

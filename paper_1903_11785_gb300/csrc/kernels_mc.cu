@@ -18,6 +18,7 @@
 // Vertex and triangle order is therefore (ROI, key) and (ROI, cell, table
 // order): independent of scheduling, identical to a serial scan.
 #include <atomic>
+#include <climits>
 
 #include "fvv_device.cuh"
 
@@ -301,6 +302,70 @@ __device__ __forceinline__ uint64_t pack_trec(uint32_t w, int b, int j, int cs, 
     return (uint64_t)w | (uint64_t)b << 26 | (uint64_t)j << 31 | (uint64_t)cs << 35 | (uint64_t)k << 43;
 }
 
+// The boxes that hold every pixel this frame's z-buffer can write, for the clear
+// of the slot's next frame, by the threads of one block: every mesh vertex lies
+// in its ROI's fine grid box grown by one fine voxel (padding samples and
+// surface points), so every covered pixel centre lies in the convex hull
+// of the projections of that box's eight corners, widened by two pixels and
+// clamped to the image; the whole image if a corner is not in front of the
+// camera.  One box per ROI and camera, or their union where that has fewer
+// pixels.  `area` and `bound`: shared memory, per camera.
+__device__ __forceinline__ void list_depth_boxes(const CamSet& cams, const Grid& g, const Layout& L, int slot,
+                                                 const DRoi* rois, int nrois, unsigned long long* area, int4* bound) {
+    int4* box = slot_ptr<int4>(L, slot, L.dbox);
+    int* count = slot_ptr<int>(L, slot, L.dcount);
+    for (int n = threadIdx.x; n < cams.n; n += blockDim.x) {
+        area[n] = 0ull;
+        bound[n] = make_int4(INT_MAX, -1, INT_MAX, -1);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < cams.n * nrois; i += blockDim.x) {
+        const int n = i / nrois, k = i - n * nrois;
+        const Cam& c = cams.c[n];
+        const DRoi& r = rois[k];
+        float lo[3], hi[3];
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = r.fo[a] - g.sf;
+            hi[a] = r.fo[a] + (float)(r.fdim[a] + 1) * g.sf;
+        }
+        float umin = 3.0e38f, umax = -3.0e38f, vmin = 3.0e38f, vmax = -3.0e38f;
+        bool front = true;
+        for (int q = 0; q < 8; ++q) {
+            float xh, yh, wh;
+            project(c.P, (q & 1) ? hi[0] : lo[0], (q & 2) ? hi[1] : lo[1], (q & 4) ? hi[2] : lo[2], xh, yh, wh);
+            front &= wh > 0.0f;
+            const float u = __fdiv_rn(xh, wh), v = __fdiv_rn(yh, wh);
+            umin = fminf(umin, u); umax = fmaxf(umax, u);
+            vmin = fminf(vmin, v); vmax = fmaxf(vmax, v);
+        }
+        int x0 = 0, x1 = c.W - 1, y0 = 0, y1 = c.H - 1;
+        if (front && umin > -1.0e6f && umax < 1.0e6f && vmin > -1.0e6f && vmax < 1.0e6f) {
+            x0 = max(0, (int)floorf(umin) - 2);
+            x1 = min(c.W - 1, (int)floorf(umax) + 2);
+            y0 = max(0, (int)floorf(vmin) - 2);
+            y1 = min(c.H - 1, (int)floorf(vmax) + 2);
+        }
+        const bool none = x0 > x1 || y0 > y1;
+        box[(size_t)n * (unsigned)g.max_rois + (unsigned)k] = none ? make_int4(0, -1, 0, -1) : make_int4(x0, x1, y0, y1);
+        if (none) continue;
+        atomicAdd(area + n, (unsigned long long)(x1 - x0 + 1) * (unsigned)(y1 - y0 + 1));
+        int* b = reinterpret_cast<int*>(bound + n);
+        atomicMin(b + 0, x0);
+        atomicMax(b + 1, x1);
+        atomicMin(b + 2, y0);
+        atomicMax(b + 3, y1);
+    }
+    __syncthreads();
+    for (int n = threadIdx.x; n < cams.n; n += blockDim.x) {
+        const int4 b = bound[n];
+        const bool any = b.x <= b.y && b.z <= b.w;
+        const bool one = any && area[n] > (unsigned long long)(b.y - b.x + 1) * (unsigned)(b.w - b.z + 1);
+        if (one) box[(size_t)n * (unsigned)g.max_rois] = b;
+        count[n] = !any ? 0 : one ? 1 : nrois;
+    }
+    __syncthreads();
+}
+
 // Sec. II-C classify and compact, in one pass over each slot's fine words:
 // 256-word chunks are claimed in order from a per-slot counter; a chunk's
 // words and the neighbours its cells reach (a slab) are copied into shared
@@ -314,7 +379,8 @@ __device__ __forceinline__ uint64_t pack_trec(uint32_t w, int b, int j, int cs, 
 // one record per vertex and one per triangle; the last chunk sets the
 // totals and the capacity flags.  A chunk waits only on chunks claimed
 // before it, whose blocks are running, so the look-back always ends.
-__global__ void __launch_bounds__(kChunk) k_mc_compact(const __grid_constant__ Grid g,
+__global__ void __launch_bounds__(kChunk) k_mc_compact(const __grid_constant__ CamSet cams,
+                                                       const __grid_constant__ Grid g,
                                                        const __grid_constant__ Layout L,
                                                        const __grid_constant__ SlotList sl,
                                                        const __grid_constant__ McTable mc) {
@@ -340,6 +406,10 @@ __global__ void __launch_bounds__(kChunk) k_mc_compact(const __grid_constant__ G
     uint64_t* trec = slot_ptr<uint64_t>(L, slot, L.trec);
     unsigned long long* cst = slot_ptr<unsigned long long>(L, slot, L.chunk_st);
     const uint32_t* clen = slot_ptr<uint32_t>(L, slot, L.chunk_len);
+    // one block of the slot lists the frame's depth boxes first (the slab is not in use yet)
+    if (blockIdx.x == gridDim.x - 1u)
+        list_depth_boxes(cams, g, L, slot, rois, nwords ? nrois : 0, reinterpret_cast<unsigned long long*>(slab),
+                         reinterpret_cast<int4*>(slab) + FVV_MAX_CAMS);
     uint32_t parity = 0;
     bool pending = false;   // a copy whose wait ran out may still be in flight (thread 0's view)
     RoiCursor p;
@@ -989,11 +1059,11 @@ __global__ void __launch_bounds__(256) k_mc_triangles(const __grid_constant__ La
 
 }  // namespace
 
-cudaError_t launch_mc_prefix(const Grid& g, const Layout& L, const SlotList& sl, const McTable& mc, int sms,
+cudaError_t launch_mc_prefix(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl, const McTable& mc, int sms,
                              cudaStream_t st) {
     const int gc = grid_x(sms, sl.n, g.max_chunks, 1);
-    const cudaError_t e = launch_pdl(k_mc_compact, dim3(gc, sl.n), dim3(kChunk), kSlabWords * sizeof(uint32_t), st, g,
-                                     L, sl, mc);
+    const cudaError_t e = launch_pdl(k_mc_compact, dim3(gc, sl.n), dim3(kChunk), kSlabWords * sizeof(uint32_t), st,
+                                     cams, g, L, sl, mc);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

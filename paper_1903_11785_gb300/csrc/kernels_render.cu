@@ -10,11 +10,11 @@
 namespace fvv {
 namespace {
 
-// The depth images only ever hold values inside each camera's box (x0, x1,
-// y0, y1, none when x1 < x0), which contains every pixel the slot's last
-// z-buffer could write: a depth stage clears the previous box, sets the box
-// for this frame (k_depth_box) and runs the z-buffer, so every pixel outside
-// it is empty (+infinity) without clearing the whole image each frame.
+// The depth images only ever hold values inside each camera's boxes
+// (Layout::dbox), which contain every pixel the slot's last z-buffer could
+// write: a reconstruction clears them (k_clear_fine) and lists its own
+// (list_depth_boxes), so every pixel outside them is empty (+infinity)
+// without clearing whole images each frame.
 __global__ void __launch_bounds__(256) k_init_depth(const __grid_constant__ Layout L, size_t n16,
                                                     int n_cams) {
     const int slot = blockIdx.y;
@@ -22,78 +22,7 @@ __global__ void __launch_bounds__(256) k_init_depth(const __grid_constant__ Layo
     const uint4 v = make_uint4(kEmptyDepth, kEmptyDepth, kEmptyDepth, kEmptyDepth);
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (size_t)gridDim.x * blockDim.x)
         d[i] = v;
-    if (blockIdx.x == 0 && threadIdx.x < (unsigned)n_cams) {
-        int4* box = slot_ptr<int4>(L, slot, L.dbox);
-        box[threadIdx.x] = make_int4(INT_MAX, -1, INT_MAX, -1);
-    }
-}
-
-// Clear each camera's written box (grid: blocks, cameras, slots).
-__global__ void __launch_bounds__(256) k_clear_depth(const __grid_constant__ CamSet cams,
-                                                     const __grid_constant__ Layout L,
-                                                     const __grid_constant__ SlotList sl) {
-    pdl_begin();
-    const int slot = sl.s[blockIdx.z];
-    const Cam& c = cams.c[blockIdx.y];
-    const int4 b = slot_ptr<int4>(L, slot, L.dbox)[blockIdx.y];
-    if (b.y < b.x || b.w < b.z) return;
-    uint32_t* D = slot_ptr<uint32_t>(L, slot, L.depth) + c.pix_off;
-    for (int y = b.z + (int)blockIdx.x; y <= b.w; y += (int)gridDim.x) {
-        uint32_t* row = D + (size_t)y * (unsigned)c.W;
-        for (int x = b.x + (int)threadIdx.x; x <= b.y; x += (int)blockDim.x) __stcs(row + x, kEmptyDepth);
-    }
-}
-
-// The box each camera's z-buffer can write this frame (after k_clear_depth,
-// before k_zbuffer): every mesh vertex lies in its ROI's fine grid box grown
-// by one fine voxel (padding samples and bisection points), so every covered
-// pixel centre lies in the convex hull of the projections of that box's
-// eight corners; the union over the ROIs, widened by two pixels and clamped
-// to the image, or the whole image if a corner is not in front of the
-// camera.  One block per slot, a thread per (camera, ROI).
-__global__ void k_depth_box(const __grid_constant__ CamSet cams, const __grid_constant__ Grid g,
-                            const __grid_constant__ Layout L, const __grid_constant__ SlotList sl) {
-    pdl_begin();
-    const int slot = sl.s[blockIdx.x];
-    int4* box = slot_ptr<int4>(L, slot, L.dbox);
-    for (int n = threadIdx.x; n < cams.n; n += blockDim.x) box[n] = make_int4(INT_MAX, -1, INT_MAX, -1);
-    __syncthreads();
-    const SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
-    const int nrois = info->n_words ? info->n_rois : 0;
-    const DRoi* rois = slot_ptr<DRoi>(L, slot, L.rois);
-    for (int i = threadIdx.x; i < cams.n * nrois; i += blockDim.x) {
-        const int n = i / nrois, k = i - n * nrois;
-        const Cam& c = cams.c[n];
-        const DRoi& r = rois[k];
-        float lo[3], hi[3];
-        for (int a = 0; a < 3; ++a) {
-            lo[a] = r.fo[a] - g.sf;
-            hi[a] = r.fo[a] + (float)(r.fdim[a] + 1) * g.sf;
-        }
-        float umin = 3.0e38f, umax = -3.0e38f, vmin = 3.0e38f, vmax = -3.0e38f;
-        bool front = true;
-        for (int q = 0; q < 8; ++q) {
-            float xh, yh, wh;
-            project(c.P, (q & 1) ? hi[0] : lo[0], (q & 2) ? hi[1] : lo[1], (q & 4) ? hi[2] : lo[2], xh, yh, wh);
-            front &= wh > 0.0f;
-            const float u = __fdiv_rn(xh, wh), v = __fdiv_rn(yh, wh);
-            umin = fminf(umin, u); umax = fmaxf(umax, u);
-            vmin = fminf(vmin, v); vmax = fmaxf(vmax, v);
-        }
-        int x0 = 0, x1 = c.W - 1, y0 = 0, y1 = c.H - 1;
-        if (front && umin > -1.0e6f && umax < 1.0e6f && vmin > -1.0e6f && vmax < 1.0e6f) {
-            x0 = max(0, (int)floorf(umin) - 2);
-            x1 = min(c.W - 1, (int)floorf(umax) + 2);
-            y0 = max(0, (int)floorf(vmin) - 2);
-            y1 = min(c.H - 1, (int)floorf(vmax) + 2);
-        }
-        if (x0 > x1 || y0 > y1) continue;
-        int* b = reinterpret_cast<int*>(box + n);
-        atomicMin(b + 0, x0);
-        atomicMax(b + 1, x1);
-        atomicMin(b + 2, y0);
-        atomicMax(b + 3, y1);
-    }
+    if (blockIdx.x == 0 && threadIdx.x < (unsigned)n_cams) slot_ptr<int>(L, slot, L.dcount)[threadIdx.x] = 0;
 }
 
 // Eq. (4) coverage of one triangle (world vertices X, Y, Z) in camera c, in
@@ -557,11 +486,7 @@ cudaError_t launch_init_depth(const CamSet& cams, const Layout& L, int n_slots, 
 }
 
 cudaError_t launch_depth(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl, int sms,
-                         size_t depth_bytes, const Tuning& tu, cudaStream_t st) {
-    (void)depth_bytes;
-    const int gc = std::max(1, sms * 4 / std::max(1, sl.n * cams.n));
-    launch_pdl(k_clear_depth, dim3(gc, cams.n, sl.n), dim3(256), 0, st, cams, L, sl);
-    launch_pdl(k_depth_box, dim3(sl.n), dim3(256), 0, st, cams, g, L, sl);
+                         const Tuning& tu, cudaStream_t st) {
     const int gz = tuned_grid(tu, FVV_TUNE_ZBUFFER, sms, sl.n, (long long)g.max_tris);
     const int th = tu.threads[FVV_TUNE_ZBUFFER];
     // warps that the GPU can hold for a slot: 1024 threads per SM at the kernel's 64 registers
