@@ -422,6 +422,7 @@ fvv_status fvv_create_rig(const fvv_rig_desc* desc, const fvv_recon_params* para
     build_mc_table(ntri.data(), edges.data());
     e = cudaMemcpy(rig->mc_ntri, ntri.data(), ntri.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(rig->mc_edges, edges.data(), edges.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = prepare_ccl();
     if (pl.table_cams) {
         uint32_t* tab = reinterpret_cast<uint32_t*>(rig->arena + pl.table);
         rig->table = CoarseTable{tab, pl.table_cams};

@@ -235,6 +235,8 @@ cudaError_t launch_coarse_table(const CamSet& cams, const Grid& g, uint32_t* e, 
 cudaError_t launch_reset_coarse(const Layout& L, const SlotList& sl, cudaStream_t st);
 cudaError_t launch_coarse_carve(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl,
                                 const CoarseTable& tab, int sms, const Tuning& tu, cudaStream_t st);
+// The labelling's kernels made ready on the current device (once, when a rig is created).
+cudaError_t prepare_ccl();
 cudaError_t launch_ccl(const Grid& g, const Layout& L, const SlotList& sl, int sms, cudaStream_t st);
 // The filter and ROI table alone (k_filter), e.g. again for another fine-carve tile shape.
 cudaError_t launch_filter(const Grid& g, const Layout& L, const SlotList& sl, cudaStream_t st);

@@ -212,18 +212,21 @@ __global__ void __launch_bounds__(256) k_stats(const __grid_constant__ Grid g, c
 // clamped (Sec. II-B-3 treats it as a volume of its own), covered by whole
 // fine voxels counted in integer micrometres, with the fine grid's origin and
 // word layout.  Capacity overflows set a flag and leave the slot with no ROIs.
-// `label` is indexed by the components' places in the order found.
+// `label` is indexed by the components' places in the order found.  It reads the
+// roots and statistics only, not the parents, which the coarse hull run again
+// (fvv_autotune) has started afresh.
+constexpr size_t kFilterSmem = kMaxComponents * (sizeof(int) + sizeof(uint16_t));
 __global__ void __launch_bounds__(1024) k_filter(const __grid_constant__ Grid g, const __grid_constant__ Layout L,
                                                  const __grid_constant__ SlotList sl) {
     pdl_begin();
-    __shared__ int key[kMaxComponents];
+    extern __shared__ int key[];                                          // roots, sorted below,
+    uint16_t* place = reinterpret_cast<uint16_t*>(key + kMaxComponents);   // and their places in the order found
     __shared__ uint32_t sh[33];
     __shared__ unsigned long long sh64[33];
     __shared__ int s_fail;
     const int slot = sl.s[blockIdx.x];
     SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
     const int* cstat = slot_ptr<int>(L, slot, L.cstat);
-    const int* parent = slot_ptr<int>(L, slot, L.parent);
     const int* roots = slot_ptr<int>(L, slot, L.roots);
     int* label = slot_ptr<int>(L, slot, L.roi_label);
     DRoi* rois = slot_ptr<DRoi>(L, slot, L.rois);
@@ -238,7 +241,10 @@ __global__ void __launch_bounds__(1024) k_filter(const __grid_constant__ Grid g,
     }
     int m = 1;
     while (m < n) m <<= 1;
-    for (int i = threadIdx.x; i < m; i += blockDim.x) key[i] = i < n ? roots[i] : 0x7FFFFFFF;
+    for (int i = threadIdx.x; i < m; i += blockDim.x) {
+        key[i] = i < n ? roots[i] : 0x7FFFFFFF;
+        place[i] = (uint16_t)i;
+    }
     __syncthreads();
     for (int k = 2; k <= m; k <<= 1) {
         for (int j = k >> 1; j > 0; j >>= 1) {
@@ -250,6 +256,9 @@ __global__ void __launch_bounds__(1024) k_filter(const __grid_constant__ Grid g,
                     if ((a > b) == up) {
                         key[i] = b;
                         key[p] = a;
+                        const uint16_t t = place[i];
+                        place[i] = place[p];
+                        place[p] = t;
                     }
                 }
             }
@@ -261,7 +270,7 @@ __global__ void __launch_bounds__(1024) k_filter(const __grid_constant__ Grid g,
     uint32_t base = 0;
     for (int t0 = 0; t0 < n; t0 += blockDim.x) {
         const int i = t0 + threadIdx.x;
-        const int id = i < n ? -parent[key[i]] - 1 : 0;   // its place in the order found
+        const int id = i < n ? (int)place[i] : 0;
         uint32_t keep = 0;
         if (i < n) {
             const int c = cstat[7 * id];
@@ -343,18 +352,22 @@ __global__ void __launch_bounds__(1024) k_filter(const __grid_constant__ Grid g,
 
 }  // namespace
 
+cudaError_t prepare_ccl() {
+    return cudaFuncSetAttribute(k_filter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFilterSmem);
+}
+
 cudaError_t launch_ccl(const Grid& g, const Layout& L, const SlotList& sl, int sms, cudaStream_t st) {
     const long long words = (long long)g.nz * g.ny * g.nxw;
     const int gx = grid_x(sms, sl.n, words, 256);
     launch_pdl(k_union, dim3(gx, sl.n), dim3(256), 0, st, g, L, sl);
     launch_pdl(k_compress, dim3(gx, sl.n), dim3(256), 0, st, g, L, sl);
     launch_pdl(k_stats, dim3(gx, sl.n), dim3(256), 0, st, g, L, sl);
-    launch_pdl(k_filter, dim3(sl.n), dim3(1024), 0, st, g, L, sl);
+    launch_pdl(k_filter, dim3(sl.n), dim3(1024), kFilterSmem, st, g, L, sl);
     return cudaGetLastError();
 }
 
 cudaError_t launch_filter(const Grid& g, const Layout& L, const SlotList& sl, cudaStream_t st) {
-    launch_pdl(k_filter, dim3(sl.n), dim3(1024), 0, st, g, L, sl);
+    launch_pdl(k_filter, dim3(sl.n), dim3(1024), kFilterSmem, st, g, L, sl);
     return cudaGetLastError();
 }
 
