@@ -279,7 +279,7 @@ fvv_status make_plan(const fvv_rig_desc* d, const fvv_recon_params* p, Plan& pl,
     take(L.front, (size_t)g.nz * g.ny * g.nxw * 16);
     take(L.parent, nvox * 4);
     take(L.roots, (size_t)g.max_comp * 4);
-    take(L.cstat, (size_t)g.max_comp * 7 * 4);
+    take(L.cstat, (size_t)g.max_comp * kStatStride * 4);
     take(L.rois, (size_t)g.max_rois * sizeof(DRoi));
     take(L.roi_label, (size_t)g.max_comp * 4);
     take(L.fine, (size_t)fw * 4);

@@ -42,7 +42,13 @@ __device__ __forceinline__ uint32_t coarse_word(const uint32_t* bits, const Grid
 // l+1 if N has l empty and l+1 occupied: at most two unions per voxel and
 // row, almost all of them at run starts.  A warp reads 32 words of the
 // bitset (a lane each) and then takes its non-empty words one at a time
-// with a lane per voxel.
+// with a lane per voxel: it lists the word's pairs and then makes the unions
+// a lane per pair.  A union is a chain of loads that depend on one another
+// and an atomic, and only a few of a word's lanes have one in each of the
+// nine places: made where they are found, nine such chains follow one another
+// (a court frame: 22.1 us, listed 16.4; four 4K frames 51 and 38; 64 court
+// frames, where other warps fill the gaps, 184 and 176).
+constexpr int kWordPairs = 4 * 32 + 1;   // per row 16 runs and 16 starts of the row's runs at most
 __global__ void __launch_bounds__(256) k_union(const __grid_constant__ Grid g, const __grid_constant__ Layout L,
                                                const __grid_constant__ SlotList sl) {
     pdl_begin();
@@ -52,6 +58,9 @@ __global__ void __launch_bounds__(256) k_union(const __grid_constant__ Grid g, c
     const uint32_t nwords = (uint32_t)g.nz * g.ny * g.nxw;
     const int lane = threadIdx.x & 31;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+    __shared__ int2 s_pair[8][kWordPairs];
+    int2* pair = s_pair[threadIdx.x >> 5];
+    const uint32_t below = (1u << lane) - 1u;
     int budget = kStepBudget;
     const uint32_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     for (uint32_t base = 0; base < nwords; base += nwarps * 32u) {
@@ -66,29 +75,37 @@ __global__ void __launch_bounds__(256) k_union(const __grid_constant__ Grid g, c
             pending &= pending - 1u;
             const uint32_t w = base + (uint32_t)src * nwarps + gw;
             const uint32_t word = __shfl_sync(kFull, mine, src);
-            if (!((word >> lane) & 1u) || budget <= 0) continue;
             const uint32_t row = w / (uint32_t)g.nxw;
             const int wx = (int)(w - row * g.nxw);
             const int y = (int)(row % (uint32_t)g.ny), z = (int)(row / (uint32_t)g.ny);
             const int x0 = wx * 32;
             const uint32_t starts = word & ~(word << 1);
-            const bool first = (starts >> lane) & 1u;                      // lane starts its run
+            const bool on = (word >> lane) & 1u, first = (starts >> lane) & 1u;   // lane starts its run
             const int run0 = (int)row * g.nx + x0 + (31 - __clz(starts & (0xFFFFFFFFu >> (31 - lane))));
+            int n = 0;                                                     // pairs so far
+            auto put = [&](bool want, int b) {
+                const uint32_t m = __ballot_sync(kFull, want);
+                if (want) pair[n + __popc(m & below)] = make_int2(run0, b);
+                n += __popc(m);
+            };
             // the run across the boundary with the word before, same row
-            if (lane == 0 && (coarse_word(bits, g, y, z, wx - 1) >> 31))
-                unite(parent, run0, run0 - 1, budget);
+            put(lane == 0 && on && (coarse_word(bits, g, y, z, wx - 1) >> 31), run0 - 1);
+#pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int dy = k == 0 ? -1 : k - 2, dz = k == 0 ? 0 : -1;
-                const uint32_t n = coarse_word(bits, g, y + dy, z + dz, wx);
+                const uint32_t own = coarse_word(bits, g, y + dy, z + dz, wx);
                 const uint32_t np = coarse_word(bits, g, y + dy, z + dz, wx - 1);
                 const uint32_t nn = coarse_word(bits, g, y + dy, z + dz, wx + 1);
-                const bool left = lane > 0 ? (n >> (lane - 1)) & 1u : np >> 31;
-                const bool mid = (n >> lane) & 1u;
-                const bool right = lane < 31 ? (n >> (lane + 1)) & 1u : nn & 1u;
+                const bool left = lane > 0 ? (own >> (lane - 1)) & 1u : np >> 31;
+                const bool mid = (own >> lane) & 1u;
+                const bool right = lane < 31 ? (own >> (lane + 1)) & 1u : nn & 1u;
                 const int nrow = ((z + dz) * g.ny + (y + dy)) * g.nx + x0;
-                if (first && (left || mid)) unite(parent, run0, nrow + (left ? lane - 1 : lane), budget);
-                if (!mid && right) unite(parent, run0, nrow + lane + 1, budget);
+                put(first && (left || mid), nrow + (left ? lane - 1 : lane));
+                put(on && !mid && right, nrow + lane + 1);
             }
+            __syncwarp();
+            for (int i = lane; i < n && budget > 0; i += 32) unite(parent, pair[i].x, pair[i].y, budget);
+            __syncwarp();
         }
     }
     if (budget <= 0) atomicOr(&slot_ptr<SlotInfo>(L, slot, L.info)->flags, (unsigned)FVV_FLAG_LOOP);
@@ -135,7 +152,7 @@ __global__ void __launch_bounds__(256) k_compress(const __grid_constant__ Grid g
                 if (k < g.max_comp) {
                     roots[k] = Lin;
                     parent[Lin] = -(k + 1);
-                    int* st = cstat + 7 * k;
+                    int* st = cstat + kStatStride * k;
                     st[0] = 0;
                     st[1] = st[2] = st[3] = 0x7FFFFFFF;
                     st[4] = st[5] = st[6] = -1;
@@ -153,7 +170,9 @@ __global__ void __launch_bounds__(256) k_compress(const __grid_constant__ Grid g
 // as in k_union: a non-empty word (one row segment: y and z are the same for
 // all its voxels) with a lane per voxel; lanes of the same component are
 // merged (__match_any_sync) and the lowest of them makes the atomics for the
-// group, whose x range is the span of its lanes.
+// group, whose x range is the span of its lanes.  (Reading a bound first, to
+// leave out the atomics that would not move it: 10 -> 20 us on a court frame,
+// as the reads wait behind the atomics.)
 __global__ void __launch_bounds__(256) k_stats(const __grid_constant__ Grid g, const __grid_constant__ Layout L,
                                                const __grid_constant__ SlotList sl) {
     pdl_begin();
@@ -191,7 +210,7 @@ __global__ void __launch_bounds__(256) k_stats(const __grid_constant__ Grid g, c
             }
             const uint32_t grp = __match_any_sync(kFull, idx);
             if (idx >= 0 && lane == __ffs(grp) - 1) {
-                int* st = cstat + 7 * idx;
+                int* st = cstat + kStatStride * idx;
                 atomicAdd(st, __popc(grp));
                 atomicMin(st + 1, wx * 32 + lane);
                 atomicMax(st + 4, wx * 32 + 31 - __clz(grp));
@@ -273,7 +292,7 @@ __global__ void __launch_bounds__(1024) k_filter(const __grid_constant__ Grid g,
         const int id = i < n ? (int)place[i] : 0;
         uint32_t keep = 0;
         if (i < n) {
-            const int c = cstat[7 * id];
+            const int c = cstat[kStatStride * id];
             keep = (c >= g.t_np && c <= g.t_nb) ? 1u : 0u;
         }
         uint32_t tot;
@@ -281,7 +300,7 @@ __global__ void __launch_bounds__(1024) k_filter(const __grid_constant__ Grid g,
         if (i < n) label[id] = keep ? (int)(base + ex + 1) : 0;
         if (keep && base + ex < (uint32_t)g.max_rois) {
             DRoi r;
-            const int* s = cstat + 7 * id;
+            const int* s = cstat + kStatStride * id;
             const int dims[3] = {g.nx, g.ny, g.nz};
             bool ok = true;
             for (int a = 0; a < 3; ++a) {
