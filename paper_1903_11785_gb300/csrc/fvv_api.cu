@@ -283,8 +283,7 @@ fvv_status make_plan(const fvv_rig_desc* d, const fvv_recon_params* p, Plan& pl,
     take(L.rois, (size_t)g.max_rois * sizeof(DRoi));
     take(L.roi_label, (size_t)g.max_comp * 4);
     take(L.fine, (size_t)fw * 4);
-    take(L.emask, (size_t)fw * 12);
-    take(L.vpre, (size_t)fw * 4);
+    take(L.emask, (size_t)fw * 16);
     take(L.chunk_st, (size_t)g.max_chunks * 16);
     take(L.chunk_len, (size_t)g.max_chunks * 4);
     take(L.vrec, (size_t)mv * 8);
@@ -423,6 +422,7 @@ fvv_status fvv_create_rig(const fvv_rig_desc* desc, const fvv_recon_params* para
     e = cudaMemcpy(rig->mc_ntri, ntri.data(), ntri.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(rig->mc_edges, edges.data(), edges.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = prepare_ccl();
+    if (e == cudaSuccess) e = prepare_mc();
     if (pl.table_cams) {
         uint32_t* tab = reinterpret_cast<uint32_t*>(rig->arena + pl.table);
         rig->table = CoarseTable{tab, pl.table_cams};
@@ -720,7 +720,7 @@ fvv_status fvv_autotune(fvv_rig* rig, const int* slots, int n_slots, void* strea
                 if (knob == FVV_TUNE_FINE) {
                     tu.fine_tile = tile;
                     // the ROI table's tile offsets for this shape (not timed)
-                    if (th == threads[0] && wv == waves[0]) e = launch_filter(tuned_grid_params(rig->grid, tu), rig->L, sl, st);
+                    if (th == threads[0] && wv == waves[0]) e = launch_filter(tuned_grid_params(rig->grid, tu), rig->L, sl, rig->sms, st);
                     if (e != cudaSuccess) break;
                 }
                 e = run(knob, tu);  // warm

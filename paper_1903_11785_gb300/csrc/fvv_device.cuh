@@ -316,19 +316,36 @@ struct RoiCursor {
     // word position
     int wx, yp, zp;
 
+    __device__ __forceinline__ void take(const DRoi& r) {
+        lo = r.word_off;
+        hi = lo + r.n_words;
+        nxw = r.nxw;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            fdim[a] = r.fdim[a];
+            fo[a] = r.fo[a];
+        }
+    }
+
     __device__ __forceinline__ void seek(const DRoi* rois, int n, uint32_t w) {
         if (w >= hi || w < lo) {
             k = roi_of_word(rois, n, w);
-            const DRoi& r = rois[k];
-            lo = r.word_off;
-            hi = lo + r.n_words;
-            nxw = r.nxw;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                fdim[a] = r.fdim[a];
-                fo[a] = r.fo[a];
-            }
+            take(rois[k]);
         }
+        place(w);
+    }
+
+    // seek for a word at or after the first word of ROI k0
+    __device__ __forceinline__ void seek_from(const DRoi* rois, int n, uint32_t w, int k0) {
+        if (w >= hi || w < lo) {
+            k = k0;
+            take(rois[k]);
+            while (w >= hi && k + 1 < n) take(rois[++k]);
+        }
+        place(w);
+    }
+
+    __device__ __forceinline__ void place(uint32_t w) {
         const uint32_t lw = w - lo;
         const uint32_t row = lw / (uint32_t)nxw;
         wx = (int)(lw - row * (uint32_t)nxw);

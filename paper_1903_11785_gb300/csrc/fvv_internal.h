@@ -22,12 +22,17 @@ constexpr int kMaxComponents = 8192;  // raw components sortable by one block
 // whose ten or so components take 2,700 words x 7 atomics: 42.2 us with 7
 // int32 each, 40.6 with 8, 38.4 with 32).
 constexpr int kStatStride = 32;
-// Words of the slab the MC compaction stages per 256-word chunk: the chunk
+// Words of the slab the MC compaction stages per chunk: the chunk
 // and the neighbours its cells reach (a word in +x, a row in +y, a plane in
 // +z).  Chunks whose ROIs reach further read global memory instead.
 constexpr uint32_t kSlabWords = 6144;
 constexpr int kMaxRois = 4096;
-constexpr int kChunk = 256;           // fine words per scan chunk (= block size)
+constexpr uint32_t kChunkRoi = 8192;  // a chunk's slab words + kChunkRoi * the ROI of its first word
+static_assert(kSlabWords < kChunkRoi && (unsigned long long)kChunkRoi * kMaxRois < 1ull << 32, "chunk_len");
+constexpr int kChunk = 256;           // threads of a block of k_mc_compact, fine words per turn of its chunks
+constexpr int kMaxTurns = 4;          // turns per chunk, by the words in the launch (launch_filter):
+constexpr int kTurnChunks = 4;
+constexpr int kMcBlocksPerSm = 4;     // resident blocks of k_mc_compact
 constexpr uint32_t kEmptyDepth = 0xFFFFFFFFu;  // depth-buffer bits meaning +inf
 constexpr int kMaxTriPerCell = 12;
 
@@ -84,9 +89,10 @@ struct SlotInfo {
     uint32_t n_chunks;
     uint32_t n_tiles;           // fine-carve tiles of all ROIs
     uint32_t next_tile;         // the fine carve's next unclaimed tile
-    uint32_t next_chunk;        // the compaction's next unclaimed 256-word chunk
+    uint32_t next_chunk;        // the compaction's next unclaimed chunk
     uint32_t n_verts, n_tris;
     uint32_t n_on;
+    uint32_t chunk_words;       // fine words per scan chunk
     uint32_t n_front;           // coarse words that camera 0 does not empty
     unsigned long long tests_coarse, tests_fine, tests_bisect;
     unsigned long long look_fine, look_bisect;   // silhouette words read
@@ -122,10 +128,9 @@ struct Layout {
     size_t rois;                // DRoi, max_rois
     size_t roi_label;           // int32 label per sorted component (0 = removed)
     size_t fine;                // uint32 fine bits, max_fine_words
-    size_t emask;               // uint32 x3 bipolar-edge masks per fine word
-    size_t vpre;                // uint32 exclusive vertex prefix per fine word
-    size_t chunk_st;            // uint64 x2 per 256-word chunk: look-back states (vertices, triangles)
-    size_t chunk_len;           // uint32 per chunk: words of its staged slab (a multiple of 4), 0: not staged
+    size_t emask;               // uint4 per fine word with a bipolar edge: masks in x, y, z, vertices of earlier words
+    size_t chunk_st;            // uint64 x2 per chunk: look-back states (vertices, triangles)
+    size_t chunk_len;           // uint32 per chunk: kChunkRoi * the ROI of its first word + words of its staged slab (a multiple of 4; 0: not staged)
     size_t vrec;                // uint64 vertex records, max_verts
     size_t verts;               // float x3, max_verts
     size_t vcell;               // uint2 per vertex and four cameras: its pixel cells (write_cells), max_verts
@@ -240,11 +245,12 @@ cudaError_t launch_coarse_table(const CamSet& cams, const Grid& g, uint32_t* e, 
 cudaError_t launch_reset_coarse(const Layout& L, const SlotList& sl, cudaStream_t st);
 cudaError_t launch_coarse_carve(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl,
                                 const CoarseTable& tab, int sms, const Tuning& tu, cudaStream_t st);
-// The labelling's kernels made ready on the current device (once, when a rig is created).
+// The labelling's and the compaction's kernels made ready on the current device (once, when a rig is created).
 cudaError_t prepare_ccl();
+cudaError_t prepare_mc();
 cudaError_t launch_ccl(const Grid& g, const Layout& L, const SlotList& sl, int sms, cudaStream_t st);
 // The filter and ROI table alone (k_filter), e.g. again for another fine-carve tile shape.
-cudaError_t launch_filter(const Grid& g, const Layout& L, const SlotList& sl, cudaStream_t st);
+cudaError_t launch_filter(const Grid& g, const Layout& L, const SlotList& sl, int sms, cudaStream_t st);
 cudaError_t launch_fine_carve(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl,
                               int sms, const Tuning& tu, cudaStream_t st);
 cudaError_t launch_mc_prefix(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl, const McTable& mc, int sms,

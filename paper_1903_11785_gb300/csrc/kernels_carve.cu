@@ -334,8 +334,8 @@ __global__ void __launch_bounds__(256) k_clear_fine(const __grid_constant__ CamS
     // the compaction's look-back states of this reconstruction's chunks, and
     // each chunk's slab: words lo .. hi-1, hi past the farthest neighbour of
     // its words, in whole 16-byte units (the fine array is padded to 256
-    // bytes), or 0 when that is more than kSlabWords
-    const uint32_t nchunks = info->n_chunks;
+    // bytes), or 0 when that is more than kSlabWords; with it the ROI of word lo
+    const uint32_t nchunks = info->n_chunks, cw = info->chunk_words;
     const int nrois = info->n_rois;
     const DRoi* rois = slot_ptr<DRoi>(L, slot, L.rois);
     unsigned long long* cst = slot_ptr<unsigned long long>(L, slot, L.chunk_st);
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(256) k_clear_fine(const __grid_constant__ CamS
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nchunks; i += gridDim.x * blockDim.x) {
         cst[2 * (size_t)i] = 0ull;
         cst[2 * (size_t)i + 1] = 0ull;
-        const uint32_t lo = i * kChunk, last = min(lo + (uint32_t)kChunk, nwords) - 1u;
+        const uint32_t lo = i * cw, last = min(lo + cw, nwords) - 1u;
         const int k0 = roi_of_word(rois, nrois, lo), k1 = roi_of_word(rois, nrois, last);
         uint32_t reach = 0;
         for (int k = k0; k <= k1; ++k) {
@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(256) k_clear_fine(const __grid_constant__ CamS
             reach = max(reach, 1u + rs + rs * (uint32_t)(rois[k].fdim[1] + 2));
         }
         const uint32_t n4 = (min(nwords, last + 1u + reach) - lo + 3u) & ~3u;
-        clen[i] = n4 <= kSlabWords ? n4 : 0u;
+        clen[i] = (n4 <= kSlabWords ? n4 : 0u) + (uint32_t)k0 * kChunkRoi;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) info->next_tile = 0u;
     // Depth boxes: a camera's rows, counted through all its boxes, are dealt out

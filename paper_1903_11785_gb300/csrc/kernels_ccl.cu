@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(256) k_stats(const __grid_constant__ Grid g, c
 // (fvv_autotune) has started afresh.
 constexpr size_t kFilterSmem = kMaxComponents * (sizeof(int) + sizeof(uint16_t));
 __global__ void __launch_bounds__(1024) k_filter(const __grid_constant__ Grid g, const __grid_constant__ Layout L,
-                                                 const __grid_constant__ SlotList sl) {
+                                                 const __grid_constant__ SlotList sl, uint32_t turn_words) {
     pdl_begin();
     extern __shared__ int key[];                                          // roots, sorted below,
     uint16_t* place = reinterpret_cast<uint16_t*>(key + kMaxComponents);   // and their places in the order found
@@ -364,7 +364,10 @@ __global__ void __launch_bounds__(1024) k_filter(const __grid_constant__ Grid g,
             info->n_rois = K;
             info->n_words = (uint32_t)wbase;
             info->n_tiles = (uint32_t)sbase;
-            info->n_chunks = (uint32_t)((wbase + kChunk - 1) / kChunk);
+            // (k_mc_compact) a turn more for every turn_words words
+            const uint32_t cw = kChunk * min((uint32_t)kMaxTurns, max(1u, (uint32_t)wbase / turn_words));
+            info->chunk_words = cw;
+            info->n_chunks = ((uint32_t)wbase + cw - 1u) / cw;
         }
     }
 }
@@ -381,12 +384,14 @@ cudaError_t launch_ccl(const Grid& g, const Layout& L, const SlotList& sl, int s
     launch_pdl(k_union, dim3(gx, sl.n), dim3(256), 0, st, g, L, sl);
     launch_pdl(k_compress, dim3(gx, sl.n), dim3(256), 0, st, g, L, sl);
     launch_pdl(k_stats, dim3(gx, sl.n), dim3(256), 0, st, g, L, sl);
-    launch_pdl(k_filter, dim3(sl.n), dim3(1024), kFilterSmem, st, g, L, sl);
-    return cudaGetLastError();
+    return launch_filter(g, L, sl, sms, st);
 }
 
-cudaError_t launch_filter(const Grid& g, const Layout& L, const SlotList& sl, cudaStream_t st) {
-    launch_pdl(k_filter, dim3(sl.n), dim3(1024), kFilterSmem, st, g, L, sl);
+cudaError_t launch_filter(const Grid& g, const Layout& L, const SlotList& sl, int sms, cudaStream_t st) {
+    // Words of a slot per turn of its compaction's chunks: a turn for every kTurnChunks
+    // chunks of one turn that each resident block would have of all slots.
+    const uint32_t turn_words = (uint32_t)std::max(1LL, (long long)kChunk * kTurnChunks * kMcBlocksPerSm * sms / sl.n);
+    launch_pdl(k_filter, dim3(sl.n), dim3(1024), kFilterSmem, st, g, L, sl, turn_words);
     return cudaGetLastError();
 }
 

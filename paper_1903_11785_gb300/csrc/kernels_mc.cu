@@ -167,14 +167,38 @@ __device__ __forceinline__ uint32_t mixed_cells(const Nbhd& n) {
     return (a ^ n.s[0]) | (a ^ n.w[1]) | (a ^ n.s[1]) | (a ^ n.w[2]) | (a ^ n.s[2]) | (a ^ n.w[3]) | (a ^ n.s[3]);
 }
 
-__device__ __forceinline__ int cell_case(const Nbhd& n, int b) {
-    int c = 0;
+// The cases of all 32 cells of a word (bit 2k: w[k], bit 2k + 1: s[k]), a byte
+// each, cell b's in byte b % 4 of out[b / 4 * kChunk]: four 8 x 8 bit
+// transposes by swaps of bits, pairs and nibbles, some 100 instructions for
+// what costs 24 a cell when its bits are picked out of the eight words.
+__device__ __forceinline__ void cell_cases(const Nbhd& n, uint32_t* out) {
+    uint32_t lo[4], hi[4];   // [g]: byte g of w0 s0 w1 s1, and of w2 s2 w3 s3
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        c |= (int)((n.w[k] >> b) & 1u) << (2 * k);
-        c |= (int)((n.s[k] >> b) & 1u) << (2 * k + 1);
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t a = n.w[2 * h], b = n.s[2 * h], c = n.w[2 * h + 1], d = n.s[2 * h + 1];
+        const uint32_t ab = __byte_perm(a, b, 0x5140), ab2 = __byte_perm(a, b, 0x7362);
+        const uint32_t cd = __byte_perm(c, d, 0x5140), cd2 = __byte_perm(c, d, 0x7362);
+        uint32_t* o = h ? hi : lo;
+        o[0] = __byte_perm(ab, cd, 0x5410);
+        o[1] = __byte_perm(ab, cd, 0x7632);
+        o[2] = __byte_perm(ab2, cd2, 0x5410);
+        o[3] = __byte_perm(ab2, cd2, 0x7632);
     }
-    return c;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        uint32_t x = lo[q], y = hi[q], t;
+        t = (x ^ (x >> 7)) & 0x00AA00AAu;
+        x ^= t ^ (t << 7);
+        t = (y ^ (y >> 7)) & 0x00AA00AAu;
+        y ^= t ^ (t << 7);
+        t = (x ^ (x >> 14)) & 0x0000CCCCu;
+        x ^= t ^ (t << 14);
+        t = (y ^ (y >> 14)) & 0x0000CCCCu;
+        y ^= t ^ (t << 14);
+        t = (x ^ (y << 4)) & 0xF0F0F0F0u;
+        out[2 * q * kChunk] = x ^ t;
+        out[(2 * q + 1) * kChunk] = y ^ (t >> 4);
+    }
 }
 
 // The 8 words of load_nbhd, read from a slab of the slot's fine words
@@ -367,19 +391,40 @@ __device__ __forceinline__ void list_depth_boxes(const CamSet& cams, const Grid&
 }
 
 // Sec. II-C classify and compact, in one pass over each slot's fine words:
-// 256-word chunks are claimed in order from a per-slot counter; a chunk's
-// words and the neighbours its cells reach (a slab) are copied into shared
-// memory by one bulk copy; each thread takes one word: its bipolar-edge
-// masks (x: w ^ w>>1, y: w ^ w(y+1), z: w ^ w(z+1)), vertex count (their
-// popcounts) and triangle count (table counts of its mixed cells).  Block
-// scans give the offsets within the chunk, and a decoupled look-back over
-// the earlier chunks' published counts gives the chunk's base, so vertex
-// ids follow the edge-key order (3*Lpad + axis) and triangles (ROI, cell,
-// table order) of a serial scan.  Each word then writes its prefix, masks,
-// one record per vertex and one per triangle; the last chunk sets the
-// totals and the capacity flags.  A chunk waits only on chunks claimed
-// before it, whose blocks are running, so the look-back always ends.
-__global__ void __launch_bounds__(kChunk) k_mc_compact(const __grid_constant__ CamSet cams,
+// chunks of one to kMaxTurns turns of 256 words are claimed in order from a
+// per-slot counter; a chunk's words and the neighbours its cells reach (a slab)
+// are copied into shared memory by one bulk copy; each warp takes its words 32 at
+// a time, a lane each: their bipolar-edge masks (x: w ^ w>>1, y: w ^ w(y+1), z:
+// w ^ w(z+1)), vertex counts (the masks' popcounts) and triangle counts (table
+// counts of the mixed cells).  Sums over the block give the counts of the chunk,
+// and a decoupled look-back over the earlier chunks' published counts gives its
+// base, so vertex ids follow the edge-key order (3*Lpad + axis) and triangles
+// (ROI, cell, table order) of a serial scan.  Then each turn's words write their
+// masks and prefix, and its mixed cells, listed in order in shared memory, are
+// taken a lane each to write one record per vertex and one per triangle; the last
+// chunk sets the totals and the capacity flags.  A chunk waits only on chunks
+// claimed before it, whose blocks are running, so the look-back always ends.
+//
+// What bounds it is not the memory (some 15 MB for a court frame of 0.29 M words,
+// 0.38 M vertices and 0.77 M triangles) but the claim, copy, counts and look-back
+// that follow one another in every chunk, and, written by the lane that has the
+// word, the records: a word of a level surface has 32 mixed cells, its neighbours
+// none, and 12 of 32 lanes were at work.  A lane per listed cell, one store per
+// word with a crossed edge and none for the others, no look-back for chunks
+// without a mixed cell, and the ROI of a chunk's first word found beforehand
+// (k_clear_fine): one court frame 39.4 -> 29.4 us, 64 of them 1341 -> 815.  Longer
+// chunks share the chain out over more words where there are enough (the stage's
+// kernels for 64 court frames, 118 chunks of one turn for each resident block: 2009
+// us with one turn, 1877 with two, 1707 with four, the same with eight), and leave
+// the chip idle where there are not (a frame of 28,640 vertices, 0.1 chunks, with
+// one, two and four turns: 28, 34 and 43 us; four 4K court frames, 1.2 chunks: 54,
+// 58 and 75).  In between it matters little (court, 1.9 chunks, one and two turns:
+// 54 and 51; 4K mat, 3.3 chunks, one and three: 68 and 71), so launch_filter gives a
+// turn for every kTurnChunks = 4.  Tried without gain: claiming a chunk ahead, with
+// its copy (six times the time: a claimed chunk's counts then come only after the
+// look-back before them), looking back over 64 to 512 chunks at a time (the same to
+// half as much again), pauses between polls (the same).
+__global__ void __launch_bounds__(kChunk, kMcBlocksPerSm) k_mc_compact(const __grid_constant__ CamSet cams,
                                                        const __grid_constant__ Grid g,
                                                        const __grid_constant__ Layout L,
                                                        const __grid_constant__ SlotList sl,
@@ -387,12 +432,18 @@ __global__ void __launch_bounds__(kChunk) k_mc_compact(const __grid_constant__ C
     pdl_begin();
     extern __shared__ __align__(128) uint32_t slab[];   // kSlabWords
     __shared__ uint8_t s_ntri[256];
-    __shared__ uint32_t sh[33];
+    __shared__ uint32_t s_turn[kChunk / 32][kMaxTurns], s_tot[kChunk / 32];
+    __shared__ uint32_t s_word[kChunk / 32][4][32];        // a turn's words: masks, vertices before
+    __shared__ uint16_t s_cell[kChunk / 32][32 * 32];      // a turn's mixed cells: word * 32 + cell
+    __shared__ uint32_t s_case[8][kChunk];   // (cell_cases)
     __shared__ __align__(8) uint64_t bar;
-    __shared__ uint32_t s_c, s_use;
+    __shared__ uint32_t s_c, s_len, s_fail;
     __shared__ unsigned long long s_base[2];
     for (int i = threadIdx.x; i < 256; i += blockDim.x) s_ntri[i] = mc.ntri[i];
-    if (threadIdx.x == 0) mbar_init(&bar);
+    if (threadIdx.x == 0) {
+        mbar_init(&bar);
+        s_fail = 0u;
+    }
     __syncthreads();
     const int slot = sl.s[blockIdx.y];
     SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
@@ -400,8 +451,7 @@ __global__ void __launch_bounds__(kChunk) k_mc_compact(const __grid_constant__ C
     const int nrois = info->n_rois;
     DRoi* rois = slot_ptr<DRoi>(L, slot, L.rois);
     const uint32_t* fine = slot_ptr<uint32_t>(L, slot, L.fine);
-    uint32_t* emask = slot_ptr<uint32_t>(L, slot, L.emask);
-    uint32_t* vpre = slot_ptr<uint32_t>(L, slot, L.vpre);
+    uint4* emask = slot_ptr<uint4>(L, slot, L.emask);
     uint64_t* vrec = slot_ptr<uint64_t>(L, slot, L.vrec);
     uint64_t* trec = slot_ptr<uint64_t>(L, slot, L.trec);
     unsigned long long* cst = slot_ptr<unsigned long long>(L, slot, L.chunk_st);
@@ -410,63 +460,100 @@ __global__ void __launch_bounds__(kChunk) k_mc_compact(const __grid_constant__ C
     if (blockIdx.x == gridDim.x - 1u)
         list_depth_boxes(cams, g, L, slot, rois, nwords ? nrois : 0, reinterpret_cast<unsigned long long*>(slab),
                          reinterpret_cast<int4*>(slab) + FVV_MAX_CAMS);
+    bool pending = false;   // the wait for a copy ran out, and it may still be in flight
+    const uint32_t cw = info->chunk_words, turns = cw / kChunk, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    // A warp's counts in one word: under 2^15 vertices (3 x 32 x 256) and 2^17 triangles
+    constexpr int kVertBits = 15;
+    constexpr uint32_t kVertMask = (1u << kVertBits) - 1u;
+    static_assert(3 * 32 * 32 * kMaxTurns < 1 << kVertBits && kMaxTriPerCell * 32 * 32 * kMaxTurns < 1 << (32 - kVertBits),
+                  "a warp's counts");
+    const uint8_t* my_case = reinterpret_cast<const uint8_t*>(&s_case[0][threadIdx.x]);
+    auto case_of = [&](int b) { return (int)my_case[(b >> 2) * (kChunk * 4) + (b & 3)]; };
     uint32_t parity = 0;
-    bool pending = false;   // a copy whose wait ran out may still be in flight (thread 0's view)
     RoiCursor p;
     for (;;) {
         if (threadIdx.x == 0) {
             const uint32_t c = nchunks ? atomicAdd(&info->next_chunk, 1u) : 0u;
+            const uint32_t len = c < nchunks ? __ldcg(clen + c) : 0u;   // (k_clear_fine)
             s_c = c;
-            s_use = 0;
-            const uint32_t n4 = c < nchunks && !pending ? __ldcg(clen + c) : 0u;   // (k_clear_fine)
-            if (n4) {
-                s_use = 1;
-                fence_proxy_async();
-                mbar_expect_tx(&bar, n4 * 4u);
-                bulk_copy_g2s(slab, fine + c * kChunk, n4 * 4u, &bar);
-            }
+            s_len = s_fail ? len & ~(kChunkRoi - 1u) : len;
         }
-        __syncthreads();
+        __syncthreads();                                   // the chunk is claimed, and the slab's last one written
         const uint32_t c = s_c;
         if (c >= nchunks) break;
-        bool use = s_use != 0u;
+        const uint32_t len = s_len, n4 = len & (kChunkRoi - 1u);
+        bool use = n4 != 0u;
         if (use) {
+            if (threadIdx.x == 0) {
+                fence_proxy_async();
+                mbar_expect_tx(&bar, n4 * 4u);
+                bulk_copy_g2s(slab, fine + c * cw, n4 * 4u, &bar);
+            }
             bool done = false;
             for (int it = 0; it < kMaxPolls && !done; ++it) done = mbar_try_wait(&bar, parity);
-            if (__syncthreads_or(!done)) {
-                // the copy did not complete in time: this chunk and the later
-                // ones read global memory, and the slot is flagged
-                use = false;
-                if (threadIdx.x == 0) {
-                    pending = true;
-                    atomicOr(&info->flags, (unsigned)FVV_FLAG_LOOP);
-                }
-            } else {
+            // a copy that does not complete in time: this chunk and the later
+            // ones read global memory, and the slot is flagged
+            if (done) {
                 parity ^= 1u;
+            } else {
+                s_fail = 1u;
+                pending = true;
+                atomicOr(&info->flags, (unsigned)FVV_FLAG_LOOP);
             }
+            use = done;
         }
-        const uint32_t lo = c * kChunk, w = lo + threadIdx.x;
-        const bool in = w < nwords;
-        Nbhd n;
-        uint32_t xm = 0, ym = 0, zm = 0, vc = 0, tc = 0;
-        if (in) {
-            p.seek(rois, nrois, w);
+        const uint32_t lo = c * cw;
+        auto nbhd = [&](uint32_t w, Nbhd& n) {
             if (use) load_nbhd_slab(slab, lo, p, w, n);
             else load_nbhd(fine, p, w, n);
-            xm = n.w[0] ^ n.s[0];
-            ym = n.w[0] ^ n.w[1];
-            zm = n.w[0] ^ n.w[2];
-            vc = __popc(xm) + __popc(ym) + __popc(zm);
-            uint32_t mx = mixed_cells(n);
-            while (mx) {
-                const int b = __ffs(mx) - 1;
-                mx &= mx - 1;
-                tc += s_ntri[cell_case(n, b)];
+        };
+        // counts, 32 words at a time, in a warp's order of words
+        uint32_t run = 0, passes = 0;         // counts of the warp's words so far; bit j: turn j has anything to write
+        const uint32_t wlo = lo + warp * 32u * turns + lane;
+        for (uint32_t j = 0; j < turns; ++j) {
+            const uint32_t w = wlo + 32u * j;
+            uint32_t mixed = 0;
+            bool start = false;
+            Nbhd n;
+            if (w < nwords) {
+                p.seek_from(rois, nrois, w, j ? p.k : (int)(len / kChunkRoi));
+                nbhd(w, n);
+                mixed = mixed_cells(n);
+                start = w == p.lo;
+            }
+            if (!__any_sync(kFull, mixed || start)) continue;
+            passes |= 1u << j;
+            if (lane == 0) s_turn[warp][j] = run;
+            uint32_t v = 0;
+            if (mixed) {
+                cell_cases(n, &s_case[0][threadIdx.x]);
+                uint32_t t = 0;
+                for (uint32_t m = mixed; m; m &= m - 1u) t += s_ntri[case_of(__ffs(m) - 1)];
+                v = t << kVertBits |
+                    (uint32_t)(__popc(n.w[0] ^ n.s[0]) + __popc(n.w[0] ^ n.w[1]) + __popc(n.w[0] ^ n.w[2]));
+            }
+            run += __reduce_add_sync(kFull, v);
+        }
+        if (lane == 0) s_tot[warp] = run;
+        // A chunk without a mixed cell has neither vertices nor triangles; without
+        // a ROI's first word and not the last, nothing else wants its base either.
+        const bool full = __syncthreads_or(passes || c == nchunks - 1u);
+        if (threadIdx.x == 0) {
+            if (!full) {
+                st_state(cst + 2 * (size_t)c, c ? kStAgg : kStInc);
+                st_state(cst + 2 * (size_t)c + 1, c ? kStAgg : kStInc);
             }
         }
-        uint32_t tv, tt;
-        const uint32_t ev = block_exclusive_scan(vc, sh, tv);
-        const uint32_t et = block_exclusive_scan(tc, sh, tt);
+        if (!full) continue;
+        uint32_t ev = 0, et = 0, tv = 0, tt = 0;
+#pragma unroll
+        for (int k = 0; k < kChunk / 32; ++k) {
+            const uint32_t t = s_tot[k];
+            if (k == (int)warp) ev = tv, et = tt;
+            tv += t & kVertMask;
+            tt += t >> kVertBits;
+        }
         if (threadIdx.x < 32) {
             unsigned long long bv = 0, bt = 0;
             bool ok = true;
@@ -497,41 +584,88 @@ __global__ void __launch_bounds__(kChunk) k_mc_compact(const __grid_constant__ C
             }
         }
         __syncthreads();
-        if (in) {
-            const unsigned long long vb = s_base[0] + ev, tb = s_base[1] + et;
-            vpre[w] = (uint32_t)vb;
-            if (w == p.lo) {
-                rois[p.k].vert_off = (uint32_t)vb;
-                rois[p.k].tri_off = (uint32_t)tb;
+        for (; passes; passes &= passes - 1u) {
+            const uint32_t j = __ffs(passes) - 1, w = wlo + 32u * j;
+            const uint32_t before = s_turn[warp][j];
+            const unsigned long long vb = s_base[0] + ev + (before & kVertMask), tb = s_base[1] + et + (before >> kVertBits);
+            Nbhd n;
+            uint32_t mixed = 0, xm = 0, ym = 0, zm = 0;
+            bool start = false;
+            if (w < nwords) {
+                p.seek_from(rois, nrois, w, (int)(len / kChunkRoi));
+                nbhd(w, n);
+                mixed = mixed_cells(n);
+                xm = n.w[0] ^ n.s[0];
+                ym = n.w[0] ^ n.w[1];
+                zm = n.w[0] ^ n.w[2];
+                start = w == p.lo;
+                if (turns > 1u && mixed) cell_cases(n, &s_case[0][threadIdx.x]);
             }
-            emask[3 * (size_t)w + 0] = xm;
-            emask[3 * (size_t)w + 1] = ym;
-            emask[3 * (size_t)w + 2] = zm;
-            const uint32_t own = n.w[0];
-            uint32_t any = xm | ym | zm;
-            unsigned long long id = vb;
-            while (any) {
-                const int b = __ffs(any) - 1;
-                any &= any - 1;
-                const int s0 = (own >> b) & 1u, xp = p.wx * 32 + b;
-                if (((xm >> b) & 1u) && id < g.max_verts) vrec[id] = pack_vrec(p.k, 0, s0, xp, p.yp, p.zp);
-                id += (xm >> b) & 1u;
-                if (((ym >> b) & 1u) && id < g.max_verts) vrec[id] = pack_vrec(p.k, 1, s0, xp, p.yp, p.zp);
-                id += (ym >> b) & 1u;
-                if (((zm >> b) & 1u) && id < g.max_verts) vrec[id] = pack_vrec(p.k, 2, s0, xp, p.yp, p.zp);
-                id += (zm >> b) & 1u;
+            // vertices and mixed cells of the words before this lane's
+            uint32_t x = (uint32_t)(__popc(xm) + __popc(ym) + __popc(zm)) | (uint32_t)__popc(mixed) << 16;
+            const uint32_t own = x;
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(kFull, x, o);
+                if (lane >= o) x += y;
             }
-            if (tc) {
-                uint32_t mx = mixed_cells(n);
-                unsigned long long t = tb;
-                while (mx) {
-                    const int b = __ffs(mx) - 1;
-                    mx &= mx - 1;
-                    const int cs = cell_case(n, b);
-                    for (int j = 0; j < (int)s_ntri[cs]; ++j, ++t)
-                        if (t < g.max_tris) trec[t] = pack_trec(w, b, j, cs, p.k);
+            const uint32_t cells = __shfl_sync(kFull, x, 31) >> 16;
+            x -= own;
+            const uint32_t vfirst = x & 0xFFFFu;
+            if (__any_sync(kFull, start)) {
+                uint32_t t = 0;
+                for (uint32_t m = mixed; m; m &= m - 1u) t += s_ntri[case_of(__ffs(m) - 1)];
+                uint32_t y = t;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t z = __shfl_up_sync(kFull, y, o);
+                    if (lane >= o) y += z;
+                }
+                if (start) {
+                    rois[p.k].vert_off = (uint32_t)(vb + vfirst);
+                    rois[p.k].tri_off = (uint32_t)(tb + y - t);
                 }
             }
+            // (read only for words with a crossed edge)
+            if (xm | ym | zm) emask[w] = make_uint4(xm, ym, zm, (uint32_t)(vb + vfirst));
+            // the turn's mixed cells in order, for a lane each
+            s_word[warp][0][lane] = xm;
+            s_word[warp][1][lane] = ym;
+            s_word[warp][2][lane] = zm;
+            s_word[warp][3][lane] = vfirst;
+            uint16_t* put = s_cell[warp] + (x >> 16);
+            for (uint32_t m = mixed; m; m &= m - 1u) *put++ = (uint16_t)(lane * 32 + __ffs(m) - 1);
+            const uint64_t rec = pack_vrec(p.k, 0, 0, p.wx * 32, p.yp, p.zp);
+            __syncwarp();
+            unsigned long long t = tb;
+            for (uint32_t i = 0; i < cells; i += 32u) {
+                const bool has = i + lane < cells;
+                const uint32_t cell = has ? s_cell[warp][i + lane] : 0u, src = cell >> 5, b = cell & 31u;
+                const uint32_t cs = has ? reinterpret_cast<const uint8_t*>(&s_case[b >> 2][warp * 32u + src])[b & 3u] : 0u;
+                const uint32_t nt = s_ntri[cs];                       // (none for case 0)
+                uint32_t y = nt;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t z = __shfl_up_sync(kFull, y, o);
+                    if (lane >= o) y += z;
+                }
+                const uint64_t r = __shfl_sync(kFull, rec, (int)src) + ((uint64_t)b << 17 | (uint64_t)(cs & 1u) << 16);
+                if (has) {
+                    const uint32_t lm = (1u << b) - 1u;
+                    unsigned long long id = vb + s_word[warp][3][src] + __popc(s_word[warp][0][src] & lm) +
+                                            __popc(s_word[warp][1][src] & lm) + __popc(s_word[warp][2][src] & lm);
+                    // the cell's own sample (case bit 0) against the next in x, y and z (bits 1, 2 and 4)
+                    const bool fx = (cs ^ cs >> 1) & 1u, fy = (cs ^ cs >> 2) & 1u, fz = (cs ^ cs >> 4) & 1u;
+                    if (fx && id < g.max_verts) vrec[id] = r;
+                    id += fx;
+                    if (fy && id < g.max_verts) vrec[id] = r + (1u << 14);
+                    id += fy;
+                    if (fz && id < g.max_verts) vrec[id] = r + (2u << 14);
+                    const unsigned long long first = t + y - nt;
+                    const uint64_t tr = pack_trec(w - lane + src, (int)b, 0, (int)cs, (int)(r & 0x3FFFu));
+                    for (uint32_t q = 0; q < nt; ++q)
+                        if (first + q < g.max_tris) trec[first + q] = tr + ((uint64_t)q << 31);
+                }
+                t += __shfl_sync(kFull, y, 31);
+            }
+            __syncwarp();
         }
     }
     if (threadIdx.x == 0 && pending) {
@@ -997,19 +1131,23 @@ __global__ void __launch_bounds__(256) k_lambda(const __grid_constant__ CamSet c
 // its word's vertex offset plus the rank of the edge among the word's
 // bipolar edges (x, y, z masks in canonical order).  Also the centroid
 // ((v0 + v1) + v2) / 3 of each triangle, for the depth images (Sec. II-D-1).
+// Near the memory's rate with many frames: 68 bytes of records a triangle and the
+// vertices, 64 court frames (49 M triangles) 810 us.  A word's masks and offset are
+// one 16-byte load (four of 4 bytes: 897), the table 16 bytes a load (a court frame
+// 21.2 -> 17.1 us).
 __global__ void __launch_bounds__(256) k_mc_triangles(const __grid_constant__ Layout L,
                                                       const __grid_constant__ SlotList sl,
                                                       const __grid_constant__ McTable mc) {
     pdl_begin();
-    __shared__ uint8_t s_edges[256 * kMaxTriPerCell * 3];
-    for (int i = threadIdx.x; i < 256 * kMaxTriPerCell * 3; i += blockDim.x) s_edges[i] = mc.edges[i];
+    __shared__ __align__(16) uint8_t s_edges[256 * kMaxTriPerCell * 3];
+    for (int i = threadIdx.x; i < 256 * kMaxTriPerCell * 3 / 16; i += blockDim.x)
+        reinterpret_cast<uint4*>(s_edges)[i] = reinterpret_cast<const uint4*>(mc.edges)[i];   // (256-byte aligned in the arena)
     __syncthreads();
     const int slot = sl.s[blockIdx.y];
     const SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
     const uint32_t nt = info->n_words ? info->n_tris : 0u;
     const DRoi* rois = slot_ptr<DRoi>(L, slot, L.rois);
-    const uint32_t* emask = slot_ptr<uint32_t>(L, slot, L.emask);
-    const uint32_t* vpre = slot_ptr<uint32_t>(L, slot, L.vpre);
+    const uint4* emask = slot_ptr<uint4>(L, slot, L.emask);
     const uint64_t* trec = slot_ptr<uint64_t>(L, slot, L.trec);
     uint32_t* tris = slot_ptr<uint32_t>(L, slot, L.tris);
     const float* verts = slot_ptr<float>(L, slot, L.verts);
@@ -1033,11 +1171,11 @@ __global__ void __launch_bounds__(256) k_mc_triangles(const __grid_constant__ La
             const uint32_t wi = w + (uint32_t)((b + dx) >> 5) + (dy ? rs : 0u) + (dz ? ps : 0u);
             const int bb = (b + dx) & 31;
             const uint32_t lm = (1u << bb) - 1u;
-            const uint32_t xm = emask[3 * (size_t)wi], ym = emask[3 * (size_t)wi + 1], zm = emask[3 * (size_t)wi + 2];
-            uint32_t rank = __popc(xm & lm) + __popc(ym & lm) + __popc(zm & lm);
-            if (axis >= 1) rank += (xm >> bb) & 1u;
-            if (axis >= 2) rank += (ym >> bb) & 1u;
-            id[v] = vpre[wi] + rank;
+            const uint4 m = emask[wi];
+            uint32_t rank = __popc(m.x & lm) + __popc(m.y & lm) + __popc(m.z & lm);
+            if (axis >= 1) rank += (m.x >> bb) & 1u;
+            if (axis >= 2) rank += (m.y >> bb) & 1u;
+            id[v] = m.w + rank;
         }
         tris[3 * (size_t)t + 0] = id[0];
         tris[3 * (size_t)t + 1] = id[1];
@@ -1058,6 +1196,11 @@ __global__ void __launch_bounds__(256) k_mc_triangles(const __grid_constant__ La
 }
 
 }  // namespace
+
+cudaError_t prepare_mc() {
+    return cudaFuncSetAttribute(k_mc_compact, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(kSlabWords * sizeof(uint32_t)));
+}
 
 cudaError_t launch_mc_prefix(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl, const McTable& mc, int sms,
                              cudaStream_t st) {
