@@ -740,12 +740,18 @@ cudaError_t launch_pack(const CamSet& cams, const Layout& L, int n_frames, const
         max_words = std::max(max_words, (size_t)((cams.c[n].H + 3) / 4) * (unsigned)cams.c[n].Wq);   // a thread per 4 rows
     const int per_launch = std::min(kPackPtrs / 4, kPackPtrs / std::max(1, cams.n));
     // Device sources: enough blocks to stream HBM at full rate.  Masks read in
-    // place from host memory are bound by the host link, which about two
-    // blocks per SM keep busy; the rest of the GPU stays free for the work
-    // of other streams meanwhile.
-    const size_t cap = host_src ? (size_t)std::max(1, 2 * sms / std::max(1, cams.n * std::min(n_frames, per_launch)))
+    // place from host memory are bound by the host link, which some megabyte
+    // of loads in flight keeps busy (128 bytes a thread); more of them only
+    // wait longer, and hold up the other streams' work.  Blocks of 32 threads,
+    // three per SM in all, a block per image at least: 48 court frames 168 GB/s
+    // with 256 threads, 195 with 32; 20 judo frames 190 and 202; four rigs
+    // served at saturation 2200 frames/s with 256 threads, 2370 with 128, 2580
+    // with 64 and 2760 with 32 (eight such blocks per SM: 2460; two: 2820, but 20
+    // 720p frames 165 GB/s instead of 183).
+    const size_t cap = host_src ? (size_t)std::max(1, 3 * sms / std::max(1, cams.n * std::min(n_frames, per_launch)))
                                 : (size_t)2048;
-    const unsigned gx = (unsigned)std::max<size_t>(1, std::min<size_t>((max_words + 255) / 256, cap));
+    const unsigned th = host_src ? 32 : 256;
+    const unsigned gx = (unsigned)std::max<size_t>(1, std::min<size_t>((max_words + th - 1) / th, cap));
     static_assert(sizeof(CamSet) + sizeof(PackSrc) + sizeof(Layout) <= 32764, "k_pack parameters");
     thread_local PackSrc a;   // 18 KB: kept off the stack
     for (int j0 = 0; j0 < n_frames; j0 += per_launch) {
@@ -754,7 +760,7 @@ cudaError_t launch_pack(const CamSet& cams, const Layout& L, int n_frames, const
             a.slot[j] = slots[j0 + j];
             for (int n = 0; n < cams.n; ++n) a.src[j * cams.n + n] = src[(size_t)(j0 + j) * cams.n + n];
         }
-        const cudaError_t e = launch_pdl(k_pack, dim3(gx, cams.n, nf), dim3(256), 0, st, cams, a, L);
+        const cudaError_t e = launch_pdl(k_pack, dim3(gx, cams.n, nf), dim3(th), 0, st, cams, a, L);
         if (e != cudaSuccess) return e;
     }
     return cudaGetLastError();

@@ -676,9 +676,10 @@ __global__ void __launch_bounds__(kChunk, kMcBlocksPerSm) k_mc_compact(const __g
 }
 
 // What camera c sees of the grid edge m - h .. m + h, that is of every point
-// its bisection can test.  h is `half` along the axis, so (dx, dy, dw), the rows of
-// P applied to it, are one product each (nine multiply-adds with h's zeros: 3636
-// instead of 3590 us for 64 court frames).  With u = x'/w' at m the ends lie at u +- (dx - u dw) / (w' +- dw), so within
+// its bisection can test.  h is `half` along the axis, so (dx, dy, dw), the
+// rows of P applied to it, are one product each (as nine multiply-adds with h's
+// zeros: 3636 instead of 3590 us for 64 court frames).  With u = x'/w' at m the
+// ends lie at u +- (dx - u dw) / (w' +- dw), so within
 // |dx - u dw| / (w' - |dw|) of u, and 1 / (w' - |dw|) <= (1 + 2 |dw| / w') / w'
 // where |dw| <= w' / 2.  The box of that, widened by 0.2% and 2^-10 pixels for
 // the bound's own roundings and by the camera's margins (segment_margins on the
