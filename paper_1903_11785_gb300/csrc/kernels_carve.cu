@@ -29,6 +29,10 @@ __device__ __forceinline__ uint32_t nonzero_bytes4(uint32_t w) {
 // (Layout::silb), whose words are the transposed bytes of four rows' words.
 // One thread per 32 x 4 pixels; grid (blocks, cameras, frames).  Bound by
 // HBM: eight 16-byte loads are in flight per thread.
+// Rows of a width that 32 does not divide, or that do not start at 16 bytes, are
+// read by the aligned 4-byte words that hold them: a byte at a time, 8 court
+// frames of 1917 x 1079 took 2140 us instead of 2003 a call, four 4K ones of 3838
+// pixels 1023 instead of 837.
 __global__ void __launch_bounds__(256) k_pack(const __grid_constant__ CamSet cams, const __grid_constant__ PackSrc a,
                                               const __grid_constant__ Layout L) {
     pdl_begin();
@@ -61,12 +65,34 @@ __global__ void __launch_bounds__(256) k_pack(const __grid_constant__ CamSet cam
                           nonzero_bytes4(a1.z) << 24 | nonzero_bytes4(a1.w) << 28;
             }
         } else {
+            // any width and address: the words that hold the rows' 32 bytes,
+            // shifted into place; bytes where such a word reaches past the image
             const int nb = min(32, c.W - (int)wq * 32);
-#pragma unroll 1
-            for (int b = 0; b < nb; ++b)
+            const uintptr_t first = reinterpret_cast<uintptr_t>(src), end = first + (size_t)c.W * (unsigned)c.H;
+            uintptr_t q[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) q[r] = reinterpret_cast<uintptr_t>(p) + (size_t)min(r, rows - 1) * (unsigned)c.W;
+            if ((q[0] & ~(uintptr_t)3) >= first && (q[3] & ~(uintptr_t)3) + 36 <= end) {
+                uint32_t v[4][9];
 #pragma unroll
                 for (int r = 0; r < 4; ++r)
-                    if (r < rows) bits[r] |= (uint32_t)(p[(size_t)r * (unsigned)c.W + b] != 0) << b;
+#pragma unroll
+                    for (int k = 0; k < 9; ++k) v[r][k] = __ldcs(reinterpret_cast<const uint32_t*>(q[r] & ~(uintptr_t)3) + k);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const uint32_t sh = 8u * (uint32_t)(q[r] & 3u);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        bits[r] |= nonzero_bytes4(__funnelshift_r(v[r][k], v[r][k + 1], sh)) << (4 * k);
+                    bits[r] &= 0xFFFFFFFFu >> (32 - nb);
+                }
+            } else {
+#pragma unroll 1
+                for (int b = 0; b < nb; ++b)
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+                        bits[r] |= (uint32_t)(reinterpret_cast<const uint8_t*>(q[r])[b] != 0) << b;
+            }
         }
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
