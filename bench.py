@@ -82,7 +82,7 @@ def parse_args():
                     help="JSON file of tuned launch shapes: reuse the entry for this GPU and workload, "
                          "or autotune and add it")
     ap.add_argument("--zbuffer-cams", type=int, choices=(1, 2, 4), default=None,
-                    help="cameras per z-buffer block, set after any tuning (for profiling one variant)")
+                    help="groups of four cameras per unit of z-buffer work, set after any tuning (for profiling one variant)")
     ap.add_argument("--no-cpu", action="store_true")
     ap.add_argument("--study", choices=("surface", "fig10", "table1", "view"), default=None,
                     help="instead of the benchmark line: surface-rule errors (Sec. II-C), the coarse/fine "
@@ -712,7 +712,7 @@ def run_ours(args):
     # (info reset; coarse hull; 5 for CCL, boxes and filter; fine-grid clear
     # and fine hull; MC compaction; bisection; triangles; depth clear, box and
     # z-buffer); one colour launch per 48 frames
-    n_launch = args.steps * ((F + 127) // 128 + 15 + (F + 47) // 48)
+    n_launch = args.steps * ((F + 127) // 128 + 13 + (F + 47) // 48)
     p50, p99 = float(np.percentile(lat, 50)), float(np.percentile(lat, 99))
     line = {"metric": METRIC, "value": value, "unit": "frames/s", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",

@@ -292,9 +292,10 @@ typedef struct {
 
 /* The outputs of Sec. II-C to II-E (as fvv_get_results returns them) for
  * several slots with one wait: the counts of all n_slots slots (1..256) are
- * read together, with one synchronisation of `stream`, then the copies of
+ * read together, with one synchronisation of `stream`, and the copies of
  * every slot's vertices, triangles, colours and cameras into dst[i]'s
- * buffers are enqueued on `stream` (wait for the stream before reading
+ * buffers are enqueued on `stream`: by one launch before that wait where the
+ * buffers are device memory, else after it (wait for the stream before reading
  * them).  A slot whose reconstruction exceeded a capacity gets its counts
  * but no copies, and the call returns FVV_ERR_CAPACITY; a slot not
  * reconstructed gives FVV_ERR_NOT_READY and a bad argument
@@ -355,7 +356,7 @@ fvv_status fvv_debug_label_coarse(fvv_rig *rig, int slot, const uint32_t *coarse
  *                in which case every label is 0; LOOP if a union-find bound
  *                was hit)
  * Work is enqueued on `stream`; nothing is allocated.  Its scratch is one
- * static device array inside the library (about 32.4 MB, held on every GPU
+ * static device array inside the library (about 33.6 MB, held on every GPU
  * that loads the library until the process exits), which limits the grid to
  * nx*ny*nz <= 8,388,608 voxels: larger grids, non-positive sizes or NULL
  * pointers give FVV_ERR_INVALID_ARG without launching anything.  The first

@@ -7,7 +7,7 @@
 // one file-scope static __device__ array, so the call
 // allocates nothing: no cudaMalloc, no cudaFree, no allocating library call.
 // The array is part of the library image, so every GPU that loads the
-// library holds it (kScratchInts ints, about 32.4 MB) until the process exits.
+// library holds it (kScratchInts ints, about 33.6 MB) until the process exits.
 //
 // Host code cannot use the array's name as a device address (in host code it
 // names a host-side stand-in), so the first call on each device, with that
