@@ -147,15 +147,13 @@ void cell_cameras(CamSet& cs, const Grid& g) {
 }
 
 // Cameras of the coarse table: the first eight, which settle nearly every
-// voxel, or as many as fit 1 GiB, but at least one (a court frame's grid of 7
-// million voxels takes 28 MB each; 64 frames: 1220 us with four, 1110 with 16),
-// of those whose images are not too large for a 32-bit bit index.  At the others voxels are tested by projecting them.
+// voxel, or as many as fit 1 GiB, but always one, which the first pass reads
+// without asking (a court frame's grid of 7 million voxels takes 28 MB each; 64
+// frames: 1220 us with four, 1110 with 16; the largest grids take up to 8 GiB for
+// the one).  At the others voxels are tested by projecting them.
 int coarse_table_cams(const CamSet& cs, const Grid& g) {
     const double per = (double)g.nx * g.ny * g.nz * 4.0;
-    const int most = std::min(cs.n, (int)std::min(8.0, std::max(1.0, (double)(1ull << 30) / per)));
-    for (int n = 0; n < most; ++n)
-        if ((unsigned long long)((cs.c[n].H + 31) / 32) * cs.c[n].Wq * 1024ull >= kNoPixel) return n;
-    return most;
+    return std::min(cs.n, (int)std::min(8.0, std::max(1.0, (double)(1ull << 30) / per)));
 }
 
 struct Plan {
@@ -193,7 +191,7 @@ fvv_status make_plan(const fvv_rig_desc* d, const fvv_recon_params* p, Plan& pl,
         }
         c.W = d->width[n];
         c.H = d->height[n];
-        if (c.W < 1 || c.W > 65535 || c.H < 1 || c.H > 65535) { err = "image sizes must be 1..65535"; return FVV_ERR_INVALID_ARG; }
+        if (c.W < 1 || c.W > kMaxSide || c.H < 1 || c.H > kMaxSide) { err = "image sizes must be 1..65535"; return FVV_ERR_INVALID_ARG; }
         c.Wq = (c.W + 31) / 32;
         c.Wf = (float)c.W;
         c.Hf = (float)c.H;
@@ -423,11 +421,9 @@ fvv_status fvv_create_rig(const fvv_rig_desc* desc, const fvv_recon_params* para
     if (e == cudaSuccess) e = cudaMemcpy(rig->mc_edges, edges.data(), edges.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = prepare_ccl();
     if (e == cudaSuccess) e = prepare_mc();
-    if (pl.table_cams) {
-        uint32_t* tab = reinterpret_cast<uint32_t*>(rig->arena + pl.table);
-        rig->table = CoarseTable{tab, pl.table_cams};
-        if (e == cudaSuccess) e = launch_coarse_table(rig->cams, rig->grid, tab, pl.table_cams, nullptr);
-    }
+    uint32_t* tab = reinterpret_cast<uint32_t*>(rig->arena + pl.table);
+    rig->table = CoarseTable{tab, pl.table_cams};
+    if (e == cudaSuccess) e = launch_coarse_table(rig->cams, rig->grid, tab, pl.table_cams, nullptr);
     // every depth image starts empty; each depth stage then clears only the
     // box its slot's previous z-buffer wrote
     if (e == cudaSuccess) e = launch_init_depth(rig->cams, rig->L, rig->max_slots, rig->sms, nullptr);

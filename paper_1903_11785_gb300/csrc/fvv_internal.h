@@ -156,15 +156,25 @@ __host__ __device__ inline T* slot_ptr(const Layout& L, int slot, size_t off) {
     return reinterpret_cast<T*>(L.base + (size_t)slot * L.stride + off);
 }
 
+// Bit (word * 32 + bit, see Layout::silb) of pixel (px, py) in the blocked
+// silhouette of an image of Wq words a row.
+__host__ __device__ constexpr uint32_t blocked_bit(uint32_t px, uint32_t py, uint32_t Wq) {
+    const uint32_t tile = (py >> 5) * Wq + (px >> 5);
+    return (tile * 32u + (py & 28u) + (px >> 3 & 3u)) * 32u + (py & 3u) * 8u + (px & 7u);
+}
+
 // Where the coarse voxels fall in the first n cameras' silhouettes: the cameras
 // are static and so is the grid, so this is laid out once, when the rig is
-// created.  e[c * voxels + L]: the bit of voxel L's pixel in camera c's blocked
-// silhouette (word * 32 + bit, see Layout::silb), or kNoPixel where the voxel is
-// not in front of the camera or not inside its image.
+// created.  e[c * voxels + L]: blocked_bit of voxel L's pixel in camera c, or
+// kNoPixel where the voxel is not in front of the camera or not inside its image.
+constexpr int kMaxSide = 65535;         // pixels of an image's side
 constexpr uint32_t kNoPixel = 0xFFFFFFFFu;
+static_assert(blocked_bit(kMaxSide - 1, kMaxSide - 1, (kMaxSide + 31) / 32) < kNoPixel &&
+                  (unsigned long long)((kMaxSide + 31) / 32) * ((kMaxSide + 31) / 32) * 1024u <= 1ull << 32,
+              "every pixel of the largest image has a bit of its own below kNoPixel");
 struct CoarseTable {
     const uint32_t* e;
-    int n;                      // see coarse_table_cams in fvv_api.cu
+    int n;                      // at least 1 (see coarse_table_cams in fvv_api.cu)
 };
 
 struct SlotList {

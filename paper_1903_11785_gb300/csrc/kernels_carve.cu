@@ -122,9 +122,8 @@ __global__ void __launch_bounds__(256) k_coarse_table(const __grid_constant__ Ca
         for (int n = 0; n < ncams; ++n) {
             int px, py;
             cam_pixel(cams.c[n], X, Y, Z, px, py);
-            const uint32_t tile = (uint32_t)(py >> 5) * (uint32_t)cams.c[n].Wq + (uint32_t)(px >> 5);
-            const uint32_t word = tile * 32u + ((uint32_t)py & 28u) + ((uint32_t)px >> 3 & 3u);
-            table[n * nvox + i] = px < 0 ? kNoPixel : word * 32u + ((uint32_t)py & 3u) * 8u + ((uint32_t)px & 7u);
+            table[n * nvox + i] =
+                px < 0 ? kNoPixel : blocked_bit((uint32_t)px, (uint32_t)py, (uint32_t)cams.c[n].Wq);
         }
     }
 }
