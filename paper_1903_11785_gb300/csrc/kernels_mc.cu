@@ -437,17 +437,21 @@ __global__ void __launch_bounds__(kChunk, kMcBlocksPerSm) k_mc_compact(const __g
     __shared__ uint16_t s_cell[kChunk / 32][32 * 32];      // a turn's mixed cells: word * 32 + cell
     __shared__ uint32_t s_case[8][kChunk];   // (cell_cases)
     __shared__ __align__(8) uint64_t bar;
-    __shared__ uint32_t s_c, s_len, s_fail;
+    __shared__ uint32_t s_c, s_len, s_fail, s_words;
     __shared__ unsigned long long s_base[2];
+    const int slot = sl.s[blockIdx.y];
+    SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
     for (int i = threadIdx.x; i < 256; i += blockDim.x) s_ntri[i] = mc.ntri[i];
     if (threadIdx.x == 0) {
         mbar_init(&bar);
         s_fail = 0u;
+        s_words = info->n_words;
     }
     __syncthreads();
-    const int slot = sl.s[blockIdx.y];
-    SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
-    const uint32_t nwords = info->n_words, nchunks = info->n_chunks;
+    // n_words is read once a block: the block with the slot's last chunk sets it to
+    // zero where a capacity is exceeded, and a block that starts that late has to
+    // see one value in all its threads, or it would list some of its boxes only
+    const uint32_t nwords = s_words, nchunks = info->n_chunks;
     const int nrois = info->n_rois;
     DRoi* rois = slot_ptr<DRoi>(L, slot, L.rois);
     const uint32_t* fine = slot_ptr<uint32_t>(L, slot, L.fine);
