@@ -855,8 +855,8 @@ static_assert(kSortBuckets * kBisectWin % 32 == 0 && kBisectWin <= 8, "sort coun
 // warp of the block).
 template <class Mask>
 struct BisectWarpSmem {
-    Mask und[32 * kBisectWin];                 // undecided cameras, in window order
-    uint32_t id[32 * kBisectWin];              // vertex | inside << 30 | seen_fg << 31, or ~0u for an empty place
+    Mask und[32 * kBisectWin];                 // undecided cameras of the window's vertices
+    uint8_t seen[32 * kBisectWin];             // inside | seen_fg << 1
     uint8_t perm[32 * kBisectWin];             // window places in sorted order
     int cnt[kSortBuckets * kBisectWin];        // bucket-major counts, then their exclusive prefix
 };
@@ -944,21 +944,17 @@ __global__ void __launch_bounds__(256) k_bisect(const __grid_constant__ CamSet c
         // condition is the same in every lane)
         for (uint32_t base = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * win; base < nv;
              base += nwarps * win) {
-            // (1) each lane's kv vertices: their undecided cameras
+            // (1) each lane's kv vertices (place p of the window: vertex
+            // base + p, empty from nv on): their undecided cameras
             for (int j = 0; j < kv; ++j) {
-                const uint32_t i = base + (uint32_t)(j * 32 + lane);
-                Mask und = 0;
-                uint32_t id = ~0u;
-                if (i < nv) {
-                    const Edge e = edge_of_record(vrec[i], rois, g);
-                    bool seen_fg, inside;
-                    uint32_t rd = 0;
-                    und = edge_undecided<Mask>(sc, ncam, sil, e, seen_fg, inside, rd);
-                    reads += rd;
-                    id = i | (inside ? 0x40000000u : 0u) | (seen_fg ? 0x80000000u : 0u);
-                }
-                w.und[j * 32 + lane] = und;
-                w.id[j * 32 + lane] = id;
+                const int p = j * 32 + lane;
+                if (base + (uint32_t)p >= nv) break;
+                const Edge e = edge_of_record(vrec[base + (uint32_t)p], rois, g);
+                bool seen_fg, inside;
+                uint32_t rd = 0;
+                w.und[p] = edge_undecided<Mask>(sc, ncam, sil, e, seen_fg, inside, rd);
+                w.seen[p] = (uint8_t)((inside ? 1u : 0u) | (seen_fg ? 2u : 0u));
+                reads += rd;
             }
             // (2) counting sort of the window's places by list length
 #pragma unroll
@@ -968,7 +964,7 @@ __global__ void __launch_bounds__(256) k_bisect(const __grid_constant__ CamSet c
             // that key (worked out twice, so that nothing stays in registers)
             auto place = [&](int j, int& key, int& rank) {
                 const int p = j * 32 + lane;
-                key = w.id[p] == ~0u ? kSortCap : min(__popcll((unsigned long long)w.und[p]), kSortCap - 1);
+                key = base + (uint32_t)p >= nv ? kSortCap : min(__popcll((unsigned long long)w.und[p]), kSortCap - 1);
                 const unsigned same = __match_any_sync(kFull, key);
                 rank = __popc(same & ((1u << lane) - 1u));
                 return __popc(same);
@@ -1001,13 +997,13 @@ __global__ void __launch_bounds__(256) k_bisect(const __grid_constant__ CamSet c
             // (3) the bisections, 32 at a time in sorted order (empty places last)
             for (int j = 0; j < kv; ++j) {
                 const int p = w.perm[j * 32 + lane];
-                const uint32_t id = w.id[p];
-                if (__all_sync(kFull, id == ~0u)) break;
-                const bool have = id != ~0u;
-                const uint32_t i = id & 0x3FFFFFFFu;
+                const uint32_t i = base + (uint32_t)p;
+                const bool have = i < nv;
+                if (!__any_sync(kFull, have)) break;
                 Edge e{};
                 if (have) e = edge_of_record(vrec[i], rois, g);
-                finish(have, i, e, w.und[p], (id >> 31) != 0u, (id >> 30 & 1u) != 0u);
+                const uint32_t seen = w.seen[p];
+                finish(have, i, e, w.und[p], (seen & 2u) != 0u, (seen & 1u) != 0u);
             }
             __syncwarp();   // the window's shared memory is read before the next one writes it
         }
