@@ -90,6 +90,14 @@ def slot_bytes(scene_rig, staging: int = 1, **caps) -> int:
     return b - a
 
 
+def shared_bytes(scene_rig, staging: int = 1, **caps) -> int:
+    """Device bytes a rig costs beside its slots: for a court rig 226 MB, nearly
+    all of it the coarse hull's table of pixels, which a calibration has once per
+    library rig (up to 1 GiB, or one camera's 4 bytes per coarse voxel if more)."""
+    a = fvv.fvv_query_arena(fvv.make_desc(scene_rig, 1, staging), fvv.make_params(scene_rig, **caps))
+    return a - slot_bytes(scene_rig, staging, **caps)
+
+
 def calibration_key(rig) -> tuple:
     """What must agree for two rigs to share one library rig: cameras, image
     sizes and every reconstruction parameter."""
@@ -183,11 +191,14 @@ class Server:
         staging = [_staging(pools[mem[0]], mask_copies) for mem in members]
         gcaps = [fitted_caps(pools[mem[0]], st, base_caps) if fit_caps else dict(base_caps)
                  for mem, st in zip(members, staging)]
-        # overflow slots (default capacities) beside fitted ones come out of the budget first
-        over_bytes = [slot_bytes(pools[mem[0]].scene_rig, st, **base_caps) if fit_caps else 0
-                      for mem, st in zip(members, staging)]
-        sizes = [slot_bytes(pools[mem[0]].scene_rig, st, **c) for mem, st, c in zip(members, staging, gcaps)]
-        left = self.budget - sum(over_bytes)
+        # out of the budget first: what every library rig holds beside its slots, and
+        # the overflow slots (default capacities) beside fitted ones
+        rigs = [(pools[mem[0]].scene_rig, st) for mem, st in zip(members, staging)]
+        fixed = sum(shared_bytes(r, st, **c) for (r, st), c in zip(rigs, gcaps))
+        if fit_caps:
+            fixed += sum(shared_bytes(r, st, **base_caps) + slot_bytes(r, st, **base_caps) for r, st in rigs)
+        sizes = [slot_bytes(r, st, **c) for (r, st), c in zip(rigs, gcaps)]
+        left = self.budget - fixed
         demand = sum(len(mem) * s for mem, s in zip(members, sizes))
         n = [int(min(max_slots_per_group, max(0, left) * len(mem) // max(1, demand))) for mem in members]
         if any(x < 1 for x in n):
