@@ -242,6 +242,25 @@ inline int tuned_grid(const Tuning& tu, int knob, int sms, int n_slots, long lon
     return (int)std::max(1LL, std::min(want, cap));
 }
 
+// Blocks per slot of the fine hull, whose warps claim tiles until none is left:
+// the slot's share of the blocks that the GPU holds at a time, whatever its
+// capacity.  More of them delay the next slot (four 4K court frames 104 us with all
+// 608 each, 88 with 152; four court frames 231 and 208).  From 16 slots on the
+// launch has a round of resident blocks for every eight (fewer, and more frames'
+// silhouettes are in work than the L2 holds: 64 court frames 2964 us with four
+// rounds, 3072 with one; 16 of them 762 with two, 772 with one), in whole rounds
+// (12 court frames 570 us with one, 627 with one and a half; 24 of them 1133 with
+// three, 1218 with one and a half).  One block per 2048 words of capacity starved
+// slots fitted to their frames (the clear and the hull of one small frame 84 us
+// instead of 22, of one court frame 142 instead of 74) and is a little better only
+// where a frame has a few hundred tiles (eight mat frames at 4 cm: 40.4, now 42.6).
+inline int fine_blocks(const Tuning& tu, int sms, int n_slots, uint32_t max_fine_words) {
+    const long long resident = (long long)sms * 1024 / tu.threads[FVV_TUNE_FINE];   // at the kernel's 64 registers
+    const long long share = resident * std::max(1, n_slots / 8) / n_slots;
+    return (int)std::max(1LL, std::min<long long>(share, tuned_grid(tu, FVV_TUNE_FINE, sms, n_slots,
+                                                                   (long long)max_fine_words * 32)));
+}
+
 // Builds the 256-case table from the face rule (host).
 void build_mc_table(uint8_t ntri[256], uint8_t edges[256 * kMaxTriPerCell * 3]);
 

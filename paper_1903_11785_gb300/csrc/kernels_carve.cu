@@ -837,12 +837,7 @@ cudaError_t launch_fine_carve(const CamSet& cams, const Grid& g, const Layout& L
     const int gc = grid_x(sms, sl.n, (long long)g.max_fine_words, 256);
     launch_pdl(k_clear_fine, dim3(gc, sl.n), dim3(256), 0, st, cams, g, L, sl);
     const int th = tu.threads[FVV_TUNE_FINE];
-    // Blocks per slot: no more than can be resident for one, nor than one per
-    // 2048 words of capacity (frames use about a sixth of it; a slot given more
-    // blocks than its tiles keep busy only delays the next: four 4K court frames
-    // took 104 us with 608 blocks each, 72 with 152).
-    const int gx = std::max(1, std::min({tuned_grid(tu, FVV_TUNE_FINE, sms, sl.n, (long long)g.max_fine_words * 32),
-                                         sms * 1024 / th, (int)(g.max_fine_words * 256ll / ((long long)th * 2048))}));
+    const int gx = fine_blocks(tu, sms, sl.n, g.max_fine_words);
     // the tile shape (tile_y, tile_z) the k_filter of this sequence counted tiles with
     const uint32_t resident = (uint32_t)sms * 32u;   // 1024 threads per SM at the kernel's 64 registers
 #define FVV_LAUNCH(CG, TY, TZ) \
