@@ -834,7 +834,9 @@ cudaError_t launch_coarse_carve(const CamSet& cams, const Grid& g, const Layout&
 
 cudaError_t launch_fine_carve(const CamSet& cams, const Grid& g, const Layout& L, const SlotList& sl, int sms,
                               const Tuning& tu, cudaStream_t st) {
-    const int gc = grid_x(sms, sl.n, (long long)g.max_fine_words, 256);
+    long long rows = 0;
+    for (int n = 0; n < cams.n; ++n) rows += cams.c[n].H;
+    const int gc = clear_blocks(sms, sl.n, g.max_fine_words, rows);
     launch_pdl(k_clear_fine, dim3(gc, sl.n), dim3(256), 0, st, cams, g, L, sl);
     const int th = tu.threads[FVV_TUNE_FINE];
     const int gx = fine_blocks(tu, sms, sl.n, g.max_fine_words);
