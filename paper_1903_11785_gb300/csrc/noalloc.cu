@@ -53,12 +53,14 @@ __device__ __forceinline__ uint32_t na_word_at(const NaGrid& g, int y, int z, in
     return (g.nx & 31) && wx == g.nxw - 1 ? word & ((1u << (g.nx & 31)) - 1u) : word;
 }
 
-// Calls f(word, row, wx) for the words of the grid that are not empty, one at a
-// time and the same in every lane, so that a lane can take a voxel: a warp
+// Calls f(word, row, wx) for the words of the grid that are not empty, G lanes
+// to a word, so that a lane can take a voxel (number lane % G of its word): a warp
 // reads 32 words, a lane each, interleaved over the warps (lane l of warp k
 // reads word base + l * nwarps + k), so that neighbouring words, which often
-// belong to one object, are worked on by different warps.
-template <class F>
+// belong to one object, are worked on by different warps.  G = 32 takes the words
+// one at a time, the same in every lane; G < 32 is for rows of one word, of at
+// most G voxels: 32 / G words at a time, some of which may be empty.
+template <int G, class F>
 __device__ __forceinline__ void na_for_words(const NaGrid& g, F&& f) {
     const uint32_t nwords = (uint32_t)g.nz * (uint32_t)g.ny * (uint32_t)g.nxw;
     const int lane = threadIdx.x & 31;
@@ -66,34 +68,46 @@ __device__ __forceinline__ void na_for_words(const NaGrid& g, F&& f) {
     for (uint32_t base = 0; base < nwords; base += nwarps * 32u) {
         const uint32_t mw = base + (uint32_t)lane * nwarps + gw;
         const uint32_t mine = mw < nwords ? na_word(g, mw) : 0u;
-        for (uint32_t pending = __ballot_sync(kFull, mine != 0u); pending; pending &= pending - 1u) {
-            const int src = __ffs(pending) - 1;
-            const uint32_t w = base + (uint32_t)src * nwarps + gw;
-            const uint32_t row = w / (uint32_t)g.nxw;
-            f(__shfl_sync(kFull, mine, src), row, (int)(w - row * (uint32_t)g.nxw));
+        uint32_t pending = __ballot_sync(kFull, mine != 0u);
+        if constexpr (G < 32) {
+            constexpr int kAtOnce = 32 / G;
+#pragma unroll 1
+            for (int q = 0; q < G && pending >> (q * kAtOnce); ++q) {
+                const int src = q * kAtOnce + lane / G;
+                const uint32_t word = __shfl_sync(kFull, mine, src);
+                if (pending >> (q * kAtOnce) & (kFull >> (32 - kAtOnce))) f(word, base + (uint32_t)src * nwarps + gw, 0);
+            }
+        } else {
+            for (; pending; pending &= pending - 1u) {
+                const int src = __ffs(pending) - 1;
+                const uint32_t w = base + (uint32_t)src * nwarps + gw;
+                const uint32_t row = w / (uint32_t)g.nxw;
+                f(__shfl_sync(kFull, mine, src), row, (int)(w - row * (uint32_t)g.nxw));
+            }
         }
     }
 }
 
-// First voxel (bit) of the run of `word` that voxel `lane` belongs to.
-__device__ __forceinline__ int run_start(uint32_t word, int lane) {
+// First voxel (bit) of the run of `word` that voxel b belongs to.
+__device__ __forceinline__ int run_start(uint32_t word, int b) {
     const uint32_t starts = word & ~(word << 1);
-    return 31 - __clz(starts & (0xFFFFFFFFu >> (31 - lane)));
+    return 31 - __clz(starts & (0xFFFFFFFFu >> (31 - b)));
 }
 
 // Zero the counters, start a tree at each run of consecutive occupied voxels of
 // a word, and a count at its first voxel.  `count` (the labels' array, written in
 // full at the end) holds a component's voxels at its root.
+template <int G>
 __global__ void __launch_bounds__(256) k_na_seed(NaGrid g, int* sc, int32_t* __restrict__ count) {
     pdl_begin();
     if (blockIdx.x == 0 && threadIdx.x < 64) sc[threadIdx.x] = 0;
     int* parent = sc + kNaParent;
-    const int lane = threadIdx.x & 31;
-    na_for_words(g, [&](uint32_t word, uint32_t row, int wx) {
-        if (!((word >> lane) & 1u)) return;
-        const int first = (int)row * g.nx + wx * 32, run = run_start(word, lane);
-        parent[first + lane] = first + run;
-        if (run == lane) count[first + lane] = 0;
+    const int b = threadIdx.x % G;
+    na_for_words<G>(g, [&](uint32_t word, uint32_t row, int wx) {
+        if (!((word >> b) & 1u)) return;
+        const int first = (int)row * g.nx + wx * 32, run = run_start(word, b);
+        parent[first + b] = first + run;
+        if (run == b) count[first + b] = 0;
     });
 }
 
@@ -103,25 +117,26 @@ __global__ void __launch_bounds__(256) k_na_seed(NaGrid g, int* sc, int32_t* __r
 // the other, took 318 us on a court-sized grid (400 x 220 x 80, 12 players and
 // 2,000 stray voxels), this takes 24; the call 496 -> 63 us, and 10.1 ms -> 0.7
 // on that grid with a quarter of its voxels occupied at random.
+template <int G>
 __global__ void __launch_bounds__(256) k_na_union(NaGrid g, int* sc) {
     pdl_begin();
     int* parent = sc + kNaParent;
-    const int lane = threadIdx.x & 31;
+    const int b = threadIdx.x % G;
     int budget = kStepBudget;
-    na_for_words(g, [&](uint32_t word, uint32_t row, int wx) {
-        if (!((word >> lane) & 1u) || budget <= 0) return;
+    na_for_words<G>(g, [&](uint32_t word, uint32_t row, int wx) {
+        if (!((word >> b) & 1u) || budget <= 0) return;
         const int y = (int)(row % (uint32_t)g.ny), z = (int)(row / (uint32_t)g.ny);
-        const int run = run_start(word, lane), run0 = (int)row * g.nx + wx * 32 + run;
-        if (lane == 0 && (na_word_at(g, y, z, wx - 1) >> 31)) unite(parent, run0, run0 - 1, budget);
+        const int run = run_start(word, b), run0 = (int)row * g.nx + wx * 32 + run;
+        if (b == 0 && (na_word_at(g, y, z, wx - 1) >> 31)) unite(parent, run0, run0 - 1, budget);
         for (int k = 0; k < 4; ++k) {
             const int dy = k == 0 ? -1 : k - 2, dz = k == 0 ? 0 : -1;
             const uint32_t n = na_word_at(g, y + dy, z + dz, wx);
-            const bool left = lane > 0 ? (n >> (lane - 1)) & 1u : na_word_at(g, y + dy, z + dz, wx - 1) >> 31;
-            const bool mid = (n >> lane) & 1u;
-            const bool right = lane < 31 ? (n >> (lane + 1)) & 1u : na_word_at(g, y + dy, z + dz, wx + 1) & 1u;
+            const bool left = b > 0 ? (n >> (b - 1)) & 1u : na_word_at(g, y + dy, z + dz, wx - 1) >> 31;
+            const bool mid = (n >> b) & 1u;
+            const bool right = b < 31 ? (n >> (b + 1)) & 1u : na_word_at(g, y + dy, z + dz, wx + 1) & 1u;
             const int nrow = ((z + dz) * g.ny + (y + dy)) * g.nx + wx * 32;
-            if (run == lane && (left || mid)) unite(parent, run0, nrow + (left ? lane - 1 : lane), budget);
-            if (!mid && right) unite(parent, run0, nrow + lane + 1, budget);
+            if (run == b && (left || mid)) unite(parent, run0, nrow + (left ? b - 1 : b), budget);
+            if (!mid && right) unite(parent, run0, nrow + b + 1, budget);
         }
     });
     if (budget <= 0) atomicOr(sc + 1, (int)FVV_FLAG_LOOP);
@@ -130,15 +145,16 @@ __global__ void __launch_bounds__(256) k_na_union(NaGrid g, int* sc) {
 // Point every voxel at its root, list the roots and count each component's
 // voxels.  A warp keeps the count of the component it met last, so that a
 // large one costs it one atomic and not one a word.
+template <int G>
 __global__ void __launch_bounds__(256) k_na_compress(NaGrid g, int* sc, int32_t* __restrict__ count) {
     pdl_begin();
     int* parent = sc + kNaParent;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, b = threadIdx.x % G;
     int budget = kStepBudget, cur = -1, held = 0;   // cur, held: the same in every lane
-    na_for_words(g, [&](uint32_t word, uint32_t row, int wx) {
-        const int L = (int)row * g.nx + wx * 32 + lane;
+    na_for_words<G>(g, [&](uint32_t word, uint32_t row, int wx) {
+        const int L = (int)row * g.nx + wx * 32 + b;
         int r = -1;
-        if (((word >> lane) & 1u) && budget > 0) {
+        if (((word >> b) & 1u) && budget > 0) {
             r = find_root_readonly(parent, L, budget);
             if (r != L) parent[L] = r;
         }
@@ -222,7 +238,9 @@ __global__ void __launch_bounds__(256) k_na_rank(NaGrid g, int* sc, const int32_
 
 // Every voxel of the output: its canonical label, 0 for empty or removed.  A
 // warp takes 32 words, a lane per voxel of each, so that a word's labels go out
-// in one piece.
+// in one piece; of rows of one word (G < 32) a lane per voxel of all of them,
+// whose labels follow one another.
+template <int G>
 __global__ void __launch_bounds__(256) k_na_labels(NaGrid g, const int* sc, int32_t* __restrict__ labels) {
     pdl_begin();
     const int* parent = sc + kNaParent;
@@ -232,21 +250,56 @@ __global__ void __launch_bounds__(256) k_na_labels(NaGrid g, const int* sc, int3
     for (uint32_t base = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32u; base < nwords; base += nwarps * 32u) {
         const uint32_t mw = base + (uint32_t)lane;
         const uint32_t mine = mw < nwords ? na_word(g, mw) : 0u;
+        auto put = [&](uint32_t word, int b, int L) {
+            int lab = 0;
+            if ((word >> b) & 1u) {
+                const int r = __ldg(parent + L), t = r < 0 ? r : __ldg(parent + r);
+                lab = t < 0 ? -t - 1 : 0;           // else: roots were not tagged (too many components)
+            }
+            __stcs(labels + L, lab);
+        };
+        const int m = (int)min(32u, nwords - base);
+        if constexpr (G < 32) {
+            for (int i0 = 0; i0 < m * g.nx; i0 += 32) {
+                const int i = i0 + lane, k = min(i / g.nx, 31);
+                const uint32_t word = __shfl_sync(kFull, mine, k);
+                if (i < m * g.nx) put(word, i - k * g.nx, (int)base * g.nx + i);
+            }
+            continue;
+        }
         const uint32_t row = min(mw, nwords - 1u) / (uint32_t)g.nxw;
         const int x0 = (int)(min(mw, nwords - 1u) - row * (uint32_t)g.nxw) * 32;
         const int first = (int)row * g.nx + x0, nv = min(32, g.nx - x0);
-        const int m = (int)min(32u, nwords - base);
 #pragma unroll 4
         for (int k = 0; k < m; ++k) {
             const uint32_t word = __shfl_sync(kFull, mine, k);
             const int L = __shfl_sync(kFull, first, k) + lane;
-            int lab = 0;
-            if ((word >> lane) & 1u) {
-                const int r = __ldg(parent + L), t = r < 0 ? r : __ldg(parent + r);
-                lab = t < 0 ? -t - 1 : 0;           // else: roots were not tagged (too many components)
-            }
-            if (lane < __shfl_sync(kFull, nv, k)) __stcs(labels + L, lab);
+            if (lane < __shfl_sync(kFull, nv, k)) put(word, lane, L);
         }
+    }
+}
+
+// The call's five kernels, G lanes to a word.
+template <int G>
+void na_launch(const NaGrid& g, int* sc, int32_t* labels, int32_t* counts, unsigned blocks, cudaStream_t st) {
+    const dim3 ranks(kNaMaxComponents / kNaRankRoots);
+    // Dependent launch hides the gaps between a small grid's kernels (3,600 words: 44
+    // us without and 35 with it; 39,000: 38 and 30; 84,000: 45 and 42); a large
+    // one's run slower with it, as the next kernel's waiting blocks take room on the
+    // SMs (140,000: 44 and 46; 229,000: 51 and 61).  They are even at some 130,000
+    // words; the line lies at 65,536, where the blocks stop growing with the grid.
+    if (blocks < 2048) {
+        launch_pdl(k_na_seed<G>, dim3(blocks), dim3(256), 0, st, g, sc, labels);
+        launch_pdl(k_na_union<G>, dim3(blocks), dim3(256), 0, st, g, sc);
+        launch_pdl(k_na_compress<G>, dim3(blocks), dim3(256), 0, st, g, sc, labels);
+        launch_pdl(k_na_rank, ranks, dim3(256), 0, st, g, sc, labels, counts);
+        launch_pdl(k_na_labels<G>, dim3(blocks), dim3(256), 0, st, g, sc, labels);
+    } else {
+        k_na_seed<G><<<blocks, 256, 0, st>>>(g, sc, labels);
+        k_na_union<G><<<blocks, 256, 0, st>>>(g, sc);
+        k_na_compress<G><<<blocks, 256, 0, st>>>(g, sc, labels);
+        k_na_rank<<<ranks, 256, 0, st>>>(g, sc, labels, counts);
+        k_na_labels<G><<<blocks, 256, 0, st>>>(g, sc, labels);
     }
 }
 
@@ -280,21 +333,15 @@ extern "C" fvv_status fvv_label_components_noalloc(const uint32_t* coarse_bits, 
     const long long words = (long long)nz * ny * g.nxw;
     // four words a warp, so that a small grid's objects are spread over many, up to 2048 blocks
     const unsigned blocks = (unsigned)std::max(1LL, std::min((words + 31) / 32, 2048LL));
-    // Dependent launch hides the gaps between a small grid's kernels (60 x 60 x 30
-    // voxels: 67 -> 57 us); a large one's run slower with it (400 x 220 x 80: 63
-    // -> 71 us, the next kernel's waiting blocks take room on the SMs).
-    if (blocks < 2048) {
-        launch_pdl(k_na_seed, dim3(blocks), dim3(256), 0, st, g, sc, labels);
-        launch_pdl(k_na_union, dim3(blocks), dim3(256), 0, st, g, sc);
-        launch_pdl(k_na_compress, dim3(blocks), dim3(256), 0, st, g, sc, labels);
-        launch_pdl(k_na_rank, dim3(kNaMaxComponents / kNaRankRoots), dim3(256), 0, st, g, sc, labels, counts);
-        launch_pdl(k_na_labels, dim3(blocks), dim3(256), 0, st, g, sc, labels);
-    } else {
-        k_na_seed<<<blocks, 256, 0, st>>>(g, sc, labels);
-        k_na_union<<<blocks, 256, 0, st>>>(g, sc);
-        k_na_compress<<<blocks, 256, 0, st>>>(g, sc, labels);
-        k_na_rank<<<kNaMaxComponents / kNaRankRoots, 256, 0, st>>>(g, sc, labels, counts);
-        k_na_labels<<<blocks, 256, 0, st>>>(g, sc, labels);
-    }
+    // Rows of up to four voxels are taken several words at a time: one at a time, a
+    // warp has one to four lanes at work, where a thread per word had them all
+    // (nx = 1, 7.8 million words, 30% occupied: 859 us with a thread per word, 2120
+    // one word at a time, 601 with a lane a word; 0.04% occupied: 142, 281 and 146;
+    // nx = 4, 2 million words, 2%: 202, 246 and 165).  From five voxels on a warp on
+    // one word is the faster of the first two everywhere (nx = 6: 263 and 211 us).
+    if (nx == 1) na_launch<1>(g, sc, labels, counts, blocks, st);
+    else if (nx == 2) na_launch<2>(g, sc, labels, counts, blocks, st);
+    else if (nx <= 4) na_launch<4>(g, sc, labels, counts, blocks, st);
+    else na_launch<32>(g, sc, labels, counts, blocks, st);
     return cudaGetLastError() == cudaSuccess ? FVV_OK : FVV_ERR_CUDA;
 }
