@@ -153,7 +153,7 @@ void cell_cameras(CamSet& cs, const Grid& g) {
 // the one).  At the others voxels are tested by projecting them.
 int coarse_table_cams(const CamSet& cs, const Grid& g) {
     const double per = (double)g.nx * g.ny * g.nz * 4.0;
-    return std::min(cs.n, (int)std::min(8.0, std::max(1.0, (double)(1ull << 30) / per)));
+    return std::min(cs.n, (int)std::min((double)kTableCams, std::max(1.0, (double)(1ull << 30) / per)));
 }
 
 struct Plan {
@@ -178,7 +178,7 @@ fvv_status make_plan(const fvv_rig_desc* d, const fvv_recon_params* p, Plan& pl,
     cs.n = d->n_cams;
     if (p->oob_policy != FVV_OOB_STRICT && p->oob_policy != FVV_OOB_ABSTAIN) { err = "bad oob_policy"; return FVV_ERR_INVALID_ARG; }
     cs.oob = p->oob_policy;
-    size_t words = 0, blocked = 0, pix = 0;
+    size_t words = 0, blocked = 0, pix = 0;   // blocked: tiles
     for (int n = 0; n < cs.n; ++n) {
         Cam& c = cs.c[n];
         for (int k = 0; k < 12; ++k) {
@@ -198,10 +198,10 @@ fvv_status make_plan(const fvv_rig_desc* d, const fvv_recon_params* p, Plan& pl,
         c.bit_off = (uint32_t)words;
         c.blk_off = (uint32_t)blocked;
         c.pix_off = pix;
-        blocked += (size_t)((c.H + 31) / 32) * c.Wq * 32;
+        blocked += (size_t)((c.H + 31) / 32) * c.Wq;
         words += (size_t)c.H * c.Wq;
         pix += (size_t)c.H * c.W;
-        if (std::max(words, blocked) >= (1ull << 32)) { err = "silhouettes too large"; return FVV_ERR_INVALID_ARG; }
+        if (words >= (1ull << 32)) { err = "silhouettes too large"; return FVV_ERR_INVALID_ARG; }
     }
     pl.sil_words = words;
     pl.npix = pix;
@@ -272,7 +272,7 @@ fvv_status make_plan(const fvv_rig_desc* d, const fvv_recon_params* p, Plan& pl,
     const size_t nvox = (size_t)g.nx * g.ny * g.nz;
     take(L.info, sizeof(SlotInfo));
     take(L.sil, words * 4);
-    take(L.silb, blocked * 4);
+    take(L.silb, blocked * kBlkWords * 4);
     take(L.coarse, (size_t)g.nz * g.ny * g.nxw * 4);
     take(L.front, (size_t)g.nz * g.ny * g.nxw * 16);
     take(L.parent, nvox * 4);
@@ -422,7 +422,8 @@ fvv_status fvv_create_rig(const fvv_rig_desc* desc, const fvv_recon_params* para
     if (e == cudaSuccess) e = prepare_ccl();
     if (e == cudaSuccess) e = prepare_mc();
     uint32_t* tab = reinterpret_cast<uint32_t*>(rig->arena + pl.table);
-    rig->table = CoarseTable{tab, pl.table_cams};
+    rig->table = CoarseTable{tab, pl.table_cams, {}};
+    for (int n = 0; n < pl.table_cams; ++n) rig->table.word[n] = pl.cams.c[n].blk_off * kBlkWords;
     if (e == cudaSuccess) e = launch_coarse_table(rig->cams, rig->grid, tab, pl.table_cams, nullptr);
     // every depth image starts empty; each depth stage then clears only the
     // box its slot's previous z-buffer wrote

@@ -42,7 +42,7 @@ struct Cam {
     int W, H, Wq;        // Wq = 32-bit words per silhouette row
     float Wf, Hf;        // W and H as floats
     uint32_t bit_off;    // first silhouette word of this camera in a slot
-    uint32_t blk_off;    // first word of its blocked silhouette
+    uint32_t blk_off;    // first tile of its blocked silhouette (Layout::silb), kBlkWords words each
     uint64_t pix_off;    // first pixel of this camera in per-slot pixel arrays
     // Bound (pixels) on how far the computed image position of any point the
     // bisection of a grid edge can test lies from the box of the edge ends'
@@ -156,11 +156,13 @@ __host__ __device__ inline T* slot_ptr(const Layout& L, int slot, size_t off) {
     return reinterpret_cast<T*>(L.base + (size_t)slot * L.stride + off);
 }
 
+constexpr uint32_t kBlkWords = 32;      // words of a tile of a blocked silhouette
+
 // Bit (word * 32 + bit, see Layout::silb) of pixel (px, py) in the blocked
 // silhouette of an image of Wq words a row.
 __host__ __device__ constexpr uint32_t blocked_bit(uint32_t px, uint32_t py, uint32_t Wq) {
     const uint32_t tile = (py >> 5) * Wq + (px >> 5);
-    return (tile * 32u + (py & 28u) + (px >> 3 & 3u)) * 32u + (py & 3u) * 8u + (px & 7u);
+    return (tile * kBlkWords + (py & 28u) + (px >> 3 & 3u)) * 32u + (py & 3u) * 8u + (px & 7u);
 }
 
 // Where the coarse voxels fall in the first n cameras' silhouettes: the cameras
@@ -172,9 +174,13 @@ constexpr uint32_t kNoPixel = 0xFFFFFFFFu;
 static_assert(blocked_bit(kMaxSide - 1, kMaxSide - 1, (kMaxSide + 31) / 32) < kNoPixel &&
                   (unsigned long long)((kMaxSide + 31) / 32) * ((kMaxSide + 31) / 32) * 1024u <= 1ull << 32,
               "every pixel of the largest image has a bit of its own below kNoPixel");
+constexpr int kTableCams = 8;
+static_assert(kTableCams * (unsigned long long)((kMaxSide + 31) / 32) * ((kMaxSide + 31) / 32) * kBlkWords < 1ull << 32,
+              "the words of the blocked silhouettes of the table's cameras have 32-bit offsets");
 struct CoarseTable {
     const uint32_t* e;
-    int n;                      // at least 1 (see coarse_table_cams in fvv_api.cu)
+    int n;                      // 1 to kTableCams (see coarse_table_cams in fvv_api.cu)
+    uint32_t word[kTableCams];  // first words of its cameras' blocked silhouettes
 };
 
 struct SlotList {

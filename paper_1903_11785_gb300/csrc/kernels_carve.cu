@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(256) k_pack(const __grid_constant__ CamSet cam
     const Cam& c = cams.c[blockIdx.y];
     const uint8_t* src = a.src[blockIdx.z * (unsigned)cams.n + blockIdx.y];
     uint32_t* __restrict__ sil = slot_ptr<uint32_t>(L, a.slot[blockIdx.z], L.sil) + c.bit_off;
-    uint32_t* __restrict__ silb = slot_ptr<uint32_t>(L, a.slot[blockIdx.z], L.silb) + c.blk_off;
+    uint32_t* __restrict__ silb = slot_ptr<uint32_t>(L, a.slot[blockIdx.z], L.silb) + (size_t)c.blk_off * kBlkWords;
     const unsigned Wq = (unsigned)c.Wq;
     const size_t units = (size_t)((c.H + 3) >> 2) * Wq;
     const bool vec = (c.W % 32 == 0) && ((reinterpret_cast<uintptr_t>(src) & 15u) == 0);
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(256) k_coarse_first(const __grid_constant__ Ca
                 e[q] = lane < __shfl_sync(kFull, nv, q) ? __ldg(tab.e + f + lane) : kNoPixel;
             }
 #pragma unroll
-            for (int q = 0; q < kWords; ++q) word[q] = e[q] != kNoPixel ? __ldg(silb + cams.c[0].blk_off + (e[q] >> 5)) : 0u;
+            for (int q = 0; q < kWords; ++q) word[q] = e[q] != kNoPixel ? __ldg(silb + tab.word[0] + (e[q] >> 5)) : 0u;
 #pragma unroll
             for (int q = 0; q < kWords; ++q) {
                 const bool bit = (word[q] >> (e[q] & 31u)) & 1u;
@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(256) k_coarse_first(const __grid_constant__ Ca
         const uint32_t* te = tab.e + nvox + lane;
 #pragma unroll 1
         for (int c = 1; MORE && c < levels && any; ++c, te += nvox) {
-            const uint32_t* __restrict__ sb = silb + cams.c[c].blk_off;
+            const uint32_t* __restrict__ sb = silb + tab.word[c];
             uint32_t e[kWords], word[kWords];
 #pragma unroll
             for (int q = 0; q < kWords; ++q) {
@@ -270,13 +270,13 @@ __global__ void __launch_bounds__(256) k_coarse_rest(const __grid_constant__ Cam
                                                      const __grid_constant__ SlotList sl,
                                                      const __grid_constant__ CoarseTable tab, int levels) {
     pdl_begin();
-    __shared__ uint32_t s_blk[FVV_MAX_CAMS];
+    __shared__ uint32_t s_blk[kTableCams];
     __shared__ unsigned long long sh[32];
     const int slot = sl.s[blockIdx.y];
     SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
     const uint32_t nfront = min(info->n_front, (uint32_t)g.nz * (uint32_t)g.ny * (uint32_t)g.nxw);
     if (((blockIdx.x * blockDim.x) >> 5) >= nfront) return;   // the whole block
-    for (int n = threadIdx.x; n < cams.n; n += blockDim.x) s_blk[n] = cams.c[n].blk_off;
+    for (int n = threadIdx.x; n < tab.n; n += blockDim.x) s_blk[n] = tab.word[n];
     __syncthreads();
     const uint32_t* __restrict__ silb = slot_ptr<uint32_t>(L, slot, L.silb);
     const uint32_t* __restrict__ sil = slot_ptr<uint32_t>(L, slot, L.sil);
