@@ -441,18 +441,19 @@ __global__ void __launch_bounds__(kChunk, kMcBlocksPerSm) k_mc_compact(const __g
     __shared__ unsigned long long s_base[2];
     const int slot = sl.s[blockIdx.y];
     SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) s_ntri[i] = mc.ntri[i];
-    if (threadIdx.x == 0) {
-        mbar_init(&bar);
-        s_fail = 0u;
-        s_words = info->n_words;
-    }
-    __syncthreads();
     // n_words is read once a block: the block with the slot's last chunk sets it to
     // zero where a capacity is exceeded, and a block that starts that late has to
     // see one value in all its threads, or it would list some of its boxes only
-    const uint32_t nwords = s_words, nchunks = info->n_chunks;
+    const uint32_t nchunks = info->n_chunks, cw = info->chunk_words;
     const int nrois = info->n_rois;
+    if (threadIdx.x == 0) {
+        s_words = info->n_words;
+        mbar_init(&bar);
+        s_fail = 0u;
+    }
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) s_ntri[i] = mc.ntri[i];
+    __syncthreads();
+    const uint32_t nwords = s_words;
     DRoi* rois = slot_ptr<DRoi>(L, slot, L.rois);
     const uint32_t* fine = slot_ptr<uint32_t>(L, slot, L.fine);
     uint4* emask = slot_ptr<uint4>(L, slot, L.emask);
@@ -465,7 +466,7 @@ __global__ void __launch_bounds__(kChunk, kMcBlocksPerSm) k_mc_compact(const __g
         list_depth_boxes(cams, g, L, slot, rois, nwords ? nrois : 0, reinterpret_cast<unsigned long long*>(slab),
                          reinterpret_cast<int4*>(slab) + FVV_MAX_CAMS);
     bool pending = false;   // the wait for a copy ran out, and it may still be in flight
-    const uint32_t cw = info->chunk_words, turns = cw / kChunk, warp = threadIdx.x >> 5;
+    const uint32_t turns = cw / kChunk, warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     // A warp's counts in one word: under 2^15 vertices (3 x 32 x 256) and 2^17 triangles
     constexpr int kVertBits = 15;
