@@ -121,46 +121,9 @@ __device__ __forceinline__ void test_cam(const Cam& c, const uint32_t* __restric
     }
 }
 
-template <int NC, bool ABSTAIN>
-__device__ __forceinline__ bool warp_test_p(const CamSet& cams, const uint32_t* __restrict__ sil, float X, float Y,
-                                            float Z, bool alive, uint32_t& tests) {
-    bool voted = !ABSTAIN;
-    if constexpr (NC > 0) {
-#pragma unroll
-        for (int n = 0; n < NC; ++n) {
-            if (!__any_sync(kFull, alive)) break;
-            if (alive) {
-                ++tests;
-                test_cam<ABSTAIN>(cams.c[n], sil, X, Y, Z, alive, voted);
-            }
-        }
-    } else {
-        for (int n = 0; n < cams.n; ++n) {
-            if (!__any_sync(kFull, alive)) break;
-            if (alive) {
-                ++tests;
-                test_cam<ABSTAIN>(cams.c[n], sil, X, Y, Z, alive, voted);
-            }
-        }
-    }
-    return alive && voted;
-}
-
-// Occupancy of the 32 points of a warp (one per lane; lanes with alive ==
-// false take no part), cameras in index order, each lane stopping at its
-// first background vote and the warp stopping when no lane is left; `tests`
-// counts each lane's camera tests.  All 32 lanes must call it together.
-// NC > 0 unrolls the camera loop for NC cameras, so the camera matrices are
-// read as constant-bank operands instead of indexed constant loads.
-template <int NC>
-__device__ __forceinline__ bool warp_test(const CamSet& cams, const uint32_t* __restrict__ sil, float X, float Y,
-                                          float Z, bool alive, uint32_t& tests) {
-    return cams.oob == FVV_OOB_ABSTAIN ? warp_test_p<NC, true>(cams, sil, X, Y, Z, alive, tests)
-                                       : warp_test_p<NC, false>(cams, sil, X, Y, Z, alive, tests);
-}
-
-// Camera counts with an unrolled instantiation of the hull-test kernels
-// (anything else runs the generic loop).
+// Camera counts with an unrolled instantiation of k_lambda (anything else runs its
+// generic loop), so that the camera matrices are read as constant-bank operands
+// instead of indexed constant loads.
 #define FVV_DISPATCH_NC(n, F)   \
     switch (n) {                \
         case 4: F(4); break;    \
@@ -304,15 +267,15 @@ __device__ __forceinline__ int roi_of_word(const DRoi* rois, int n, uint32_t w) 
     return lo;
 }
 
-// Position of fine word w in its ROI's padded grid, with the ROI fields the
-// kernels need kept in registers; a new ROI is looked up only when w leaves
-// the current one (grid-stride loops visit words in increasing order).
+// Position of fine word w in its ROI's padded grid, with the ROI fields that the
+// compaction needs kept in registers; another ROI is read only when w leaves
+// the current one (a chunk's words are visited in increasing order, a few ROIs at
+// most, from the chunk's first one on).
 struct RoiCursor {
     int k = -1;
     uint32_t lo = 0, hi = 0;
     int fdim[3];
     int nxw;
-    float fo[3];
     // word position
     int wx, yp, zp;
 
@@ -321,21 +284,10 @@ struct RoiCursor {
         hi = lo + r.n_words;
         nxw = r.nxw;
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            fdim[a] = r.fdim[a];
-            fo[a] = r.fo[a];
-        }
+        for (int a = 0; a < 3; ++a) fdim[a] = r.fdim[a];
     }
 
-    __device__ __forceinline__ void seek(const DRoi* rois, int n, uint32_t w) {
-        if (w >= hi || w < lo) {
-            k = roi_of_word(rois, n, w);
-            take(rois[k]);
-        }
-        place(w);
-    }
-
-    // seek for a word at or after the first word of ROI k0
+    // (w: at or after the first word of ROI k0)
     __device__ __forceinline__ void seek_from(const DRoi* rois, int n, uint32_t w, int k0) {
         if (w >= hi || w < lo) {
             k = k0;
