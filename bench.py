@@ -708,10 +708,10 @@ def run_ours(args):
         cpu["single_core_per_config"] = per_cfg
         flips = fp64_flips(rig, cpu_sample[0][0])
 
-    # kernels per step: one packing launch per 128 frames; the reconstruction's 15
-    # (info reset; coarse hull; 5 for CCL, boxes and filter; fine-grid clear
-    # and fine hull; MC compaction; bisection; triangles; depth clear, box and
-    # z-buffer); one colour launch per 48 frames
+    # kernels per step: one packing launch per 128 frames; the reconstruction's 13
+    # (info reset; 2 for the coarse hull; 4 for CCL, boxes and filter; clear of the
+    # fine grids and depth images, and fine hull; MC compaction; bisection;
+    # triangles; z-buffer); one colour launch per 48 frames
     n_launch = args.steps * ((F + 127) // 128 + 13 + (F + 47) // 48)
     p50, p99 = float(np.percentile(lat, 50)), float(np.percentile(lat, 99))
     line = {"metric": METRIC, "value": value, "unit": "frames/s", "n_gpus": world, "steps": args.steps,

@@ -193,8 +193,12 @@ enum {
 
 /* Bytes of device memory fvv_create_rig needs for these arguments (after the
  * defaults for zero capacities are applied): the memory that, as in
- * Sec. III-B, is taken once at start-up.  desc, params and bytes are host
- * pointers; NULL or an invalid argument gives FVV_ERR_INVALID_ARG. */
+ * Sec. III-B, is taken once at start-up.  Beside the slots' parts, which are
+ * all alike, it holds a table of the coarse voxels' pixels: 4 bytes per
+ * voxel of the coarse grid for each of the first eight cameras, or for as
+ * many as 1 GiB holds, but always for one (up to 8 GiB for the largest
+ * grid).  desc, params and bytes are host pointers; NULL or an invalid
+ * argument gives FVV_ERR_INVALID_ARG. */
 fvv_status fvv_query_arena(const fvv_rig_desc *desc, const fvv_recon_params *params,
                            size_t *bytes);
 

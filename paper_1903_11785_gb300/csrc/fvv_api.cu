@@ -425,8 +425,8 @@ fvv_status fvv_create_rig(const fvv_rig_desc* desc, const fvv_recon_params* para
     rig->table = CoarseTable{tab, pl.table_cams, {}};
     for (int n = 0; n < pl.table_cams; ++n) rig->table.word[n] = pl.cams.c[n].blk_off * kBlkWords;
     if (e == cudaSuccess) e = launch_coarse_table(rig->cams, rig->grid, tab, pl.table_cams, nullptr);
-    // every depth image starts empty; each depth stage then clears only the
-    // box its slot's previous z-buffer wrote
+    // every depth image starts empty; each reconstruction then clears only the
+    // boxes that its slot's previous z-buffer may have written (k_clear_fine)
     if (e == cudaSuccess) e = launch_init_depth(rig->cams, rig->L, rig->max_slots, rig->sms, nullptr);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e == cudaSuccess) e = cudaHostAlloc(reinterpret_cast<void**>(&rig->host_info), FVV_MAX_BATCH * sizeof(SlotInfo),

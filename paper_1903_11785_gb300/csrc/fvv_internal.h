@@ -208,7 +208,7 @@ struct Tuning {
     int threads[FVV_N_TUNE];
     int waves[FVV_N_TUNE];
     int fine_tile;       // index into kFineTiles
-    int zb_cams;         // groups of four cameras per z-buffer block: 1, 2 or 4
+    int zb_cams;         // groups of four cameras a z-buffer warp takes its triangles through: 1, 2 or 4
 };
 
 // The grid with the tuned fine-carve tile shape.

@@ -815,8 +815,13 @@ cudaError_t launch_coarse_carve(const CamSet& cams, const Grid& g, const Layout&
     const int g1 = tuned_grid(tu, FVV_TUNE_COARSE, sms, sl.n, (words + kWords - 1) / kWords * 32);
     const int g2 = tuned_grid(tu, FVV_TUNE_COARSE, sms, sl.n, words * 32);
     // Cameras of the first pass: three where the launch is too small to hide the
-    // second pass's chains of loads (a court frame, 229,000 words: 49 us with one
-    // camera, 37 with three), else one (64 frames: 988 us against 1085).
+    // second pass's chains of loads (one court frame, 229,000 words: 46 us with one
+    // camera, 34 with three; two, 458,000: 67 and 57), else one (64 frames: 988 and
+    // 1085).  Where the two cross depends on the rig: below 0.8 million words for
+    // one 4K court frame of abstaining cameras (81 and 89 us, twice that 133 and
+    // 159), at 0.9 for 720p frames (640,000: 62.5 and 61; 960,000: 83 and 85), above
+    // 1.8 for court frames (1.8 million: 168 and 165), so the line lies below the
+    // first, and the others lose a tenth at most (three court frames: 84 and 76).
     const int levels = std::min(tab.n, words * sl.n < 600000 ? 3 : 1);
 #define FVV_LAUNCH(A, M) launch_pdl(k_coarse_first<A, M>, dim3(g1, sl.n), dim3(th), 0, st, cams, g, L, sl, tab, levels)
     if (cams.oob == FVV_OOB_ABSTAIN) {

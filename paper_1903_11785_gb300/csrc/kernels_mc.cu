@@ -5,9 +5,9 @@
 // with word-wide bit operations:
 //   compact   bipolar-edge masks (x: w ^ w>>1, y: w ^ w(y+1), z: w ^ w(z+1)),
 //             vertices = popcounts, triangles = table counts of mixed cells;
-//             exclusive prefix per word (block scan + a look-back over the
-//             earlier 256-word chunks) and one record per bipolar edge, in
-//             edge-key order (3*Lpad + axis), and one per triangle; the
+//             exclusive prefix per word (sums over the block + a look-back
+//             over the earlier chunks, of 256 to 1024 words) and one record per
+//             bipolar edge, in edge-key order (3*Lpad + axis), and one per triangle; the
 //             grid slab a chunk reads is staged in shared memory by a bulk
 //             copy.
 //   bisect    one thread per vertex: fixed-count bisection of its edge
