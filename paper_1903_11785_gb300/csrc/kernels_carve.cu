@@ -5,6 +5,8 @@
 // 16-camera frame 4 MB, so a frame's silhouettes stay in L2), row by row for
 // the fine hull and the surface, which scan short rows of them, and once more in
 // square blocks for the coarse hull, whose gathers run across them.
+#include <climits>
+
 #include "fvv_device.cuh"
 
 namespace fvv {
@@ -354,6 +356,13 @@ __global__ void __launch_bounds__(256) k_clear_fine(const __grid_constant__ CamS
     const int slot = sl.s[blockIdx.y];
     SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
     const uint32_t nwords = info->n_words;
+    // the first camera's depth boxes (below) are on their way meanwhile
+    const int lane = threadIdx.x & 31, bw = blockDim.x >> 5;
+    const int blocks = (int)gridDim.x, block = (int)blockIdx.x, n0 = block % cams.n;
+    const int* counts = slot_ptr<int>(L, slot, L.dcount);
+    const int4* boxes = slot_ptr<int4>(L, slot, L.dbox);
+    const int count0 = counts[n0];
+    const int4 first0 = boxes[(size_t)n0 * (unsigned)g.max_rois + (unsigned)min(lane, g.max_rois - 1)];
     uint32_t* fine = slot_ptr<uint32_t>(L, slot, L.fine);
     for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < nwords; w += gridDim.x * blockDim.x) fine[w] = 0u;
     // the compaction's look-back states of this reconstruction's chunks, and
@@ -381,29 +390,56 @@ __global__ void __launch_bounds__(256) k_clear_fine(const __grid_constant__ CamS
     if (blockIdx.x == 0 && threadIdx.x == 0) info->next_tile = 0u;
     // Depth boxes: a camera's rows, counted through all its boxes, are dealt out
     // to the warps of its blocks (blocks i, i + cameras, ...; fewer blocks than
-    // cameras take several cameras each).
-    const int lane = threadIdx.x & 31, bw = blockDim.x >> 5;
-    const int blocks = (int)gridDim.x, block = (int)blockIdx.x;
+    // cameras take several cameras each).  Where the boxes overlap so much that
+    // their union's box has fewer pixels, its rows are taken instead.  A warp goes
+    // from one of its rows to the next (box by box, each warp walked through all
+    // boxes: a frame of 500 ROIs 114 us for this kernel and the hull, now 69).
     const bool many = blocks >= cams.n;
     const int sub = many ? block / cams.n : 0;
-    const int subs = many ? (blocks - block % cams.n + cams.n - 1) / cams.n : 1;
+    const int subs = many ? (blocks - n0 + cams.n - 1) / cams.n : 1;
     const int nw = subs * bw, me = sub * bw + (int)(threadIdx.x >> 5);
-    for (int n = block % cams.n; n < cams.n; n += many ? cams.n : blocks) {
-        const int W = cams.c[n].W, count = slot_ptr<int>(L, slot, L.dcount)[n];
-        const int4* box = slot_ptr<int4>(L, slot, L.dbox) + (size_t)n * (unsigned)g.max_rois;
+    const int4 none = make_int4(0, -1, 0, -1);
+    for (int n = n0; n < cams.n; n += many ? cams.n : blocks) {
+        const int W = cams.c[n].W, count = n == n0 ? count0 : counts[n];
+        const int4* box = boxes + (size_t)n * (unsigned)g.max_rois;
         uint32_t* D = slot_ptr<uint32_t>(L, slot, L.depth) + cams.c[n].pix_off;
-        int at = me;                       // this warp's first row of the box at hand
-        for (int k0 = 0; k0 < count; k0 += 32) {
-            const int4 mine = k0 + lane < count ? box[k0 + lane] : make_int4(0, -1, 0, -1);
-            for (int k = 0; k < min(32, count - k0); ++k) {
-                const int x0 = __shfl_sync(kFull, mine.x, k), x1 = __shfl_sync(kFull, mine.y, k);
-                const int y0 = __shfl_sync(kFull, mine.z, k), rows = __shfl_sync(kFull, mine.w, k) - y0 + 1;
-                for (; at < rows; at += nw) {
-                    uint32_t* row = D + (size_t)(y0 + at) * (unsigned)W;
-                    for (int x = x0 + lane; x <= x1; x += 32) __stcs(row + x, kEmptyDepth);
-                }
-                at -= rows;
+        auto clear = [&](int x0, int x1, int y) {
+            uint32_t* row = D + (size_t)y * (unsigned)W;
+            for (int x = x0 + lane; x <= x1; x += 32) __stcs(row + x, kEmptyDepth);
+        };
+        int4 mine = lane < count ? (n == n0 ? first0 : box[lane]) : none;
+        int4 u = make_int4(INT_MAX, -1, INT_MAX, -1);
+        float area = 0.0f;
+        for (int k = lane; k < count; k += 32) {
+            const int4 b = k < 32 ? mine : box[k];
+            if (b.y < 0) continue;             // none
+            area += (float)(b.y - b.x + 1) * (float)(b.w - b.z + 1);
+            u = make_int4(min(u.x, b.x), max(u.y, b.y), min(u.z, b.z), max(u.w, b.w));
+        }
+        for (int o = 16; o > 0; o >>= 1) area += __shfl_xor_sync(kFull, area, o);
+        u = make_int4(__reduce_min_sync(kFull, u.x), __reduce_max_sync(kFull, u.y), __reduce_min_sync(kFull, u.z),
+                      __reduce_max_sync(kFull, u.w));
+        if (u.y < 0) continue;                 // no box
+        if (area > (float)(u.y - u.x + 1) * (float)(u.w - u.z + 1)) {
+            for (int y = u.z + me; y <= u.w; y += nw) clear(u.x, u.y, y);
+            continue;
+        }
+        int at = me;                           // this warp's next row, counted from the boxes at hand
+        for (int k0 = 0;;) {
+            int end = mine.w - mine.z + 1;     // rows of the boxes of lanes 0 .. this one
+            for (int o = 1; o < 32; o <<= 1) {
+                const int e = __shfl_up_sync(kFull, end, o);
+                if (lane >= o) end += e;
             }
+            const int rows = __shfl_sync(kFull, end, 31);
+            for (; at < rows; at += nw) {
+                const int k = __ffs(__ballot_sync(kFull, end > at)) - 1;
+                clear(__shfl_sync(kFull, mine.x, k), __shfl_sync(kFull, mine.y, k), __shfl_sync(kFull, mine.w + 1 - end, k) + at);
+            }
+            at -= rows;
+            k0 += 32;
+            if (k0 >= count) break;
+            mine = k0 + lane < count ? box[k0 + lane] : none;
         }
     }
 }

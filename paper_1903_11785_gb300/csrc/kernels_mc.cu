@@ -18,7 +18,6 @@
 // Vertex and triangle order is therefore (ROI, key) and (ROI, cell, table
 // order): independent of scheduling, identical to a serial scan.
 #include <atomic>
-#include <climits>
 
 #include "fvv_device.cuh"
 
@@ -327,40 +326,45 @@ __device__ __forceinline__ uint64_t pack_trec(uint32_t w, int b, int j, int cs, 
 }
 
 // The boxes that hold every pixel this frame's z-buffer can write, for the clear
-// of the slot's next frame, by the threads of one block: every mesh vertex lies
+// of the slot's next frame: every mesh vertex lies
 // in its ROI's fine grid box grown by one fine voxel (padding samples and
 // surface points), so every covered pixel centre lies in the convex hull
 // of the projections of that box's eight corners, widened by two pixels and
 // clamped to the image; the whole image if a corner is not in front of the
-// camera.  One box per ROI and camera, or their union where that has fewer
-// pixels.  `area` and `bound`: shared memory, per camera.
+// camera.  One box per ROI and camera, (0, -1, 0, -1) for none, whether or not a
+// capacity turns out to be exceeded and nothing is drawn in them; eight lanes, a
+// corner each, work a box out, from the launch's last block on.  (By one block, a
+// thread per box, a frame of 500 ROIs and 16 cameras waited 130 us for it, one of
+// 3,000 a millisecond; now some microseconds.  In k_mc_triangles, which has no
+// registers to spare, 64 court frames took 190 us more; in k_zbuffer a 720p frame
+// one and a half.)
 __device__ __forceinline__ void list_depth_boxes(const CamSet& cams, const Grid& g, const Layout& L, int slot,
-                                                 const DRoi* rois, int nrois, unsigned long long* area, int4* bound) {
+                                                 const DRoi* rois, int nrois) {
     int4* box = slot_ptr<int4>(L, slot, L.dbox);
     int* count = slot_ptr<int>(L, slot, L.dcount);
-    for (int n = threadIdx.x; n < cams.n; n += blockDim.x) {
-        area[n] = 0ull;
-        bound[n] = make_int4(INT_MAX, -1, INT_MAX, -1);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < cams.n * nrois; i += blockDim.x) {
+    if (blockIdx.x == 0)
+        for (int n = threadIdx.x; n < cams.n; n += blockDim.x) count[n] = nrois;
+    const int boxes = cams.n * nrois, lane = threadIdx.x & 31, q = lane & 7;
+    const int step = (int)(gridDim.x * blockDim.x >> 5) * 4;
+    for (int i0 = (int)(((gridDim.x - 1u - blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * 4; i0 < boxes; i0 += step) {
+        const int i = min(i0 + (lane >> 3), boxes - 1);       // (the last ones once more)
         const int n = i / nrois, k = i - n * nrois;
         const Cam& c = cams.c[n];
         const DRoi& r = rois[k];
-        float lo[3], hi[3];
-        for (int a = 0; a < 3; ++a) {
-            lo[a] = r.fo[a] - g.sf;
-            hi[a] = r.fo[a] + (float)(r.fdim[a] + 1) * g.sf;
-        }
-        float umin = 3.0e38f, umax = -3.0e38f, vmin = 3.0e38f, vmax = -3.0e38f;
-        bool front = true;
-        for (int q = 0; q < 8; ++q) {
-            float xh, yh, wh;
-            project(c.P, (q & 1) ? hi[0] : lo[0], (q & 2) ? hi[1] : lo[1], (q & 4) ? hi[2] : lo[2], xh, yh, wh);
-            front &= wh > 0.0f;
-            const float u = __fdiv_rn(xh, wh), v = __fdiv_rn(yh, wh);
-            umin = fminf(umin, u); umax = fmaxf(umax, u);
-            vmin = fminf(vmin, v); vmax = fmaxf(vmax, v);
+        float X[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            X[a] = (q >> a) & 1 ? r.fo[a] + (float)(r.fdim[a] + 1) * g.sf : r.fo[a] - g.sf;
+        float xh, yh, wh;
+        project(c.P, X[0], X[1], X[2], xh, yh, wh);
+        const bool front = (__ballot_sync(kFull, wh > 0.0f) >> (lane & 24) & 0xFFu) == 0xFFu;
+        float umin = __fdiv_rn(xh, wh), vmin = __fdiv_rn(yh, wh), umax = umin, vmax = vmin;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+            umin = fminf(umin, __shfl_xor_sync(kFull, umin, o));
+            umax = fmaxf(umax, __shfl_xor_sync(kFull, umax, o));
+            vmin = fminf(vmin, __shfl_xor_sync(kFull, vmin, o));
+            vmax = fmaxf(vmax, __shfl_xor_sync(kFull, vmax, o));
         }
         int x0 = 0, x1 = c.W - 1, y0 = 0, y1 = c.H - 1;
         if (front && umin > -1.0e6f && umax < 1.0e6f && vmin > -1.0e6f && vmax < 1.0e6f) {
@@ -369,25 +373,10 @@ __device__ __forceinline__ void list_depth_boxes(const CamSet& cams, const Grid&
             y0 = max(0, (int)floorf(vmin) - 2);
             y1 = min(c.H - 1, (int)floorf(vmax) + 2);
         }
-        const bool none = x0 > x1 || y0 > y1;
-        box[(size_t)n * (unsigned)g.max_rois + (unsigned)k] = none ? make_int4(0, -1, 0, -1) : make_int4(x0, x1, y0, y1);
-        if (none) continue;
-        atomicAdd(area + n, (unsigned long long)(x1 - x0 + 1) * (unsigned)(y1 - y0 + 1));
-        int* b = reinterpret_cast<int*>(bound + n);
-        atomicMin(b + 0, x0);
-        atomicMax(b + 1, x1);
-        atomicMin(b + 2, y0);
-        atomicMax(b + 3, y1);
+        if (q == 0)
+            box[(size_t)n * (unsigned)g.max_rois + (unsigned)k] =
+                x0 > x1 || y0 > y1 ? make_int4(0, -1, 0, -1) : make_int4(x0, x1, y0, y1);
     }
-    __syncthreads();
-    for (int n = threadIdx.x; n < cams.n; n += blockDim.x) {
-        const int4 b = bound[n];
-        const bool any = b.x <= b.y && b.z <= b.w;
-        const bool one = any && area[n] > (unsigned long long)(b.y - b.x + 1) * (unsigned)(b.w - b.z + 1);
-        if (one) box[(size_t)n * (unsigned)g.max_rois] = b;
-        count[n] = !any ? 0 : one ? 1 : nrois;
-    }
-    __syncthreads();
 }
 
 // Sec. II-C classify and compact, in one pass over each slot's fine words:
@@ -437,23 +426,21 @@ __global__ void __launch_bounds__(kChunk, kMcBlocksPerSm) k_mc_compact(const __g
     __shared__ uint16_t s_cell[kChunk / 32][32 * 32];      // a turn's mixed cells: word * 32 + cell
     __shared__ uint32_t s_case[8][kChunk];   // (cell_cases)
     __shared__ __align__(8) uint64_t bar;
-    __shared__ uint32_t s_c, s_len, s_fail, s_words;
+    __shared__ uint32_t s_c, s_len, s_fail;
     __shared__ unsigned long long s_base[2];
     const int slot = sl.s[blockIdx.y];
     SlotInfo* info = slot_ptr<SlotInfo>(L, slot, L.info);
-    // n_words is read once a block: the block with the slot's last chunk sets it to
-    // zero where a capacity is exceeded, and a block that starts that late has to
-    // see one value in all its threads, or it would list some of its boxes only
-    const uint32_t nchunks = info->n_chunks, cw = info->chunk_words;
+    // (n_words is set to zero where a capacity is exceeded, by the block with the
+    // slot's last chunk, when every other chunk is claimed: a block that may still
+    // read that finds no chunk left)
+    const uint32_t nwords = info->n_words, nchunks = info->n_chunks, cw = info->chunk_words;
     const int nrois = info->n_rois;
     if (threadIdx.x == 0) {
-        s_words = info->n_words;
         mbar_init(&bar);
         s_fail = 0u;
     }
     for (int i = threadIdx.x; i < 256; i += blockDim.x) s_ntri[i] = mc.ntri[i];
     __syncthreads();
-    const uint32_t nwords = s_words;
     DRoi* rois = slot_ptr<DRoi>(L, slot, L.rois);
     const uint32_t* fine = slot_ptr<uint32_t>(L, slot, L.fine);
     uint4* emask = slot_ptr<uint4>(L, slot, L.emask);
@@ -461,10 +448,7 @@ __global__ void __launch_bounds__(kChunk, kMcBlocksPerSm) k_mc_compact(const __g
     uint64_t* trec = slot_ptr<uint64_t>(L, slot, L.trec);
     unsigned long long* cst = slot_ptr<unsigned long long>(L, slot, L.chunk_st);
     const uint32_t* clen = slot_ptr<uint32_t>(L, slot, L.chunk_len);
-    // one block of the slot lists the frame's depth boxes first (the slab is not in use yet)
-    if (blockIdx.x == gridDim.x - 1u)
-        list_depth_boxes(cams, g, L, slot, rois, nwords ? nrois : 0, reinterpret_cast<unsigned long long*>(slab),
-                         reinterpret_cast<int4*>(slab) + FVV_MAX_CAMS);
+    list_depth_boxes(cams, g, L, slot, rois, nrois);
     bool pending = false;   // the wait for a copy ran out, and it may still be in flight
     const uint32_t turns = cw / kChunk, warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
