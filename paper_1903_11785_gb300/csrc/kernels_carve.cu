@@ -68,7 +68,10 @@ __global__ void __launch_bounds__(256) k_pack(const __grid_constant__ CamSet cam
             }
         } else {
             // any width and address: the words that hold the rows' 32 bytes,
-            // shifted into place; bytes where such a word reaches past the image
+            // shifted into place; bytes where such a word reaches past the image.
+            // (Kept in L1: a thread's last word is the next one's first, and a
+            // sector is read by several loads; evict-first, twelve unaligned 4K
+            // masks read in place took 529 us instead of 512.)
             const int nb = min(32, c.W - (int)wq * 32);
             const uintptr_t first = reinterpret_cast<uintptr_t>(src), end = first + (size_t)c.W * (unsigned)c.H;
             uintptr_t q[4];
@@ -79,7 +82,7 @@ __global__ void __launch_bounds__(256) k_pack(const __grid_constant__ CamSet cam
 #pragma unroll
                 for (int r = 0; r < 4; ++r)
 #pragma unroll
-                    for (int k = 0; k < 9; ++k) v[r][k] = __ldcs(reinterpret_cast<const uint32_t*>(q[r] & ~(uintptr_t)3) + k);
+                    for (int k = 0; k < 9; ++k) v[r][k] = __ldg(reinterpret_cast<const uint32_t*>(q[r] & ~(uintptr_t)3) + k);
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
                     const uint32_t sh = 8u * (uint32_t)(q[r] & 3u);
@@ -808,7 +811,9 @@ cudaError_t launch_pack(const CamSet& cams, const Layout& L, int n_frames, const
     // with 256 threads, 195 with 32; 20 judo frames 190 and 202; four rigs
     // served at saturation 2200 frames/s with 256 threads, 2370 with 128, 2580
     // with 64 and 2760 with 32 (eight such blocks per SM: 2460; two: 2820, but 20
-    // 720p frames 165 GB/s instead of 183).
+    // 720p frames 165 GB/s instead of 183).  With the link to itself a call on large
+    // masks takes up to 3% longer than by two blocks of 256 per SM (twelve 4K masks
+    // 482 -> 497 us).
     const size_t cap = host_src ? (size_t)std::max(1, 3 * sms / std::max(1, cams.n * std::min(n_frames, per_launch)))
                                 : (size_t)2048;
     const unsigned th = host_src ? 32 : 256;
