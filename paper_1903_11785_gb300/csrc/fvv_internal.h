@@ -267,7 +267,7 @@ inline int clear_blocks(int sms, int n_slots, uint32_t max_fine_words, long long
 // three, 1218 with one and a half).  One block per 2048 words of capacity starved
 // slots fitted to their frames (the clear and the hull of one small frame 84 us
 // instead of 22, of one court frame 142 instead of 74) and is a little better only
-// where a frame has a few hundred tiles (eight mat frames at 4 cm: 40.4, now 42.6).
+// where a frame has a few hundred tiles (eight mat frames at 4 cm: 40.4, now 44).
 inline int fine_blocks(const Tuning& tu, int sms, int n_slots, uint32_t max_fine_words) {
     const long long resident = (long long)sms * 1024 / tu.threads[FVV_TUNE_FINE];   // at the kernel's 64 registers
     const long long share = resident * std::max(1, n_slots / 8) / n_slots;
